@@ -19,18 +19,17 @@
 //    marker by marker (a stable partition by allele; the new run length of a
 //    neighbour pair is 1 + the minimum over the old pairs it spans).  At every
 //    core of the stage it writes M, the class boundary n0 (and, for XPEHH, the
-//    population of each sorted position) to a slot, with the boundaries of
-//    the first walk steps already grouped by step.  A chunk starts `warmup`
+//    population of each sorted position) to a slot.  A chunk starts `warmup`
 //    markers before its first core, so its sort is exact for walks that stay
 //    within that history.
-//  * split_walk_kernel: one warp per slot runs the walk steps of that core
-//    (both allele classes of iHS, or the pooled XPEHH walk): gaps, the map,
-//    the cutoff and the trapezoid exactly as the per-step walk does, with S(i)
-//    from the boundaries of step i (from the slot's first window, then from
-//    64-step windows it finds in M).  A walk that would step beyond its
-//    chunk's history is handed to the per-step walk kernel (second pass).
+//  * split_walk_kernel: one warp per slot runs the walks of that core (both
+//    allele classes of iHS, or the pooled XPEHH walk) 32 or 64 steps at a
+//    time, lane l taking step l of the window: S of every step of the window
+//    comes from one pass over the window's boundaries, then gaps, the map, the
+//    cutoff and the trapezoid apply to all its steps at once, exactly as the
+//    per-step walk applies them.  A walk that would step beyond its chunk's
+//    history is handed to the per-step walk kernel (second pass).
 #include <cooperative_groups.h>
-#include <cooperative_groups/reduce.h>
 #include <limits.h>
 
 #include "../../include/selscan.h"
@@ -43,9 +42,9 @@ namespace {
 
 constexpr unsigned kInf16 = 0xFFFFu;
 constexpr int kRowRing = 4;                 // rows in flight ahead of the sort (cp.async)
-constexpr int kSlotListCap = 1024;          // first-window boundaries kept per slot
-constexpr int kSplitListSmem = 1024;        // window list entries a walking warp keeps on chip
-constexpr int kWin = 64;                    // steps of a window the walker groups itself (a power of 2)
+constexpr int kTokSmem = 1024;              // window boundaries a walking warp keeps on chip (multiple of 4)
+constexpr int kSparseMax = kTokSmem;        // most new boundaries of a window taken one per lane
+constexpr int kWin = 64;                    // steps of such a window (two blocks of 32)
 
 __host__ __device__ inline int sweep_e(int n, int T)
 {
@@ -104,32 +103,27 @@ __device__ __forceinline__ unsigned bit_index(const SweepArgs &w, int h)
 
 }  // namespace
 
-// Slot of one core: header {n0, history horizon, W1, 0}, the run lengths M
-// (u16 per sorted position), for XPEHH the population-A flags of the sorted
-// positions, then the first window: W1 + 1 step offsets (u16) and its
-// boundaries ordered by step (u16 positions).  The window is the longest run
-// of steps 1..W1 (W1 <= 64) whose boundaries fit slot_list_cap(n) entries.
+// Slot of one core: header {n0, history horizon, 0, 0}, the run lengths M and,
+// for XPEHH, the population-A flags of the sorted positions.  M is kept in
+// groups of 32 positions (16 words, u16 pairs): word j of group g holds the run
+// lengths of positions 32 g + j (low half) and 32 g + 16 + j (high half), so
+// that the walker turns a group into a 32-bit mask in position order with
+// 16-bit SIMD operations alone.
 namespace {
-__host__ __device__ inline int slot_list_cap(int n) { return n < kSlotListCap ? n : kSlotListCap; }
-__host__ __device__ inline size_t slot_isa_at(int n) { return 16 + (((size_t)n * 2 + 15) & ~(size_t)15); }
-__host__ __device__ inline size_t slot_off_at(int n, int xpehh)
-{
-    return slot_isa_at(n) + (xpehh ? (((size_t)split_nw(n) * 4 + 15) & ~(size_t)15) : 0);
-}
-__host__ __device__ inline size_t slot_list_at(int n, int xpehh) { return slot_off_at(n, xpehh) + 144; }
+__host__ __device__ inline size_t slot_isa_at(int n) { return 16 + (size_t)((n + 31) / 32) * 64; }
 }  // namespace
 
 size_t sweep_smem_bytes(int n, int W, int T, int R)
 {
     const int W32 = ((2 * W) + 4) & ~3;
-    return (size_t)sweep_npad(n, T) * 4 * 2 + (size_t)W32 * 4 * kRowRing + T / 32 * 12 + 2 * 65 * 4 +
+    return (size_t)sweep_npad(n, T) * 4 * 2 + (size_t)W32 * 4 * kRowRing + T / 32 * 12 +
            (size_t)((R + 31) / 32) * 4;
 }
 
 size_t sweep_slot_bytes(int n, int xpehh)
 {
     // a multiple of 16 bytes: every slot's M region is read and written in 16-byte units
-    return slot_list_at(n, xpehh) + (((size_t)slot_list_cap(n) * 2 + 15) & ~(size_t)15);
+    return slot_isa_at(n) + (xpehh ? (((size_t)split_nw(n) * 4 + 15) & ~(size_t)15) : 0);
 }
 
 size_t sweep_state_bytes(int n, int T) { return (size_t)sweep_npad(n, T) * 4; }
@@ -140,8 +134,7 @@ size_t sweep_elements(int n, int T) { return (size_t)sweep_npad(n, T); }
 // Shared memory: two buffers of np packed elements (bit index of the haplotype
 // in the row | run length with its predecessor << 16), a ring of kRowRing row
 // buffers (filled by cp.async, each with one extra all-ones word), the warp
-// totals, a core's first-window counts and offsets, and the stage's core
-// bitmap.  Positions n..np-1 hold padding elements whose allele is that
+// totals and the stage's core bitmap.  Positions n..np-1 hold padding elements whose allele is that
 // all-ones word: they sort after every real haplotype and never touch a real
 // element's run length.  T threads (32 to 512); EMAX bounds the elements per
 // thread (at most 32, one allele bit each in a 32-bit mask), up to 24 stay in
@@ -163,9 +156,7 @@ __global__ void __launch_bounds__(T, T == 512 ? 2 : (T == 256 ? 3 : 512 / T)) sw
     unsigned *P0 = (unsigned *)smem;             // buffer b at P0 + b * np
     unsigned *R0 = P0 + 2 * np;                  // row ring: slot r at R0 + r * W32r
     unsigned *wsum = R0 + kRowRing * W32r;
-    unsigned *hcnt = wsum + 3 * NW;              // a core's first window: per-step counts,
-    unsigned *hoff = hcnt + 65;                  // then cursors and (at [64]) W1
-    unsigned *cbits = hoff + 65;                 // the stage's cores that pass the filter
+    unsigned *cbits = wsum + 3 * NW;             // the stage's cores that pass the filter
 
     const int dir = blockIdx.x / w.nch;          // 0: walks toward lower indices
     const int c = blockIdx.x % w.nch;
@@ -218,7 +209,6 @@ __global__ void __launch_bounds__(T, T == 512 ? 2 : (T == 256 ? 3 : 512 / T)) sw
         cp_async_commit();
     };
     for (int q = 0; q < kRowRing; ++q) fetch_row(q);
-    for (int t = tid; t < 64; t += T) hcnt[t] = 0u;
     for (int r = 0; r < kRowRing; ++r)          // the padding elements' all-ones word
         if (tid < W32r - W32) R0[r * W32r + W32 + tid] = 0xFFFFFFFFu;
     {
@@ -388,25 +378,15 @@ __global__ void __launch_bounds__(T, T == 512 ? 2 : (T == 256 ? 3 : 512 / T)) sw
                 hdr[1] = (int)hz;
             }
             const unsigned *Ps = P0 + cur * np;
-            // run lengths, 4 per 8-byte store (four elements per item: finer
-            // items even out the threads' shares; the slot's M region is a
-            // multiple of 16 bytes, values past n are never read), counting the
-            // boundaries of each of steps 1..64 (M in [1, 64])
+            // run lengths, 8 per 16-byte store (the padding elements fill the last
+            // group; np is a multiple of 32).  Nothing waits for the stores: the
+            // next marker's partition reads this buffer and writes the other one
             const uint4 *P4 = (const uint4 *)Ps;
-            uint2 *M2 = (uint2 *)(slot + 16);
-            for (int t = tid; t < (n + 3) / 4; t += T) {
-                const uint4 a = P4[t];
-                M2[t] = make_uint2(__byte_perm(a.x, a.y, 0x7632u), __byte_perm(a.z, a.w, 0x7632u));
-                const unsigned e4[4] = {a.x, a.y, a.z, a.w};
-                if (4 * t + 4 <= n) {
-#pragma unroll
-                    for (int j = 0; j < 4; ++j)
-                        if (e4[j] - 0x10000u < 0x400000u) atomicAdd(hcnt + (e4[j] >> 16) - 1, 1u);
-                } else {
-#pragma unroll
-                    for (int j = 0; j < 4; ++j)
-                        if (e4[j] - 0x10000u < 0x400000u && 4 * t + j < n) atomicAdd(hcnt + (e4[j] >> 16) - 1, 1u);
-                }
+            uint4 *M4 = (uint4 *)(slot + 16);
+            for (int t = tid; t < (n + 31) / 32 * 4; t += T) {
+                const uint4 lo = P4[(t >> 2) * 8 + (t & 3)], hi = P4[(t >> 2) * 8 + 4 + (t & 3)];
+                M4[t] = make_uint4(__byte_perm(lo.x, hi.x, 0x7632u), __byte_perm(lo.y, hi.y, 0x7632u),
+                                   __byte_perm(lo.z, hi.z, 0x7632u), __byte_perm(lo.w, hi.w, 0x7632u));
             }
             if (xp) {                            // population of each sorted position
                 // one 32-position word per warp iteration: a ballot over the lanes
@@ -417,55 +397,6 @@ __global__ void __launch_bounds__(T, T == 512 ? 2 : (T == 256 ? 3 : 512 / T)) sw
                     const int t = q * 32 + lane;
                     const unsigned word = __ballot_sync(FULLMASK, t < n && (Ps[t] & 0xFFFFu) < limA);
                     if (lane == 0) isA[q] = word;
-                }
-            }
-            __syncthreads();
-            // the first window: the longest run of steps from step 1 on whose
-            // boundaries fit the slot's list
-            unsigned short *soff = (unsigned short *)(slot + slot_off_at(n, xp));
-            if (warp == 0) {
-                const unsigned c0 = hcnt[2 * lane], c1 = hcnt[2 * lane + 1];
-                unsigned incl = c0 + c1;
-#pragma unroll
-                for (int d = 1; d < 32; d <<= 1) {
-                    const unsigned v = __shfl_up_sync(FULLMASK, incl, d);
-                    if (lane >= d) incl += v;
-                }
-                const unsigned ex = incl - c0 - c1;
-                const unsigned cap = (unsigned)slot_list_cap(n);
-                // steps 2 lane + 1 and 2 lane + 2 end at offsets ex + c0 and incl
-                const unsigned w1 = __popc(__ballot_sync(FULLMASK, ex + c0 <= cap)) +
-                                    __popc(__ballot_sync(FULLMASK, incl <= cap));
-                soff[2 * lane] = (unsigned short)min(ex, 0xFFFFu);
-                soff[2 * lane + 1] = (unsigned short)min(ex + c0, 0xFFFFu);
-                if (lane == 31) soff[64] = (unsigned short)min(incl, 0xFFFFu);
-                hoff[2 * lane] = ex;
-                hoff[2 * lane + 1] = ex + c0;
-                hcnt[2 * lane] = 0u;
-                hcnt[2 * lane + 1] = 0u;
-                if (lane == 0) {
-                    hoff[64] = w1;
-                    ((int *)slot)[2] = (int)w1;
-                    ((int *)slot)[3] = 0;
-                }
-            }
-            __syncthreads();
-            // place the window's boundaries by step
-            const unsigned lim = hoff[64] << 16;
-            unsigned short *slist = (unsigned short *)(slot + slot_list_at(n, xp));
-            for (int t = tid; t < (n + 3) / 4; t += T) {
-                const uint4 a = P4[t];
-                const unsigned e4[4] = {a.x, a.y, a.z, a.w};
-                if (4 * t + 4 <= n) {
-#pragma unroll
-                    for (int j = 0; j < 4; ++j)
-                        if (e4[j] - 0x10000u < lim)
-                            slist[atomicAdd(hoff + (e4[j] >> 16) - 1, 1u)] = (unsigned short)(4 * t + j);
-                } else {
-#pragma unroll
-                    for (int j = 0; j < 4; ++j)
-                        if (e4[j] - 0x10000u < lim && 4 * t + j < n)
-                            slist[atomicAdd(hoff + (e4[j] >> 16) - 1, 1u)] = (unsigned short)(4 * t + j);
                 }
             }
         }
@@ -481,34 +412,40 @@ __global__ void __launch_bounds__(T, T == 512 ? 2 : (T == 256 ? 3 : 512 / T)) sw
 // ---- the split walk ----------------------------------------------------------
 namespace {
 
-// Per-warp shared memory: run starts before this step (O) and all run starts
-// including this step's (A) as bitmaps over positions 0..n, one summary bit
-// per non-zero word (SO, SA), step counts / offsets of the current window, and
-// for XPEHH the population-A flags of the sorted positions with their
-// per-word prefix counts.
+// Per-warp shared memory: the window's boundaries in position order (position |
+// M << 16) with, for XPEHH, the number of population-A haplotypes before each;
+// the run starts older than the window (O) and those of it (N) as bitmaps over
+// positions 0..n, one summary bit per non-zero word of O (S); the drops of S
+// per step of a sparse window; and for XPEHH the population-A flags of the
+// sorted positions with their per-word prefix counts.
 struct SplitSmem {
-    unsigned *O, *A, *SO, *SA;
-    unsigned *cnt, *off;
-    unsigned short *lst;                  // the current window's list, when it fits
+    unsigned *tk;                         // window list on chip, first kTokSmem entries (XPEHH: pairs)
+    unsigned *gtk;                        // the rest, global: entry k at gtk[k]
+    unsigned *O, *N, *S, *dec;
     unsigned *isA, *PA;
     int nw, ns;
 };
 
-__device__ inline SplitSmem split_smem(unsigned char *base, int n, int xpehh)
+__host__ __device__ inline int split_words(int n, int xpehh)
+{
+    const int nw = split_nw(n), ns = (nw + 31) >> 5;
+    return kTokSmem * (xpehh ? 2 : 1) + 2 * nw + ns + kWin * (xpehh ? 3 : 2) + (xpehh ? 2 * nw : 0);
+}
+
+__device__ inline SplitSmem split_smem(unsigned char *base, unsigned char *scratch, int n, int xpehh)
 {
     SplitSmem s;
     s.nw = split_nw(n);
     s.ns = (s.nw + 31) >> 5;
     unsigned *p = (unsigned *)base;
+    s.tk = p; p += kTokSmem * (xpehh ? 2 : 1);
+    s.dec = p; p += kWin * (xpehh ? 3 : 2);
     s.O = p; p += s.nw;
-    s.A = p; p += s.nw;
-    s.SO = p; p += s.ns;
-    s.SA = p; p += s.ns;
-    s.cnt = p; p += kWin;
-    s.off = p; p += kWin + 1;
-    s.isA = xpehh ? p : nullptr;
-    s.PA = xpehh ? p + s.nw : nullptr;
-    s.lst = (unsigned short *)(p + (xpehh ? 2 * s.nw : 0));
+    s.N = p; p += s.nw;
+    s.S = p; p += s.ns;
+    s.isA = p; p += xpehh ? s.nw : 0;
+    s.PA = p;
+    s.gtk = (unsigned *)scratch;
     return s;
 }
 
@@ -555,228 +492,258 @@ __device__ __forceinline__ unsigned count_a(const SplitSmem &s, int x)
     return s.PA[x >> 5] + (unsigned)__popc(s.isA[x >> 5] & ((1u << (x & 31)) - 1u));
 }
 
-// Offsets of the kWin step counts and placement of the K staged boundaries
-// (position | step in window << 16 | rank in step << 32) by step.
-template <int G, typename Tile>
-__device__ const unsigned short *place_window(const Tile &tile, const SplitSmem &s, unsigned K,
-                                             const unsigned long long *stage, unsigned short *list)
+// The run boundaries of a window in position order: positions t with M[t] <=
+// hi (ALL), or only those that are no older run start (M[t] >= the window's
+// first step).  Each lane turns 32 neighbouring run lengths into a bitmap word:
+// the 16x2 clamp to [hi, hi + 1] less hi leaves the bit "not yet parted", the
+// slot's layout puts the bits in position order.  `merge` first adds the
+// previous window's boundaries (N) to the older run starts (O).  Returns the
+// number of boundaries, K0 of them before position n0; sup gets one bit per
+// summary word of O (at most 17 words: n <= 16383).
+template <int NPOP, typename Tile>
+__device__ __forceinline__ unsigned mark_window(const Tile &tile, const SplitSmem &s, const uint4 *M4,
+                                                int n, int n0, int hi, bool all, bool merge,
+                                                unsigned &K0, unsigned &sup)
 {
     const int lane = tile.thread_rank();
-    tile.sync();
-    constexpr int C = kWin / G;
-    unsigned own = 0;
+    const unsigned short *M16 = (const unsigned short *)M4;
+    const unsigned PP = (unsigned)(hi + 1) * 0x00010001u, P1 = PP - 0x00010001u;
+    unsigned K = 0u, c0 = 0u;
+    sup = 0u;
+    for (int it = 0; it < s.ns; ++it) {
+        const int wd = it * 32 + lane;
+        unsigned o = 0u, hit = 0u;
+        if (wd < s.nw) {
+            o = s.O[wd];
+            if (merge) {
+                o |= s.N[wd];
+                s.O[wd] = o;
+            }
+            if (32 * wd < n) {
+                uint4 q[4];
 #pragma unroll
-    for (int j = 0; j < C; ++j) own += s.cnt[C * lane + j];
-    unsigned incl = own;
+                for (int u = 0; u < 4; ++u) q[u] = __ldg(M4 + 4 * wd + u);
+                unsigned acc = 0u;               // word j's bits land at j and 16 + j
 #pragma unroll
-    for (int d = 1; d < G; d <<= 1) {
-        const unsigned v = tile.shfl_up(incl, d);
-        if (lane >= d) incl += v;
-    }
-    unsigned run = incl - own;
-#pragma unroll
-    for (int j = 0; j < C; ++j) {
-        const unsigned c = s.cnt[C * lane + j];
-        s.off[C * lane + j] = run;
-        run += c;
-    }
-    if (lane == G - 1) s.off[kWin] = incl;
-    tile.sync();
-    // the list goes to shared memory when it fits, else to the global scratch
-    unsigned short *dst = K <= (unsigned)kSplitListSmem ? s.lst : list;
-    for (unsigned j = lane; j < K; j += G) {
-        const unsigned long long e = stage[j];
-        dst[s.off[(unsigned)(e >> 16) & (kWin - 1u)] + (unsigned)(e >> 32)] = (unsigned short)(e & 0xFFFFu);
-    }
-    tile.sync();
-    return dst;
-}
-
-// Group the boundaries t with lo <= M[t] < lo + kWin by step: one pass over M
-// (8 values per 16-byte load, four loads in flight per lane) marks the values
-// in the window with two integer operations per 16-bit half; only the marked
-// ones are ranked inside their step and staged, then placed by step.  Done by
-// one tile of G lanes.  Window starts stay below 65,001 (run lengths are at
-// most 65,000), so the all-ones fill past the slot's end is never marked.
-template <int G, typename Tile>
-__device__ const unsigned short *build_window(const Tile &tile, const SplitSmem &s, const unsigned *M32,
-                                              int n, int lo, unsigned long long *stage,
-                                              unsigned short *list)
-{
-    const int lane = tile.thread_rank();
-    const uint4 *M4 = (const uint4 *)M32;
-    const unsigned short *M16 = (const unsigned short *)M32;
-    for (int q = lane; q < kWin; q += G) s.cnt[q] = 0u;
-    tile.sync();
-    const int n4 = (n + 7) >> 3;
-    constexpr unsigned kOut = 0xFFFFu & ~(kWin - 1u);      // a 16-bit difference is in the window
-    const unsigned ulo = (unsigned)lo, uhi = (unsigned)lo << 16;
-    unsigned K = 0;
-    for (int base = 0; base < n4; base += 4 * G) {
-        uint4 q[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int idx = base + u * G + lane;
-            q[u] = idx < n4 ? __ldg(M4 + idx) : make_uint4(~0u, ~0u, ~0u, ~0u);
-        }
-        // bit 8u + v: value v of this lane's u-th group of eight is in the window
-        unsigned hit = 0u;
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const unsigned wv[4] = {q[u].x, q[u].y, q[u].z, q[u].w};
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                if (((wv[j] - ulo) & kOut) == 0u) hit |= 1u << (8 * u + 2 * j);
-                if (((wv[j] - uhi) & (kOut << 16)) == 0u) hit |= 1u << (8 * u + 2 * j + 1);
+                for (int u = 3; u >= 0; --u) {
+                    acc = acc + acc + (__vmaxu2(__vminu2(q[u].w, PP), P1) - P1);
+                    acc = acc + acc + (__vmaxu2(__vminu2(q[u].z, PP), P1) - P1);
+                    acc = acc + acc + (__vmaxu2(__vminu2(q[u].y, PP), P1) - P1);
+                    acc = acc + acc + (__vmaxu2(__vminu2(q[u].x, PP), P1) - P1);
+                }
+                hit = ~acc & (n - 32 * wd >= 32 ? 0xFFFFFFFFu : (1u << (n - 32 * wd)) - 1u);
+                s.N[wd] = hit & ~o;
+                if (!all) hit &= ~o;
             }
         }
-        if (base + 4 * G > n4 && (n & 7)) {      // the last group holds values past n
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (base + u * G + lane == n4 - 1) hit &= ~(((0xFFu << (n & 7)) & 0xFFu) << (8 * u));
-        }
-        if (tile.ballot(hit != 0u) == 0u) continue;
+        const unsigned bal = tile.ballot(o != 0u);
+        if (lane == 0) s.S[it] = bal;
+        sup |= bal ? 1u << it : 0u;
+        const int below = n0 - 32 * wd;          // positions of this word before n0
+        c0 += (unsigned)__popc(hit & (below >= 32 ? 0xFFFFFFFFu : below > 0 ? (1u << below) - 1u : 0u));
         const unsigned c = (unsigned)__popc(hit);
         unsigned incl = c;
 #pragma unroll
-        for (int d = 1; d < G; d <<= 1) {
+        for (int d = 1; d < 32; d <<= 1) {
             const unsigned v = tile.shfl_up(incl, d);
             if (lane >= d) incl += v;
         }
         unsigned at = K + incl - c;
         while (hit) {
-            const int bb = __ffs(hit) - 1;
+            const int b = __ffs(hit) - 1;
             hit &= hit - 1u;
-            const int t = (base + (bb >> 3) * G + lane) * 8 + (bb & 7);
-            const unsigned d = (unsigned)__ldg(M16 + t) - ulo;
-            const unsigned r = atomicAdd(s.cnt + d, 1u);
-            stage[at++] = (unsigned long long)t | ((unsigned long long)d << 16) | ((unsigned long long)r << 32);
+            const int t = 32 * wd + b;
+            const unsigned tok = (unsigned)t | ((unsigned)__ldg(M16 + 32 * wd + ((b & 15) << 1 | b >> 4)) << 16);
+            unsigned *dst = at < (unsigned)kTokSmem ? s.tk : s.gtk;
+            if (NPOP == 2) *(uint2 *)(dst + 2 * at) = make_uint2(tok, count_a(s, t));
+            else dst[at] = tok;
+            ++at;
         }
-        K += tile.shfl(incl, G - 1);
+        K += tile.shfl(incl, 31);
     }
-    return place_window<G>(tile, s, K, stage, list);
+    K0 = (unsigned)__reduce_add_sync(0xFFFFFFFFu, (int)c0);
+    tile.sync();
+    return K;
 }
 
-
-// Pair counts fit 32 bits (C(16383, 2) < 2^32); the digest and the cutoff
-// product are 64-bit.
-// The trapezoid sum (Eq. 4 / Eq. 5) is kept per lane: the lane that owns
-// step i of the current G-step block (the lane whose map step it computed)
-// records that step's integer term S(i-1) + S(i) in `rec`, and once per
-// block every lane adds rec * g to its FP64 partial sum; the partial sums are
-// added over the tile by a fixed butterfly when the walk ends.  One FP64
-// multiply-add per lane and block instead of one per step (FP64 is a narrow
-// pipe on this GPU); with 32-lane tiles the additions are exactly those of the
-// per-step walk, so a walk handed over to it gives the same bits.
-struct ClassWalk {
-    unsigned D, S;
-    unsigned rec;                   // this lane's step term of the current block (0: none)
-    unsigned long long dig;
-    unsigned thr;                   // stop at the first S < thr, i.e. cut_den * S < cut_num * D
-    double acc;                     // this lane's partial trapezoid sum
-    int stop;                       // the step the walk stopped at (status: at the end)
-    bool active;
+// Sums of squared run lengths over the list entries [ka, kb), cut at the
+// boundaries of steps up to this lane's step (token < lim): d[0] all
+// haplotypes, for XPEHH d[1] population A, d[2] population B.  last / lastA:
+// the run start so far (position, population-A haplotypes before it).
+template <int NPOP>
+struct RunCut {
+    unsigned lim, last, lastA, d[NPOP == 2 ? 3 : 1];
+    __device__ __forceinline__ void cut(unsigned t, unsigned ta)
+    {
+        const unsigned p = t & 0xFFFFu, l = p - last;
+        if (NPOP == 2) {
+            const unsigned la = ta - lastA, lb = l - la;
+            if (t < lim) {
+                d[0] += l * l;
+                d[NPOP == 2 ? 1 : 0] += la * la;
+                d[NPOP == 2 ? 2 : 0] += lb * lb;
+                last = p;
+                lastA = ta;
+            }
+        } else if (t < lim) {
+            d[0] += l * l;
+            last = p;
+        }
+    }
+    // list entry k
+    __device__ __forceinline__ void one(const SplitSmem &s, unsigned k)
+    {
+        const unsigned *src = k < (unsigned)kTokSmem ? s.tk : s.gtk;
+        if (NPOP == 2) {
+            const uint2 t = *(const uint2 *)(src + 2 * k);
+            cut(t.x, t.y);
+        } else {
+            cut(src[k], 0u);
+        }
+    }
+    // iHS: entries [ka, kb), upward
+    __device__ __forceinline__ void range(const SplitSmem &s, unsigned ka, unsigned kb)
+    {
+        unsigned k = ka;
+        const unsigned kv = kb < (unsigned)kTokSmem ? kb : (unsigned)kTokSmem;
+        for (; k < kv && (k & 3u); ++k) one(s, k);
+#pragma unroll 2
+        for (; k + 4 <= kv; k += 4) {
+            const uint4 t = *(const uint4 *)(s.tk + k);
+            cut(t.x, 0u);
+            cut(t.y, 0u);
+            cut(t.z, 0u);
+            cut(t.w, 0u);
+        }
+        for (; k < kb; ++k) one(s, k);
+    }
+    // XPEHH: entries [0, K) from both ends at once: the lower half of the warp
+    // runs upward from position 0, the upper half downward from position n (the
+    // squares do not see the sign); the run between their last cuts closes it
+    template <typename Tile>
+    __device__ __forceinline__ void both_ends(const Tile &tile, const SplitSmem &s, unsigned K, unsigned n,
+                                              unsigned nA)
+    {
+        const bool up = tile.thread_rank() < 16;
+        last = up ? 0u : n;
+        lastA = up ? 0u : nA;
+        const unsigned half = K >> 1;
+        if (K <= (unsigned)kTokSmem) {
+            const uint2 *q = (const uint2 *)s.tk + (up ? 0u : K - 1u);
+            const int st = up ? 1 : -1;
+#pragma unroll 4
+            for (unsigned x = 0; x < half; ++x, q += st) cut(q->x, q->y);
+        } else {
+            for (unsigned x = 0; x < half; ++x) one(s, up ? x : K - 1u - x);
+        }
+        if ((K & 1u) && up) one(s, half);
+        const unsigned l = last - (unsigned)__shfl_xor_sync(0xFFFFFFFFu, last, 16);
+        const unsigned la = lastA - (unsigned)__shfl_xor_sync(0xFFFFFFFFu, lastA, 16), lb = l - la;
+#pragma unroll
+        for (int q = 0; q < (NPOP == 2 ? 3 : 1); ++q) d[q] += __shfl_xor_sync(0xFFFFFFFFu, d[q], 16);
+        d[0] += l * l;
+        d[NPOP == 2 ? 1 : 0] += la * la;
+        d[NPOP == 2 ? 2 : 0] += lb * lb;
+    }
 };
 
-// Reductions of S caused by the boundaries b that part at this step
-// (iHS: d0 class 0, d1 class 1; XPEHH: d0 A, d1 B, d2 pooled).  The pairs
-// whose common run ends exactly at step i are counted once, at the leftmost
-// boundary b of their span with M[b] = i: the first member lies in [p, b),
-// p the last run start before b with M <= i (the bitmap A, this step's
-// starts included), the second in [b, e), e the first old start after b
-// (M < i, the bitmap O).  So boundary b removes (b - p)(e - b) pairs, and
-// per population the products of its members on either side.
-template <int NPOP>
-__device__ __forceinline__ void split_terms(const SplitSmem &s, int b, int n0, unsigned supA,
-                                            unsigned supO, int &d0, int &d1, int &d2)
-{
-    const int p = prev_start(s.A, s.SA, supA, b);
-    const int e = next_start(s.O, s.SO, supO, b);
-    if (NPOP == 2) {
-        const unsigned ap = count_a(s, p), ab = count_a(s, b), ae = count_a(s, e);
-        const unsigned l1a = ab - ap, l2a = ae - ab;
-        const unsigned l1b = (unsigned)(b - p) - l1a, l2b = (unsigned)(e - b) - l2a;
-        d0 -= (int)(l1a * l2a);
-        d1 -= (int)(l1b * l2b);
-        d2 -= (b - p) * (e - b);
-    } else {
-        const int dd = (b - p) * (e - b);
-        if (b < n0) d0 -= dd;
-        else d1 -= dd;
-    }
-}
-
-// Steps that part more than G pairs (a few per walk): kept out of line so
-// that the common one-round path stays small in the instruction cache.
-template <int NPOP, int G, typename Tile>
-__device__ __noinline__ unsigned split_many(const Tile &tile, const SplitSmem &s,
-                                            const unsigned short *list, unsigned j0, unsigned j1,
-                                            int n0, unsigned supA, unsigned supO, int &d0, int &d1,
-                                            int &d2)
+// Drops of S by step (s.dec) from a window's K new boundaries, one per lane:
+// the pairs whose common run ends exactly at step v are counted once, at the
+// leftmost boundary b of their span with M[b] = v: the first member lies in
+// [p, b), p the last run start before b with M <= v, the second in [b, e), e
+// the first run start after b with M < v.  p and e are the nearest older run
+// start (bitmap O) or a nearer boundary of the window itself (the neighbours
+// in the list).  So boundary b removes (b - p)(e - b) pairs at step v, and per
+// population the products of its members on either side.
+template <int NPOP, typename Tile>
+__device__ __forceinline__ void sparse_terms(const Tile &tile, const SplitSmem &s, unsigned K, int lo, int n0,
+                                             unsigned sup, bool act0, bool act1)
 {
     const int lane = tile.thread_rank();
-    unsigned r = 0u;
-    for (unsigned j = j0 + lane; j < j1; j += G) {
-        const int b = list[j];
-        atomicOr(s.A + (b >> 5), 1u << (b & 31));
-        atomicOr(s.SA + (b >> 10), 1u << ((b >> 5) & 31));
-        r |= 1u << (b >> 10);
-    }
-    r = __reduce_or_sync(G == 32 ? 0xFFFFFFFFu : (0xFFFFu << (threadIdx.x & 16)), r);
+    for (int q = lane; q < kWin * (NPOP == 2 ? 3 : 2); q += 32) s.dec[q] = 0u;
     tile.sync();
-    for (unsigned j = j0 + lane; j < j1; j += G)
-        split_terms<NPOP>(s, (int)list[j], n0, supA | r, supO, d0, d1, d2);
-    tile.sync();
-    for (unsigned j = j0 + lane; j < j1; j += G) {
-        const int b = list[j];
-        atomicOr(s.O + (b >> 5), 1u << (b & 31));
-        atomicOr(s.SO + (b >> 10), 1u << ((b >> 5) & 31));
+    for (unsigned k = lane; k < K; k += 32) {
+        const unsigned t = s.tk[NPOP * k];
+        const int b = (int)(t & 0xFFFFu);
+        const unsigned v = t >> 16;
+        if (NPOP == 1 && !(b < n0 ? act0 : act1)) continue;
+        int p = prev_start(s.O, s.S, sup, b), e = next_start(s.O, s.S, sup, b);
+        for (int q = (int)k - 1; q >= 0; --q) {
+            const unsigned u = s.tk[NPOP * q];
+            const int x = (int)(u & 0xFFFFu);
+            if (x < p) break;
+            if (u >> 16 <= v) { p = x; break; }
+        }
+        for (unsigned q = k + 1; q < K; ++q) {
+            const unsigned u = s.tk[NPOP * q];
+            const int x = (int)(u & 0xFFFFu);
+            if (x > e) break;
+            if (u >> 16 < v) { e = x; break; }
+        }
+        unsigned *dec = s.dec + (v - (unsigned)lo);
+        const unsigned dd = (unsigned)((b - p) * (e - b));
+        if (NPOP == 2) {
+            const unsigned ab = s.tk[NPOP * k + 1];
+            const unsigned la = ab - count_a(s, p), ra = count_a(s, e) - ab;
+            atomicAdd(dec, la * ra);
+            atomicAdd(dec + kWin, ((unsigned)(b - p) - la) * ((unsigned)(e - b) - ra));
+            atomicAdd(dec + 2 * kWin, dd);
+        } else {
+            atomicAdd(dec + (b < n0 ? 0 : kWin), dd);
+        }
     }
-    return r;                                    // summary words that gained a start
+    tile.sync();
 }
 
 }  // namespace
 
 size_t split_smem_per_warp(int n, int xpehh)
 {
-    const int nw = split_nw(n), ns = (nw + 31) >> 5;
-    size_t b = (size_t)nw * 4 * 2 + (size_t)ns * 4 * 2 + (size_t)(2 * kWin + 1) * 4;
-    if (xpehh) b += (size_t)nw * 4 * 2;
-    b += (size_t)kSplitListSmem * 2;
-    return (b + 15) & ~(size_t)15;
+    return ((size_t)split_words(n, xpehh) * 4 + 15) & ~(size_t)15;
 }
 
-size_t split_scratch_per_warp(int n) { return (((size_t)n * 10) + 255) & ~(size_t)255; }
+size_t split_scratch_per_warp(int n) { return (((size_t)n * 8) + 255) & ~(size_t)255; }
 
-// Persistent: each tile of G lanes (a warp, or half a warp so that one warp
-// walks two cores at once) takes slots of this stage (both directions) from a
-// counter and walks the cores in them.  iHS walks run four CTAs per SM at 64
-// registers; the XPEHH walk (three pair counts per boundary, the population
-// prefix table) spills more at that cap and runs three at 80 (1M XPEHH scan:
-// 51.35 ms against 51.82).
+// Persistent: each warp takes slots of this stage (both directions) from a
+// counter and walks the cores in them.  The first window is the steps 1..32:
+// every lane runs over all boundaries with M <= 32 (shared memory, broadcast
+// reads) and cuts at those of its own step, so S(i) = (sum of squared run
+// lengths - haplotypes) / 2 of 32 steps costs about six instructions per
+// boundary, where a step at a time needs two bitmap searches, three shared
+// atomics and two warp sums per step with most lanes idle.  Later windows of
+// 64 steps hold few boundaries among many older run starts: there each lane
+// takes one boundary (sparse_terms); a window with more than kSparseMax of
+// them is cut like the first one, 32 steps at a time.
+// Pair counts fit 32 bits (C(16383, 2) < 2^32); the digest is 64-bit.  Lane
+// (i - 1) mod 32 adds step i's trapezoid term to its own FP64 partial sum, and
+// the partial sums meet in a fixed butterfly when the walk ends: the order of
+// the per-step walk, so a walk handed over to it gives the same bits.
 #ifndef SPLIT_MIN_CTAS
 #define SPLIT_MIN_CTAS 4
 #endif
 template <int NPOP, int G>
 __global__ void __launch_bounds__(kSplitWarps * 32, NPOP == 2 ? 3 : SPLIT_MIN_CTAS) split_walk_kernel(SweepArgs w)
 {
+    static_assert(G == 32, "lane l owns step l of a block of 32");
     extern __shared__ __align__(16) unsigned char smem[];
     namespace cg = cooperative_groups;
     const cg::thread_block_tile<G> tile = cg::tiled_partition<G>(cg::this_thread_block());
-    constexpr int TPC = kSplitWarps * 32 / G;            // tiles per CTA
+    constexpr int NV = NPOP == 2 ? 3 : 2;     // S values: class 0, class 1; or A, B, pooled
+    constexpr int NWK = NPOP == 2 ? 1 : 2;    // walks of a slot
+    constexpr int kDense = NPOP == 2 ? 16 : 32;   // steps of a window cut boundary by boundary
     const int lane = tile.thread_rank(), tix = threadIdx.x / G;
     const int n = w.n;
-    SplitSmem s = split_smem(smem + (size_t)tix * w.split_bytes, n, NPOP == 2);
-    unsigned char *scr = w.wscratch + ((size_t)blockIdx.x * TPC + tix) * w.wscratch_bytes;
-    unsigned long long *stage = (unsigned long long *)scr;
-    unsigned short *list = (unsigned short *)(scr + (size_t)n * 8);
+    const SplitSmem s = split_smem(smem + (size_t)tix * w.split_bytes,
+                                   w.wscratch + ((size_t)blockIdx.x * kSplitWarps + tix) * w.wscratch_bytes,
+                                   n, NPOP == 2);
     const long long per_dir = (long long)w.nch * w.R;
     const long long m = w.a.m;
+    unsigned long long nxt = 0;               // the slot after this one, fetched ahead
+    if (lane == 0) nxt = atomicAdd(w.walk_head, 1ull);
     for (;;) {
-        unsigned long long gs = 0;
-        if (lane == 0) gs = atomicAdd(w.walk_head, 1ull);
-        gs = tile.shfl(gs, 0);
+        const unsigned long long gs = tile.shfl(nxt, 0);
         if (gs >= (unsigned long long)(2 * per_dir)) break;
+        if (lane == 0) nxt = atomicAdd(w.walk_head, 1ull);
         // slot counts are below 2^31 (2 x chunks x stage cores): 32-bit decode
         const unsigned gsl = (unsigned)gs;
         const long long gslot = (long long)gs;
@@ -804,11 +771,15 @@ __global__ void __launch_bounds__(kSplitWarps * 32, NPOP == 2 ? 3 : SPLIT_MIN_CT
         const unsigned char *slot = w.slots + (size_t)gslot * w.slot_bytes;
         const int n0 = ((const int *)slot)[0];
         const int hz = ((const int *)slot)[1];
-        const int w1 = ((const int *)slot)[2];
-        const unsigned *M32 = (const unsigned *)(slot + 16);
+        const uint4 *M4 = (const uint4 *)(slot + 16);
 
-        for (int q = lane; q < s.nw; q += G) { s.O[q] = 0u; s.A[q] = 0u; }
-        for (int q = lane; q < s.ns; q += G) { s.SO[q] = 0u; s.SA[q] = 0u; }
+        for (int q = lane; q < s.nw; q += G) {   // run starts before step 1: 0, n0, n
+            unsigned o = q == 0 ? 1u : 0u;
+            if (q == n0 >> 5) o |= 1u << (n0 & 31);
+            if (q == n >> 5) o |= 1u << (n & 31);
+            s.O[q] = o;
+            s.N[q] = 0u;
+        }
         if (NPOP == 2) {
             const unsigned *isA = (const unsigned *)(slot + slot_isa_at(n));
             unsigned carry = 0u;
@@ -827,91 +798,68 @@ __global__ void __launch_bounds__(kSplitWarps * 32, NPOP == 2 ? 3 : SPLIT_MIN_CT
             }
         }
         tile.sync();
-        if (lane < 3) {                           // run starts before step 1: 0, n0, n
-            const int mk = lane == 0 ? 0 : (lane == 1 ? n0 : n);
-            atomicOr(s.O + (mk >> 5), 1u << (mk & 31));
-            atomicOr(s.SO + (mk >> 10), 1u << ((mk >> 5) & 31));
-            atomicOr(s.A + (mk >> 5), 1u << (mk & 31));
-            atomicOr(s.SA + (mk >> 10), 1u << ((mk >> 5) & 31));
-        }
-        tile.sync();
-        // summary words with a start (third level of both bitmaps)
-        unsigned supA = 1u | (1u << (n0 >> 10)) | (1u << (n >> 10)), supO = supA;
 
         // ---- step 0 (the core marker splits the sample into its allele classes)
-        constexpr int NWK = NPOP == 2 ? 1 : 2;    // walks handled by this warp
-        ClassWalk cw[NWK];
-        unsigned SA = 0, SB = 0, pA = 0, pB = 0, DA = 0, DB = 0;
-        unsigned long long dA = 0, dB = 0;
-        double accB = 0.0;                  // XPEHH: population B's partial sum (A's in cw[0])
-        unsigned recB = 0;
+        unsigned S[NV], prev[NV];             // S of this lane's step; S of the step before the block
+        unsigned D[NV], thr[NWK];             // C(N, 2); a walk stops at the first S < thr
         if (NPOP == 2) {
             const unsigned nA = (unsigned)w.a.nA, nB = (unsigned)w.a.nB;
             const unsigned a0 = count_a(s, n0), a1 = nA - a0;
             const unsigned b0 = (unsigned)n0 - a0, b1 = nB - b0;
-            SA = (unsigned)(c2i(a0) + c2i(a1));
-            SB = (unsigned)(c2i(b0) + c2i(b1));
-            DA = (unsigned)c2i(nA);
-            DB = (unsigned)c2i(nB);
-            cw[0].D = (unsigned)c2i((unsigned)n);
-            cw[0].S = (unsigned)(c2i((unsigned)n0) + c2i((unsigned)(n - n0)));
-            pA = SA; pB = SB;
-            dA = SA; dB = SB;
+            prev[0] = (unsigned)(c2i(a0) + c2i(a1));
+            prev[1] = (unsigned)(c2i(b0) + c2i(b1));
+            prev[NV - 1] = (unsigned)(c2i((unsigned)n0) + c2i((unsigned)(n - n0)));
+            D[0] = (unsigned)c2i(nA);
+            D[1] = (unsigned)c2i(nB);
+            D[NV - 1] = (unsigned)c2i((unsigned)n);
         } else {
-            cw[0].D = (unsigned)c2i((unsigned)n0);             // allele 0: positions [0, n0)
-            cw[1].D = (unsigned)c2i((unsigned)(n - n0));       // allele 1: positions [n0, n)
-            cw[0].S = cw[0].D;
-            cw[1].S = cw[1].D;
+            prev[0] = D[0] = (unsigned)c2i((unsigned)n0);             // allele 0: positions [0, n0)
+            prev[1] = D[1] = (unsigned)c2i((unsigned)(n - n0));       // allele 1: positions [n0, n)
         }
+        unsigned long long dig[NV];           // this lane's part of the digests
+        double acc[2] = {0.0, 0.0};           // this lane's partial trapezoid sums
+        bool act[NWK];
+        int stop[NWK];
+        unsigned skey[NWK];                   // S where an unfinished walk left off
         bool any = false;
 #pragma unroll
-        for (int q = 0; q < NWK; ++q) {
-            {
-                const unsigned long long t =
-                    ((unsigned long long)w.a.cut_num * cw[q].D + w.a.cut_den - 1u) / w.a.cut_den;
-                cw[q].thr = t < 0xFFFFFFFFull ? (unsigned)t : 0xFFFFFFFFu;
-            }
-            cw[q].dig = cw[q].S;
-            cw[q].acc = 0.0;
-            cw[q].rec = 0u;
-            cw[q].stop = 0;
-            cw[q].active = cw[q].D != 0u;
-            any |= cw[q].active;
-        }
-
-        const long long step = dir ? 1 : -1;
-        double gq = 0.0;        // this lane's step of the current G-step block: the map step g
-        int gk = 0;             // its kind: 0 a step, WALK_EDGE past the array end, WALK_GAP a gap abort
-        // steps [lo, lo + wlen) are grouped in cl: first the slot's window
-        // (steps 1..w1), then windows of kWin steps found in M
-        int lo = 1, wlen = w1 > 0 ? w1 : kWin;
-        const unsigned short *cl = s.lst;
-        if (any) {
-            if (w1 > 0) {                        // the slot's list, copied on chip
-                const unsigned short *so = (const unsigned short *)(slot + slot_off_at(n, NPOP == 2));
-                const unsigned *sl = (const unsigned *)(slot + slot_list_at(n, NPOP == 2));
-                for (int q = lane; q <= w1; q += G) s.off[q] = so[q];
-                const int kw = ((int)so[w1] + 1) >> 1;
-#pragma unroll 4
-                for (int q = lane; q < kw; q += G) ((unsigned *)s.lst)[q] = __ldg(sl + q);
-                tile.sync();
-            } else {
-                cl = build_window<G>(tile, s, M32, n, lo, stage, list);
-            }
-        }
-        int fin = WALK_OK;                           // how the still-active walks end
-        int i = 1;                              // walks stay below 2^31 steps (a chunk history)
-        for (; any; ++i) {
-            const int own_step = (int)((i - 1) & (G - 1));   // the lane that owns step i
-            if (own_step == 0) {                  // gaps and map steps of the next G steps
-                if (i > 1) {                      // the previous block's terms
+        for (int q = 0; q < NV; ++q) dig[q] = lane == 0 ? prev[q] : 0u;
 #pragma unroll
-                    for (int q = 0; q < NWK; ++q) { cw[q].acc += (double)cw[q].rec * gq; cw[q].rec = 0u; }
-                    if (NPOP == 2) { accB += (double)recB * gq; recB = 0u; }
-                }
-                const long long xl = k + step * (i + lane), xp = xl - step;
-                gq = 0.0;
-                gk = 0;
+        for (int q = 0; q < NWK; ++q) {
+            const unsigned Dq = D[NPOP == 2 ? NV - 1 : q];
+            const unsigned long long t =
+                ((unsigned long long)w.a.cut_num * Dq + w.a.cut_den - 1u) / w.a.cut_den;
+            thr[q] = t < 0xFFFFFFFFull ? (unsigned)t : 0xFFFFFFFFu;
+            stop[q] = 0;
+            skey[q] = 0u;
+            act[q] = Dq != 0u;
+            any |= act[q];
+        }
+        int fin = WALK_OK;                    // how the still-active walks end
+        int endstep = 0;
+        int lo = 1;                           // first step of the window
+        bool dense = true, merge = false;
+        while (any) {
+            unsigned K0, sup;
+            const int hi = lo + (dense ? kDense - 1 : kWin - 1);
+            const unsigned K = mark_window<NPOP>(tile, s, M4, n, n0, hi, dense, merge, K0, sup);
+            if (!dense && K > (unsigned)kSparseMax) {    // redo as a window of 32 steps
+                dense = true;
+                merge = false;
+                continue;
+            }
+            if (!dense) sparse_terms<NPOP>(tile, s, K, lo, n0, sup, act[0], act[NWK - 1]);
+            for (int b0 = lo; b0 <= hi; b0 += 32) {
+                // the step of this lane: its map distance g, or how the walk ends
+                // there.  Step i belongs to lane (i - 1) mod 32; the block is the
+                // lanes [la, lb)
+                const int la = (b0 - 1) & 31, i0 = b0 - la, i = i0 + lane;
+                const int lb = la + (hi - b0 + 1 < 32 ? hi - b0 + 1 : 32);
+                const bool mine = lane >= la && lane < lb;
+                double gq = 0.0;
+                int gk = 0;                   // 0 a step, WALK_EDGE past the array end, WALK_GAP a gap abort
+                const long long step = dir ? 1 : -1;
+                const long long xl = k + step * i, xp = xl - step;
                 if (xl < 0 || xl >= m) gk = WALK_EDGE;
                 else {
                     const long long p1 = __ldg(w.a.pos + xl), p0 = __ldg(w.a.pos + xp);
@@ -928,133 +876,129 @@ __global__ void __launch_bounds__(kSplitWarps * 32, NPOP == 2 ? 3 : SPLIT_MIN_CT
                         gq = gg;
                     }
                 }
-            }
-            const int kind = tile.shfl(gk, own_step);
-            if (kind != 0) { fin = kind; break; }
-            const bool own = lane == own_step;
-            if (i > hz) { fin = WALK_UNFINISHED; break; }
-            if (i >= lo + wlen) {
-                lo += wlen;
-                wlen = kWin;
-                cl = build_window<G>(tile, s, M32, n, lo, stage, list);
-            }
-            // ---- the boundaries that part at this step
-            const unsigned j0 = s.off[i - lo], j1 = s.off[i - lo + 1];
-            int d0 = 0, d1 = 0, d2 = 0;
-            if (j1 > j0) {
-                // new run starts first, then their reductions, then merge
-                if (j1 - j0 <= (unsigned)G) {     // one boundary per lane, loaded once
-                    bool has = lane < (int)(j1 - j0);
-                    const int b = has ? (int)cl[j0 + lane] : 0;
-                    // an iHS class whose walk has ended needs its runs no more
-                    if (NPOP == 1) has = has && (b < n0 ? cw[0].active : cw[NWK - 1].active);
-                    const unsigned bw = 1u << (b & 31), sw = 1u << ((b >> 5) & 31);
-                    if (tile.ballot(has) != 0u) {
-                    if (has) {
-                        atomicOr(s.A + (b >> 5), bw);
-                        atomicOr(s.SA + (b >> 10), sw);
-                    }
-                    const unsigned r = __reduce_or_sync(G == 32 ? 0xFFFFFFFFu : (0xFFFFu << (threadIdx.x & 16)),
-                                                        has ? 1u << (b >> 10) : 0u);
-                    supA |= r;
-                    tile.sync();
-                    if (has) split_terms<NPOP>(s, b, n0, supA, supO, d0, d1, d2);
-                    tile.sync();
-                    // this step's starts become old ones; the next step reads O
-                    // only after its own sync
-                    if (has) {
-                        atomicOr(s.O + (b >> 5), bw);
-                        atomicOr(s.SO + (b >> 10), sw);
-                    }
-                    supO |= r;
+                // S of this lane's step
+                if (dense) {
+                    RunCut<NPOP> rc;
+                    if (NPOP == 2) {
+                        // 16 steps, each by two lanes
+                        rc.lim = (unsigned)(i0 + la + (lane & 15) + 1) << 16;   // M <= i  <=>  token < lim
+                        rc.d[0] = rc.d[NPOP == 2 ? 1 : 0] = rc.d[NPOP == 2 ? 2 : 0] = 0u;
+                        rc.both_ends(tile, s, K, (unsigned)n, (unsigned)w.a.nA);
+                        S[0] = (rc.d[NPOP == 2 ? 1 : 0] - (unsigned)w.a.nA) >> 1;
+                        S[1] = (rc.d[NPOP == 2 ? 2 : 0] - (unsigned)w.a.nB) >> 1;
+                        S[NV - 1] = (rc.d[0] - (unsigned)n) >> 1;
+                    } else {
+                        rc.lim = (unsigned)(i + 1) << 16;
+                        S[0] = S[1] = 0u;
+                        if (act[0]) {
+                            rc.last = 0u;
+                            rc.d[0] = 0u;
+                            rc.range(s, 0u, K0);
+                            rc.cut((unsigned)n0, 0u);
+                            S[0] = (rc.d[0] - (unsigned)n0) >> 1;
+                        }
+                        if (act[NWK - 1]) {
+                            rc.last = (unsigned)n0;
+                            rc.d[0] = 0u;
+                            rc.range(s, K0, K);
+                            rc.cut((unsigned)n, 0u);
+                            S[1] = (rc.d[0] - (unsigned)(n - n0)) >> 1;
+                        }
                     }
                 } else {
-                    const unsigned r = split_many<NPOP, G>(tile, s, cl, j0, j1, n0, supA, supO, d0, d1, d2);
-                    supA |= r;
-                    supO |= r;
-                }
-                d0 = cg::reduce(tile, d0, cg::plus<int>());
-                d1 = cg::reduce(tile, d1, cg::plus<int>());
-                if (NPOP == 2) d2 = cg::reduce(tile, d2, cg::plus<int>());
-            }
-            const unsigned ii = (unsigned)(i + 1);
-            if (NPOP == 2) {
-                SA += (unsigned)d0;                  // the decrements are negative: S stays >= 0
-                SB += (unsigned)d1;
-                ClassWalk &q = cw[0];
-                q.S += (unsigned)d2;
-                dA += (unsigned long long)ii * SA;
-                dB += (unsigned long long)ii * SB;
-                q.dig += (unsigned long long)ii * q.S;
-                const bool stop = q.S < q.thr;
-                if (stop && !w.a.crossing) { q.stop = (int)i; q.active = false; }
-                else {
-                    if (own) {
-                        q.rec = pA + SA;
-                        recB = pB + SB;
+#pragma unroll
+                    for (int q = 0; q < NV; ++q) {
+                        unsigned dd = mine ? s.dec[q * kWin + (i - lo)] : 0u;
+#pragma unroll
+                        for (int d = 1; d < 32; d <<= 1) {
+                            const unsigned v = tile.shfl_up(dd, d);
+                            if (lane >= d) dd += v;
+                        }
+                        S[q] = prev[q] - dd;
                     }
-                    if (stop) { q.stop = (int)i; q.active = false; }
-                    pA = SA;
-                    pB = SB;
                 }
-            } else {
+                // where the block ends for the walks still running: a gap or the
+                // array end (tested before a step's S), else the history's end
+                const unsigned km = tile.ballot(mine && gk != 0), hm = tile.ballot(mine && i > hz);
+                const int ke = km ? __ffs(km) - 1 : lb, he = hm ? __ffs(hm) - 1 : lb;
+                const int end = ke <= he ? ke : he;
+                const int kfin = tile.shfl(gk, ke & 31);
+                any = false;
 #pragma unroll
-                for (int c_ = 0; c_ < 2; ++c_) {
-                    ClassWalk &q = cw[c_];
-                    if (!q.active) continue;
-                    q.S += (unsigned)(c_ ? d1 : d0);
-                    q.dig += (unsigned long long)ii * q.S;
-                    const bool stop = q.S < q.thr;
-                    if (stop && !w.a.crossing) { q.stop = (int)i; q.active = false; continue; }
-                    if (own) q.rec = 2u * q.S - (unsigned)(c_ ? d1 : d0);   // S(i - 1) + S(i)
-                    if (stop) { q.stop = (int)i; q.active = false; continue; }
+                for (int q = 0; q < NWK; ++q) {
+                    if (!act[q]) continue;
+                    const int sd = NPOP == 2 ? NV - 1 : q;
+                    const unsigned sm = tile.ballot(mine && S[sd] < thr[q]);
+                    const int sl = sm ? __ffs(sm) - 1 : lb;
+                    const bool stops = sl < end;
+                    const int full = stops ? sl : end;       // lanes below: whole steps
+                    const bool cnt = lane >= la && lane < full + (stops ? 1 : 0);
+                    const bool term = lane >= la && lane < full + (stops && w.a.crossing ? 1 : 0);
+                    if (end < lb) skey[q] = end > la ? tile.shfl(S[sd], (end - 1) & 31) : prev[sd];
+#pragma unroll
+                    for (int v = NPOP == 2 ? 0 : q; v <= (NPOP == 2 ? NV - 1 : q); ++v) {
+                        unsigned sp = tile.shfl_up(S[v], 1);
+                        if (lane == la) sp = prev[v];
+                        if (cnt) dig[v] += (unsigned long long)(unsigned)(i + 1) * S[v];
+                        if (term && v < 2) acc[v < 2 ? v : 0] += (double)(sp + S[v]) * gq;
+                        prev[v] = tile.shfl(S[v], lb - 1);
+                    }
+                    if (stops) {
+                        stop[q] = i0 + sl;
+                        act[q] = false;
+                    }
+                    any |= act[q];
+                }
+                if (!any) break;
+                if (end < lb) {
+                    fin = ke <= he ? kfin : WALK_UNFINISHED;
+                    endstep = i0 + end;
+                    any = false;
+                    break;
                 }
             }
-            any = false;
+            lo = hi + 1;
+            dense = (lo & 31) != 1;           // whole blocks of 32 from here on
+            merge = true;
+        }
+        // ---- the lanes' partial sums, then the results (lane 0)
 #pragma unroll
-            for (int q = 0; q < NWK; ++q) any |= cw[q].active;
-        }
-        // ---- the last block's terms, then the tile's sum of the partial sums
+        for (int q = 0; q < 2; ++q) acc[q] = lane_sum_f64<G>(acc[q]);
 #pragma unroll
-        for (int q = 0; q < NWK; ++q) {
-            cw[q].acc += (double)cw[q].rec * gq;
-            cw[q].acc = lane_sum_f64<G>(cw[q].acc);
+        for (int q = 0; q < NV; ++q) {
+#pragma unroll
+            for (int d = G / 2; d > 0; d >>= 1) dig[q] += __shfl_xor_sync(0xFFFFFFFFu, dig[q], d);
         }
-        if (NPOP == 2) {
-            accB += (double)recB * gq;
-            accB = lane_sum_f64<G>(accB);
-        }
-        // ---- results (lane 0)
         if (lane == 0) {
             const ItemSink &sk = w.sk;
 #pragma unroll
-            for (int q_ = 0; q_ < NWK; ++q_) {
-                ClassWalk &q = cw[q_];
+            for (int q = 0; q < NWK; ++q) {
+                const unsigned Dq = D[NPOP == 2 ? NV - 1 : q];
                 // iHS items: (allele 1, down), (allele 1, up), (allele 0, down), (allele 0, up)
                 const uint32_t item = NPOP == 2 ? (uint32_t)(k * 2 + dir)
-                                                : (uint32_t)(k * 4 + (q_ == 1 ? 0 : 2) + dir);
-                int status = q.D == 0u ? WALK_UNDEFINED : WALK_OK;
-                if (q.active) {
+                                                : (uint32_t)(k * 4 + (q == 1 ? 0 : 2) + dir);
+                int status = Dq == 0u ? WALK_UNDEFINED : WALK_OK;
+                if (act[q]) {
                     if (fin == WALK_UNFINISHED) {
                         const unsigned long long slot2 = atomicAdd(&sk.q->n2, 1ull);
                         sk.list2[slot2] = item;
-                        sk.key2[slot2] = bucket_of((float)((double)q.S / (double)q.D));
+                        sk.key2[slot2] = bucket_of((float)((double)skey[q] / (double)Dq));
                         continue;
                     }
                     status = fin;
-                    q.stop = (int)i;
+                    stop[q] = endstep;
                 }
                 sk.item_status[item] = (int8_t)status;
-                sk.stop[item] = q.stop;
+                sk.stop[item] = stop[q];
                 if (NPOP == 2) {
-                    sk.item_ihh[2 * (size_t)item] = DA ? q.acc / (2.0 * (double)DA) : 0.0;
-                    sk.item_ihh[2 * (size_t)item + 1] = DB ? accB / (2.0 * (double)DB) : 0.0;
-                    sk.digest[3 * (size_t)item] = dA;
-                    sk.digest[3 * (size_t)item + 1] = dB;
-                    sk.digest[3 * (size_t)item + 2] = q.dig;
+                    sk.item_ihh[2 * (size_t)item] = D[0] ? acc[0] / (2.0 * (double)D[0]) : 0.0;
+                    sk.item_ihh[2 * (size_t)item + 1] = D[1] ? acc[1] / (2.0 * (double)D[1]) : 0.0;
+                    sk.digest[3 * (size_t)item] = dig[0];
+                    sk.digest[3 * (size_t)item + 1] = dig[1];
+                    sk.digest[3 * (size_t)item + 2] = dig[NV - 1];
                 } else {
-                    sk.item_ihh[item] = q.D ? q.acc / (2.0 * (double)q.D) : 0.0;
-                    sk.digest[item] = q.D ? q.dig : 0ull;
+                    sk.item_ihh[item] = Dq ? acc[q] / (2.0 * (double)Dq) : 0.0;
+                    sk.digest[item] = Dq ? dig[q] : 0ull;
                 }
             }
         }
@@ -1068,18 +1012,14 @@ static void (*walk_kernel_for(int xpehh))(SweepArgs)
     return xpehh ? split_walk_kernel<2, G> : split_walk_kernel<1, G>;
 }
 
-static void (*walk_kernel(int xpehh, int tile))(SweepArgs)
-{
-    return tile == 16 ? walk_kernel_for<16>(xpehh) : walk_kernel_for<32>(xpehh);
-}
-
-int split_walk_ctas(int n, int xpehh, int tile)
+int split_walk_ctas(int n, int xpehh)
 {
     // resident CTAs of the persistent walker
     int per_sm = 0;
-    const size_t smem = split_smem_per_warp(n, xpehh) * (kSplitWarps * 32 / tile);
+    const size_t smem = split_smem_per_warp(n, xpehh) * kSplitWarps;
+    cudaFuncSetAttribute(walk_kernel_for<32>(xpehh), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &per_sm, walk_kernel(xpehh, tile), kSplitWarps * 32, smem);
+        &per_sm, walk_kernel_for<32>(xpehh), kSplitWarps * 32, smem);
     if (e != cudaSuccess || per_sm < 1) per_sm = 1;
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
@@ -1110,8 +1050,8 @@ cudaError_t launch_sweep_path(const SweepArgs &w0, cudaStream_t s)
         sweep = E <= 8 ? sweep_kernel<32, 8> : E <= 16 ? sweep_kernel<32, 16> : sweep_kernel<32, 32>;
     cudaError_t e = cudaFuncSetAttribute(sweep, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssm);
     if (e != cudaSuccess) return e;
-    const size_t wsm = (size_t)w.split_bytes * (kSplitWarps * 32 / w.split_tile);
-    void (*walk)(SweepArgs) = walk_kernel(w.a.nB > 0, w.split_tile);
+    const size_t wsm = (size_t)w.split_bytes * kSplitWarps;
+    void (*walk)(SweepArgs) = walk_kernel_for<32>(w.a.nB > 0);
     if ((e = cudaFuncSetAttribute(walk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wsm)) !=
         cudaSuccess)
         return e;
