@@ -127,16 +127,17 @@ typedef struct {
     void *walk_end_event;   /* optional cudaEvent_t, recorded after the last walk kernel */
     int32_t big_group_entries; /* groups with at least this many 32-bit words are split by the
                                   whole warp, smaller ones one lane each (0 = 32) */
-    int32_t sweep_warmup;      /* sweep schedule: markers sorted before a chunk's first core,
-                                  16..16384 (0 = 1536); walks longer than this may take the
-                                  second pass */
+    int32_t sweep_warmup;      /* sweep schedule: markers of history before a chunk's first core,
+                                  16..16384 (0 = 8192, or 1536 for samples above about 10,500
+                                  haplotypes, whose history is swept marker by marker); walks
+                                  longer than this may take the second pass */
     int32_t sweep_stage_cores; /* sweep schedule: cores per chunk between walk launches,
                                   1..8192 (0 = the whole chunk, capped so that the slot
                                   buffer stays near 24 GiB); sizes the slot buffer */
     int32_t sweep_threads;     /* sweep schedule: threads per sorting CTA, 32, 64, 128, 256
                                   or 512 (0 = the narrowest of 32 / 64 / 128 holding at most
-                                  8 haplotypes per thread, 16 on chromosomes with more
-                                  chunks than three 256-thread CTAs per SM hold; else 256
+                                  8 haplotypes per thread, 16 on chromosomes of more than
+                                  2,560 cores per SM; else 256
                                   up to 6144 haplotypes, else 512); a width is doubled until
                                   it holds at most 32 haplotypes per thread */
     int32_t sweep_split_tile;  /* sweep schedule: accepted for compatibility (0, 16 or 32); a
@@ -380,8 +381,10 @@ int selscan_pack(const uint8_t *hap01, int32_t n, int64_t m, int32_t hap_major,
 int32_t selscan_default_schedule(int32_t n_total, int64_t m, int32_t mode);
 
 /* Work of the sorting kernels of a sweep-schedule call: *marker_passes = the
- * markers all sorting CTAs step through over every stage (each chunk's cores
- * plus its warm-up, both directions), *elements = the sorted elements per
+ * markers all sorting CTAs step through over every stage, both directions
+ * (each chunk's cores), plus one per 32-marker word of each chunk's history
+ * (its starting state is sorted word by word; for samples above about 10,500
+ * haplotypes one per history marker), *elements = the sorted elements per
  * marker pass (n_total rounded up to the CTA's element grid).  Host only: no
  * device work.  Returns SELSCAN_OK, or SELSCAN_ERR_INVALID_ARG for bad
  * arguments or a launch that does not take the sweep schedule. */

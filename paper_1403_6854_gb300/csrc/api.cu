@@ -31,13 +31,14 @@ constexpr int kDefaultProbeSteps = 48;
 constexpr int kDefaultBigGroup = 32;
 constexpr int kMaxHaplotypes = 65000;
 constexpr int kDefaultSweepWarmup = 1536;
+constexpr int kDefaultSweepHistory = 8192;
 constexpr size_t kSweepSlotBudget = (size_t)24 << 30;  // bytes of sweep slots per scan
 constexpr long long kSweepMinMarkers = 32768;          // default sweep: m >= this +
 constexpr long long kSweepMinPerHaplotype = 4;         // this x n
 constexpr size_t kMaxSmemPerCta = 227 * 1024;
 
 struct SweepPlan {
-    int nch, L, R, nstages, threads;
+    int nch, L, R, nstages, threads, started;
     long long B;
     size_t state_bytes, slot_bytes;
     int split_bytes;
@@ -65,24 +66,28 @@ inline size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }
 SweepPlan make_sweep_plan(int n_total, long long m, int mode, const selscan_launch *L)
 {
     SweepPlan w;
-    w.L = (L && L->sweep_warmup > 0) ? L->sweep_warmup : kDefaultSweepWarmup;
+    // chunks start from a sorted state made directly from the history's 32-marker
+    // words where one CTA's shared memory holds the sort (n up to about 10,500);
+    // larger samples sweep the history marker by marker
+    w.started = start_smem_bytes(n_total, 512) <= kMaxSmemPerCta;
+    w.L = (L && L->sweep_warmup > 0) ? L->sweep_warmup : (w.started ? kDefaultSweepHistory : kDefaultSweepWarmup);
     if (w.L < 16) w.L = 16;
     if (w.L > 16384) w.L = 16384;
     w.R = (L && L->sweep_stage_cores > 0) ? L->sweep_stage_cores : 0;
     if (w.R > 8192) w.R = 8192;
-    // chunks are at least as long as their warm-up
-    const long long per = w.L > 256 ? w.L : 256;
+    // chunks of at least 256 cores; at least as long as a history that is swept
+    const long long per = !w.started && w.L > 256 ? w.L : 256;
     long long nch = (m + per - 1) / per;
     const int sms = device_sms();
     // sorting CTA width, for a small sample the narrowest of 32 / 64 / 128 /
-    // 256 threads that keeps it at about g elements per thread: g = 8 while
-    // every chunk runs at once anyway (a marker's latency is what counts: one
-    // warp sorting 8 elements a lane beats eight warps sorting mostly padding,
-    // and loses with 16), g = 16 when the chromosome has more chunks than three
-    // 256-thread CTAs per SM hold (narrow CTAs then run more, shorter chunks at
-    // once).  Larger samples: 256 threads up to 6,144 haplotypes, else 512
+    // 256 threads that keeps it at about g elements per thread.  g = 8: a
+    // marker's latency is what counts (1,000 haplotypes x 200,000 markers: 0.68
+    // ms of marker passes against 0.88 with g = 16, whose twice as many chunks
+    // also sort twice as many starting states).  g = 16 once those are a small
+    // part, above 2,560 cores per SM (1,000 x 1,000,000: sort 4.83 ms against
+    // 5.37).  Larger samples: 256 threads up to 6,144 haplotypes, else 512
     const int want = L ? L->sweep_threads : 0;
-    const long long g = nch > (3ll * sms) / 2 ? 16 : 8;
+    const long long g = m > 2560ll * sms ? 16 : 8;
     if (want == 32 || want == 64 || want == 128 || want == 256 || want == 512) w.threads = want;
     else if (n_total <= 128 * g)
         w.threads = n_total <= 32 * g ? 32 : n_total <= 64 * g ? 64 : 128;
@@ -195,7 +200,7 @@ Plan make_plan(int mode, long long ld, const selscan_launch *L, int n_total = 0,
 struct Layout {
     size_t queue, slotmap, item_status, item_ihh, list2, key2, sorted2, bucket, scratch, total;
     size_t per_warp;
-    size_t sweep_state, sweep_slots, sweep_head, sweep_wscratch;
+    size_t sweep_state, sweep_slots, sweep_head, sweep_wscratch, sweep_words;
 };
 
 Layout make_layout(int n_total, long long m, int mode, int nslots, const SweepPlan *sw = nullptr)
@@ -213,13 +218,17 @@ Layout make_layout(int n_total, long long m, int mode, int nslots, const SweepPl
     l.bucket = o;       o += up256((NBUCKET + 1) * 4);
     l.per_warp = scratch_per_warp(n_total);
     l.scratch = o;      o += (size_t)nslots * l.per_warp;
-    l.sweep_state = l.sweep_slots = l.sweep_head = l.sweep_wscratch = 0;
+    l.sweep_state = l.sweep_slots = l.sweep_head = l.sweep_wscratch = l.sweep_words = 0;
     if (sw && sw->nch > 0) {
         l.sweep_head = o;     o += 256;
         l.sweep_state = o;    o += up256((size_t)2 * sw->nch * sw->state_bytes);
         l.sweep_slots = o;    o += up256((size_t)2 * sw->nch * sw->R * sw->slot_bytes);
         l.sweep_wscratch = o;
-        o += (size_t)sw->walk_ctas * kSplitWarps * sw->wscratch_bytes;
+        o += up256((size_t)sw->walk_ctas * kSplitWarps * sw->wscratch_bytes);
+        // 32-marker words of the cores and their histories (XPEHH: one more row
+        // word when both populations end inside one)
+        l.sweep_words = o;
+        if (sw->started) o += (size_t)((m + 2 * sw->L) / 32 + 2) * ((n_total + 63) / 64 + 1) * 256;
     }
     l.total = o;
     return l;
@@ -337,9 +346,15 @@ int run_scan(int mode, const uint64_t *hap, int64_t ld, int32_t nA, int32_t nB, 
     if ((e = cudaMemsetAsync(err, 0, sizeof(int32_t), s)) != cudaSuccess) return SELSCAN_ERR_CUDA;
     if (launch_validate((const long long *)pos, gmap, m, err, s, !p->use_physical_map) != cudaSuccess)
         return SELSCAN_ERR_CUDA;
-    if (launch_core_select(a, sk.mode, p->maf_num, p->maf_den, p->xpehh_maf_filter, n1, status, s) !=
-        cudaSuccess)
-        return SELSCAN_ERR_CUDA;
+    unsigned *words = (unsigned *)(ws + l.sweep_words);
+    const long long x0 = k0 - plan.sw.L > 0 ? k0 - plan.sw.L : 0;     // markers the sweep's cores
+    const long long x1 = k1 + plan.sw.L < m ? k1 + plan.sw.L : m;     // and histories span
+    if (sweep && plan.sw.started)
+        e = launch_core_select_words(a, sk.mode, p->maf_num, p->maf_den, p->xpehh_maf_filter, n1, status,
+                                     x0, x1, words, s);
+    else
+        e = launch_core_select(a, sk.mode, p->maf_num, p->maf_den, p->xpehh_maf_filter, n1, status, s);
+    if (e != cudaSuccess) return SELSCAN_ERR_CUDA;
     const int ctas_or_slots = plan.schedule == SELSCAN_SCHED_PLAIN ? plan.nslots : plan.ctas;
     if (launch && launch->walk_begin_event &&
         cudaEventRecord((cudaEvent_t)launch->walk_begin_event, s) != cudaSuccess)
@@ -353,6 +368,10 @@ int run_scan(int mode, const uint64_t *hap, int64_t ld, int32_t nA, int32_t nB, 
         w.nch = plan.sw.nch;
         w.B = plan.sw.B;
         w.L = plan.sw.L;
+        w.started = plan.sw.started;
+        w.tw = words;
+        w.tb0 = x0 >> 5;
+        w.tld = 64 * a.W;
         w.R = plan.sw.R;
         w.stage = 0;
         w.nstages = plan.sw.nstages;
@@ -481,7 +500,10 @@ int selscan_sweep_work(int32_t n_total, int64_t m, int32_t mode, const selscan_l
         const long long c1 = c0 + p.sw.B < m ? c0 + p.sw.B : m;
         const long long s0 = c0 - p.sw.L > 0 ? c0 - p.sw.L : 0;
         const long long e0 = c1 - 1 + p.sw.L < m - 1 ? c1 - 1 + p.sw.L : m - 1;
-        passes += (c1 - s0) + (e0 - c0 + 1);       // toward lower / higher indices
+        if (p.sw.started)                          // a history is sorted word by word
+            passes += 2 * (c1 - c0) + (c0 - s0 + 31) / 32 + (e0 - c1 + 32) / 32;
+        else
+            passes += (c1 - s0) + (e0 - c0 + 1);   // toward lower / higher indices
     }
     *marker_passes = passes;
     *elements = (int64_t)sweep_elements(n_total, p.sw.threads);
@@ -493,10 +515,11 @@ int32_t selscan_launch_count(int32_t n_total, int64_t m, int32_t mode, const sel
     if (n_total < 2 || m < 1 || (mode != SELSCAN_MODE_IHS && mode != SELSCAN_MODE_XPEHH)) return -1;
     const Plan p = make_plan(mode, (n_total + 63) / 64, launch, n_total, m);
     switch (p.schedule) {
-    case SELSCAN_SCHED_LONGEST_FIRST: return 8;   // validate, select, probe pass, 3 bucket kernels, pass 2, finalize
+    case SELSCAN_SCHED_LONGEST_FIRST: return 7;   // validate, select, probe pass, 2 bucket kernels, pass 2, finalize
     case SELSCAN_SCHED_IN_ORDER:
     case SELSCAN_SCHED_PLAIN: return 4;           // validate, select, walk, finalize
-    case SELSCAN_SCHED_SWEEP: return 7 + 2 * p.sw.nstages;   // + sweep and split walk per stage
+    // validate, select, starting states, 2 bucket kernels, pass 2, finalize; sweep and split walk per stage
+    case SELSCAN_SCHED_SWEEP: return 6 + p.sw.started + 2 * p.sw.nstages;
     default: return -1;
     }
 }

@@ -83,6 +83,11 @@ cudaError_t launch_validate(const long long *pos, const double *gmap, long long 
                             cudaStream_t s, int check_map = 1);
 cudaError_t launch_core_select(const ScanArgs &a, int mode, unsigned maf_num, unsigned maf_den,
                                int maf_filter, int32_t *n1, int8_t *core_status, cudaStream_t s);
+// core_select, and the rows [x0, x1) as 32-marker words (tw holds the blocks
+// from x0 / 32 on, tld = 64 W words each)
+cudaError_t launch_core_select_words(const ScanArgs &a, int mode, unsigned maf_num, unsigned maf_den,
+                                     int maf_filter, int32_t *n1, int8_t *core_status, long long x0,
+                                     long long x1, unsigned *tw, cudaStream_t s);
 cudaError_t launch_walk(const ScanArgs &a, const ItemSink &sink, const Scratch &sc,
                         int schedule, int warps_per_cta, int ctas, int probe_steps, int fetch,
                         int minb, long long n_items, cudaStream_t s);
@@ -130,7 +135,11 @@ struct SweepArgs {
     int threads;             // threads of one sweep CTA (256 or 512)
     int nch;                 // chunks of cores per direction
     long long B;             // cores per chunk
-    int L;                   // markers swept before a chunk's first core
+    int L;                   // history markers before a chunk's first core
+    int started;             // 1: start_kernel makes the chunks' starting states from tw
+    const unsigned *tw;      // 32-marker words: bit i of word [b - tb0][bit index] = marker 32 b + i
+    long long tb0;           // first 32-marker block in tw
+    int tld;                 // words per block (64 W)
     int R;                   // cores per chunk and stage
     int stage, nstages;
     unsigned short *st;      // per chunk and direction: sorted order, run lengths
@@ -149,7 +158,8 @@ struct SweepArgs {
 size_t sweep_smem_bytes(int n, int W, int T, int R);
 size_t sweep_slot_bytes(int n, int xpehh);
 size_t sweep_state_bytes(int n, int T);
-size_t sweep_elements(int n, int T);     // sorted elements of one CTA (n and its padding)
+__host__ __device__ size_t sweep_elements(int n, int T);     // sorted elements of one CTA (n and its padding)
+size_t start_smem_bytes(int n, int T);   // shared memory of a starting state's sort
 size_t split_smem_per_warp(int n, int xpehh);
 size_t split_scratch_per_warp(int n);
 int split_walk_ctas(int n, int xpehh);

@@ -93,6 +93,88 @@ cudaError_t launch_core_select(const ScanArgs &a, int mode, unsigned maf_num, un
     return cudaGetLastError();
 }
 
+// 32 x 32 bit transpose across a warp: lane l holds row l (bit c = entry (l, c));
+// afterwards lane j holds column j (bit i = entry (i, j)).  Five butterfly stages
+// exchange the off-diagonal blocks of halving size with the partner lane.
+__device__ __forceinline__ unsigned warp_transpose32(unsigned x, int lane)
+{
+    unsigned msk = 0x0000FFFFu;
+#pragma unroll
+    for (int s = 16; s > 0; s >>= 1, msk ^= msk << s) {
+        const unsigned y = __shfl_xor_sync(FULLMASK, x, s);
+        x = (lane & s) ? ((x & ~msk) | ((y >> s) & msk)) : ((x & msk) | ((y << s) & ~msk));
+    }
+    return x;
+}
+
+// core_select fused with the transposition of the rows into 32-marker words
+// (both read every row once): a CTA stages the 32 rows of a block in shared
+// memory (odd row stride: the column reads hit distinct banks), a warp counts
+// whole rows, then takes 64-bit columns, two 32 x 32 bit transposes each.
+// Bound by HBM: a row is read once and written once.
+__global__ void __launch_bounds__(256) core_select_words_kernel(ScanArgs a, int mode, unsigned maf_num,
+                                                                unsigned maf_den, int maf_filter, int32_t *n1,
+                                                                int8_t *core_status, long long x0, long long x1,
+                                                                unsigned *tw)
+{
+    extern __shared__ __align__(16) unsigned long long rows_sm[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int W = a.W, Wp = W | 1;
+    const unsigned n_total = (unsigned)(a.nA + a.nB);
+    const unsigned long long *hap = (const unsigned long long *)a.hap;
+    const long long b = (x0 >> 5) + blockIdx.x;
+    // four rows per warp: all loads of a round before the counts
+    unsigned c[4] = {0u, 0u, 0u, 0u};
+    for (int w = lane; w < W; w += 32) {
+        const unsigned long long vm = (unsigned long long)valid32(a, 2 * w) |
+                                      ((unsigned long long)valid32(a, 2 * w + 1) << 32);
+        unsigned long long v[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const long long k = 32 * b + 4 * warp + r;
+            v[r] = k >= x0 && k < x1 ? __ldg(hap + k * a.ld + w) & vm : 0ull;
+        }
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            rows_sm[(4 * warp + r) * Wp + w] = v[r];
+            c[r] += (unsigned)__popcll(v[r]);
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const unsigned cr = __reduce_add_sync(FULLMASK, c[r]);
+        const long long k = 32 * b + 4 * warp + r;
+        if (lane == 0 && k >= a.k0 && k < a.k1) {
+            n1[k] = (int32_t)cr;
+            const unsigned minor = cr < n_total - cr ? cr : n_total - cr;
+            const bool filt = (mode == 0 || maf_filter) &&
+                              (unsigned long long)maf_den * minor < (unsigned long long)maf_num * n_total;
+            core_status[k] = filt ? (int8_t)SELSCAN_LOCUS_MAF_FILTERED : (int8_t)0;
+        }
+    }
+    __syncthreads();
+    unsigned *dst = tw + (size_t)blockIdx.x * (size_t)(64 * W);
+    for (int w = warp; w < W; w += 8) {
+        const unsigned long long v = rows_sm[lane * Wp + w];
+        dst[64 * w + lane] = warp_transpose32((unsigned)v, lane);
+        dst[64 * w + 32 + lane] = warp_transpose32((unsigned)(v >> 32), lane);
+    }
+}
+
+cudaError_t launch_core_select_words(const ScanArgs &a, int mode, unsigned maf_num, unsigned maf_den,
+                                     int maf_filter, int32_t *n1, int8_t *core_status, long long x0,
+                                     long long x1, unsigned *tw, cudaStream_t s)
+{
+    const size_t smem = (size_t)32 * (a.W | 1) * 8;
+    const cudaError_t e = cudaFuncSetAttribute(core_select_words_kernel,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    const long long blocks = ((x1 - 1) >> 5) - (x0 >> 5) + 1;
+    core_select_words_kernel<<<(unsigned)blocks, 256, smem, s>>>(a, mode, maf_num, maf_den, maf_filter, n1,
+                                                                 core_status, x0, x1, tw);
+    return cudaGetLastError();
+}
+
 // ------------------------------------------------------------ walks
 // Persistent walk kernel.  pass 1: items in core order (a warp takes one
 // core's items per queue fetch), optionally capped at max_steps; pass 2:
@@ -177,28 +259,25 @@ __global__ void __launch_bounds__(128) walk_plain_kernel(ScanArgs a, ItemSink sk
     }
 }
 
-__global__ void bucket_hist_kernel(ItemSink sk)
+// one block: histogram of the queued walks' keys, its exclusive scan (the
+// buckets' first places), and the queue's head reset
+__global__ void __launch_bounds__(1024) bucket_rank_kernel(ItemSink sk)
 {
-    const unsigned long long n2 = sk.q->n2;
-    for (unsigned long long i = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x; i < n2;
-         i += (unsigned long long)gridDim.x * blockDim.x)
-        atomicAdd(sk.bucket + sk.key2[i], 1u);
-}
-
-__global__ void bucket_scan_kernel(ItemSink sk)
-{
-    // one block of NBUCKET threads: exclusive scan in place, head reset
     __shared__ uint32_t t[NBUCKET];
     const int i = threadIdx.x;
-    t[i] = sk.bucket[i];
+    const unsigned long long n2 = sk.q->n2;
+    if (i < NBUCKET) t[i] = 0u;
     __syncthreads();
+    for (unsigned long long k = i; k < n2; k += blockDim.x) atomicAdd(t + sk.key2[k], 1u);
+    __syncthreads();
+    const uint32_t own = i < NBUCKET ? t[i] : 0u;
     for (int o = 1; o < NBUCKET; o <<= 1) {
-        uint32_t v = i >= o ? t[i - o] : 0u;
+        const uint32_t v = i < NBUCKET && i >= o ? t[i - o] : 0u;
         __syncthreads();
-        t[i] += v;
+        if (i < NBUCKET) t[i] += v;
         __syncthreads();
     }
-    sk.bucket[i] = t[i] - sk.bucket[i];
+    if (i < NBUCKET) sk.bucket[i] = t[i] - own;
     if (i == 0) sk.q->head = 0ull;
 }
 
@@ -289,8 +368,7 @@ static cudaError_t persistent_impl(const ScanArgs &a, const ItemSink &sk, const 
                                                                      cap > 0 ? 1 : fetch);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (schedule == SELSCAN_SCHED_LONGEST_FIRST && probe > 0) {
-        bucket_hist_kernel<<<2 * sm_count(), 256, 0, s>>>(sk);
-        bucket_scan_kernel<<<1, NBUCKET, 0, s>>>(sk);
+        bucket_rank_kernel<<<1, 1024, 0, s>>>(sk);
         bucket_scatter_kernel<<<2 * sm_count(), 256, 0, s>>>(sk);
         walk_persistent_kernel<NPOP, MINB><<<ctas, wpc * 32, smem, s>>>(a, sk, sc, n_cores, 2, 0, 1);
     }
@@ -329,8 +407,7 @@ static cudaError_t pass2_impl(const ScanArgs &a, const ItemSink &sk, const Scrat
     e = cudaFuncSetAttribute(walk_persistent_kernel<NPOP, MINB>,
                              cudaFuncAttributePreferredSharedMemoryCarveout, carveout_pct(smem, ctas));
     if (e != cudaSuccess) return e;
-    bucket_hist_kernel<<<2 * sm_count(), 256, 0, s>>>(sk);
-    bucket_scan_kernel<<<1, NBUCKET, 0, s>>>(sk);
+    bucket_rank_kernel<<<1, 1024, 0, s>>>(sk);
     bucket_scatter_kernel<<<2 * sm_count(), 256, 0, s>>>(sk);
     walk_persistent_kernel<NPOP, MINB><<<ctas, wpc * 32, smem, s>>>(a, sk, sc, 0, 2, 0, 1);
     return cudaGetLastError();
@@ -541,20 +618,6 @@ __device__ __forceinline__ void lsb_mask64(const uint4 *v, const uint8_t *p, int
             else b |= bit << (j - 32);
         }
     }
-}
-
-// 32 x 32 bit transpose across a warp: lane l holds row l (bit c = entry (l, c));
-// afterwards lane j holds column j (bit i = entry (i, j)).  Five butterfly stages
-// exchange the off-diagonal blocks of halving size with the partner lane.
-__device__ __forceinline__ unsigned warp_transpose32(unsigned x, int lane)
-{
-    unsigned msk = 0x0000FFFFu;
-#pragma unroll
-    for (int s = 16; s > 0; s >>= 1, msk ^= msk << s) {
-        const unsigned y = __shfl_xor_sync(FULLMASK, x, s);
-        x = (lane & s) ? ((x & ~msk) | ((y >> s) & msk)) : ((x & msk) | ((y << s) & ~msk));
-    }
-    return x;
 }
 
 // haplotype-major input [n, m] bytes, markers [kbeg, m) (the ragged tail of

@@ -19,9 +19,11 @@
 //    marker by marker (a stable partition by allele; the new run length of a
 //    neighbour pair is 1 + the minimum over the old pairs it spans).  At every
 //    core of the stage it writes M, the class boundary n0 (and, for XPEHH, the
-//    population of each sorted position) to a slot.  A chunk starts `warmup`
-//    markers before its first core, so its sort is exact for walks that stay
-//    within that history.
+//    population of each sorted position) to a slot.  A chunk's state at its
+//    first core holds `warmup` markers of history, so its sort is exact for
+//    walks that stay within it: start_kernel sorts the haplotypes by that
+//    history's 32-marker words directly (samples too large for its shared
+//    memory take the history's markers through the sweep instead).
 //  * split_walk_kernel: one warp per slot runs the walks of that core (both
 //    allele classes of iHS, or the pooled XPEHH walk) 32 or 64 steps at a
 //    time, lane l taking step l of the window: S of every step of the window
@@ -127,7 +129,7 @@ size_t sweep_slot_bytes(int n, int xpehh)
 }
 
 size_t sweep_state_bytes(int n, int T) { return (size_t)sweep_npad(n, T) * 4; }
-size_t sweep_elements(int n, int T) { return (size_t)sweep_npad(n, T); }
+__host__ __device__ size_t sweep_elements(int n, int T) { return (size_t)sweep_npad(n, T); }
 
 
 // ---- the sweep ---------------------------------------------------------------
@@ -179,18 +181,18 @@ __global__ void __launch_bounds__(T, T == 512 ? 2 : (T == 256 ? 3 : 512 / T)) sw
     const long long e0 = c1 - 1 + w.L < m - 1 ? c1 - 1 + w.L : m - 1;
     long long xfirst, xlast;                     // markers of this launch, in sweep order
     if (dir == 0) {
-        xfirst = w.stage == 0 ? s0 : klo;
+        xfirst = w.stage == 0 && !w.started ? s0 : klo;
         xlast = khi - 1;
     } else {
-        xfirst = w.stage == 0 ? e0 : khi - 1;
+        xfirst = w.stage == 0 && !w.started ? e0 : khi - 1;
         xlast = klo;
     }
     const long long step = dir == 0 ? 1 : -1;
     unsigned *st = (unsigned *)w.st + (size_t)blockIdx.x * np;
 
     if (blockIdx.x == 0 && tid == 0) *w.walk_head = 0ull;   // the next walk launch's slot counter
-    // ---- state in
-    if (w.stage == 0) {
+    // ---- state in: the identity order, the chunk's starting state, or the last stage's
+    if (w.stage == 0 && !w.started) {
         for (int t = tid; t < np; t += T) P0[t] = t < n ? bit_index(w, t) : pad_bi;
     } else {
         for (int t = tid; t < np; t += T) P0[t] = st[t];
@@ -1012,6 +1014,295 @@ static void (*walk_kernel_for(int xpehh))(SweepArgs)
     return xpehh ? split_walk_kernel<2, G> : split_walk_kernel<1, G>;
 }
 
+// ---- the starting state of a chunk ----------------------------------------------
+// The order and run lengths that the sweep would have after stepping through
+// the history [s0, c0) (toward lower indices; [c1, e0] the other way) from the
+// identity order: the haplotypes sorted by their sequence read from the nearest
+// history marker outward, ties by index, M = the common length of neighbours.
+// A multikey quicksort over the 32-marker words of w.tw, all groups of all
+// levels at once: per round every unresolved group splits three ways, stably,
+// about its middle element's word (the equal part goes on to the next word),
+// by one prefix sum over the CTA; once few are left, only they take part.
+// About 60 rounds replace 1,536 marker passes.
+// Shared memory per haplotype: element (bit index | group start << 16) and
+// group (at its start: end | word level << 16) twice, the prefix sums, and the
+// level at which each boundary arose.
+size_t start_smem_bytes(int n, int T) { return (size_t)n * 22 + 8 + (size_t)(T / 32) * 4; }
+
+namespace {
+
+template <int T>
+__device__ void start_state(const SweepArgs &w, unsigned char *smem, int dir, long long c0, long long c1,
+                            unsigned *st, int np)
+{
+    const int n = w.n, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    unsigned *el = (unsigned *)smem;             // [2][n]
+    unsigned *inf = el + 2 * n;                  // [2][n]
+    unsigned *pre = inf + 2 * n;                 // [n + 1]
+    unsigned *wsum = pre + n + 1;                // [T / 32]
+    unsigned short *bw = (unsigned short *)(wsum + T / 32);   // [n]
+    const long long m = w.a.m;
+    const long long near = dir == 0 ? c0 - 1 : c1;
+    const long long s0 = c0 - w.L > 0 ? c0 - w.L : 0;
+    const long long e0 = c1 - 1 + w.L < m - 1 ? c1 - 1 + w.L : m - 1;
+    const long long far = dir == 0 ? s0 : e0;
+    const int H = (int)(dir == 0 ? c0 - s0 : e0 - c1 + 1);    // history markers
+    const int bn = (int)((near >> 5) - w.tb0), bf = (int)((far >> 5) - w.tb0);   // blocks in tw
+    const int nlev = H == 0 ? 0 : (dir == 0 ? bn - bf : bf - bn) + 1;
+    const unsigned kn = (unsigned)near & 31u, kf = (unsigned)far & 31u;
+    const unsigned mnear = dir == 0 ? 0xFFFFFFFFu >> (31u - kn) : 0xFFFFFFFFu << kn;
+    const unsigned mfar = dir == 0 ? 0xFFFFFFFFu << kf : 0xFFFFFFFFu >> (31u - kf);
+    // word l of haplotype bit index bi, the nearest marker in the top bit
+    auto key = [&](unsigned bi, int l) {
+        unsigned v = __ldg(w.tw + (size_t)(dir == 0 ? bn - l : bn + l) * (size_t)w.tld + bi);
+        if (l == 0) v &= mnear;
+        if (l == nlev - 1) v &= mfar;
+        return dir == 0 ? v : __brev(v);
+    };
+    // exclusive prefix of v over the CTA's threads, and the total (two barriers)
+    unsigned total = 0u;
+    auto block_prefix = [&](unsigned v) {
+        unsigned incl = v;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const unsigned u = __shfl_up_sync(FULLMASK, incl, d);
+            if (lane >= d) incl += u;
+        }
+        __syncthreads();                          // the last totals have been read
+        if (lane == 31) wsum[warp] = incl;
+        __syncthreads();
+        unsigned off = incl - v;
+        total = 0u;
+#pragma unroll
+        for (int q = 0; q < T / 32; ++q) {
+            const unsigned u = wsum[q];
+            off += q < warp ? u : 0u;
+            total += u;
+        }
+        return off;
+    };
+    const int E = ((n + T - 1) / T) | 1;         // odd: a segment's strided reads hit distinct banks
+    const int base = tid * E;
+    constexpr int EC = 4;                        // late rounds: active elements per thread,
+    constexpr int LW = 4;                        // and words compared at once
+    const int few = n <= EC * T ? n : (EC * T < n * 5 / 8 ? EC * T : n * 5 / 8);
+    for (int t = tid; t < n; t += T) el[t] = bit_index(w, t);
+    if (tid == 0) inf[0] = (unsigned)n;
+    __syncthreads();
+    int cur = 0;
+    int na = nlev > 0 && n > 1 ? n : 0;          // elements in unresolved groups
+    while (na > few) {
+        const unsigned *elc = el + cur * n, *ifc = inf + cur * n;
+        // pass 1: this segment's elements below (low half) / equal to (high
+        // half) their group's pivot, counted exclusively into pre
+        unsigned cnt = 0u;
+        for (int e0_ = 0; e0_ < E; e0_ += 4) {
+            unsigned ka[4], kp[4];
+            bool un[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int p = base + e0_ + u;
+                un[u] = false;
+                ka[u] = kp[u] = 0u;
+                if (e0_ + u < E && p < n) {
+                    const unsigned v = elc[p], g = v >> 16, f = ifc[g];
+                    const unsigned end = f & 0xFFFFu;
+                    const int l = (int)(f >> 16);
+                    un[u] = end - g > 1u && l < nlev;
+                    if (un[u]) {
+                        ka[u] = key(v & 0xFFFFu, l);
+                        kp[u] = key(elc[g + ((end - g) >> 1)] & 0xFFFFu, l);
+                    }
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int p = base + e0_ + u;
+                if (e0_ + u < E && p < n) {
+                    pre[p] = cnt;
+                    if (un[u]) cnt += ka[u] < kp[u] ? 1u : (ka[u] == kp[u] ? 0x10000u : 0u);
+                }
+            }
+        }
+        const unsigned off = block_prefix(cnt);
+        for (int e = 0; e < E; ++e)
+            if (base + e < n) pre[base + e] += off;
+        if (tid == 0) pre[n] = total;
+        __syncthreads();
+        // pass 2: place the elements; the first of each part describes its group
+        unsigned *eln = el + (cur ^ 1) * n, *ifn = inf + (cur ^ 1) * n;
+        unsigned left = 0u;
+#pragma unroll 4
+        for (int p = tid; p < n; p += T) {
+            const unsigned v = elc[p], g = v >> 16, f = ifc[g];
+            const unsigned end = f & 0xFFFFu, l = f >> 16;
+            unsigned np_ = (unsigned)p, g2 = g, end2 = end, l2 = l;
+            if (end - g > 1u && (int)l < nlev) {
+                const unsigned pg = pre[g], me = pre[p], d = pre[p + 1] - me;
+                const unsigned tot = pre[end] - pg, mine = me - pg;
+                const unsigned L = tot & 0xFFFFu, Q = tot >> 16, ml = mine & 0xFFFFu, mq = mine >> 16;
+                if (d == 1u) { np_ = g + ml; end2 = g + L; }
+                else if (d != 0u) { g2 = g + L; np_ = g2 + mq; end2 = g2 + Q; l2 = l + 1u; }
+                else { g2 = g + L + Q; np_ = g2 + ((unsigned)p - g - ml - mq); }
+                left += end2 - g2 > 1u && (int)l2 < nlev ? 1u : 0u;
+            }
+            eln[np_] = (v & 0xFFFFu) | (g2 << 16);
+            if (np_ == g2) {
+                ifn[g2] = end2 | (l2 << 16);
+                if (g2 != g) bw[g2] = (unsigned short)l;
+            }
+        }
+        block_prefix(left);
+        na = (int)total;
+        cur ^= 1;
+    }
+    if (na > 0) {
+        // late rounds: the unresolved elements alone, listed in position order
+        // (a group stays contiguous in the list), at most EC per thread; a
+        // round reads them into registers and writes them back in place
+        unsigned *fin = el + cur * n;             // by position: bit index | group start << 16
+        const unsigned *ifc = inf + cur * n;
+        unsigned *ael = el + (cur ^ 1) * n;       // by list index: bit index | list index of the group << 16
+        unsigned *ainf = inf + (cur ^ 1) * n;     // at a group's first index: end | level << 16
+        unsigned short *ap = na < n ? (unsigned short *)(pre + na + 1)     // positions
+                                    : (unsigned short *)(inf + n);
+        if (na < n) {
+            unsigned cnt = 0u;
+            for (int e = 0; e < E; ++e) {
+                const int p = base + e;
+                if (p < n) {
+                    const unsigned g = fin[p] >> 16, f = ifc[g];
+                    cnt += (f & 0xFFFFu) - g > 1u && (int)(f >> 16) < nlev ? 1u : 0u;
+                }
+            }
+            unsigned at = block_prefix(cnt);
+            for (int e = 0; e < E; ++e) {
+                const int p = base + e;
+                if (p < n) {
+                    const unsigned v = fin[p], g = v >> 16, f = ifc[g];
+                    if ((f & 0xFFFFu) - g > 1u && (int)(f >> 16) < nlev) {
+                        const unsigned ag = at - ((unsigned)p - g);
+                        ael[at] = (v & 0xFFFFu) | (ag << 16);
+                        ap[at] = (unsigned short)p;
+                        if ((unsigned)p == g) ainf[ag] = (at + (f & 0xFFFFu) - g) | (f & 0xFFFF0000u);
+                        ++at;
+                    }
+                }
+            }
+        } else {
+            ainf = inf;                           // one group: every haplotype at word 0
+            for (int t = tid; t < n; t += T) {
+                ael[t] = fin[t];
+                ap[t] = (unsigned short)t;
+            }
+        }
+        bool more = true;
+        __syncthreads();
+        while (more) {
+            unsigned v[EC], f[EC], d[EC];
+            unsigned cnt = 0u;
+#pragma unroll
+            for (int u = 0; u < EC; ++u) {
+                const int i = EC * tid + u;
+                f[u] = 0u;                        // resolved (or no element)
+                d[u] = 0u;
+                if (i < na) {
+                    v[u] = ael[i];
+                    const unsigned g = v[u] >> 16;
+                    f[u] = ainf[g];
+                    const unsigned end = f[u] & 0xFFFFu;
+                    const int l = (int)(f[u] >> 16);
+                    if (end - g > 1u && l < nlev) {
+                        const unsigned bi = v[u] & 0xFFFFu, bp = ael[g + ((end - g) >> 1)] & 0xFFFFu;
+                        unsigned ka[LW], kp[LW];
+#pragma unroll
+                        for (int j = 0; j < LW; ++j) ka[j] = l + j < nlev ? key(bi, l + j) : 0u;
+#pragma unroll
+                        for (int j = 0; j < LW; ++j) kp[j] = l + j < nlev ? key(bp, l + j) : 0u;
+                        d[u] = 0x10000u;
+#pragma unroll
+                        for (int j = LW - 1; j >= 0; --j)
+                            d[u] = ka[j] < kp[j] ? 1u : (ka[j] == kp[j] ? d[u] : 0u);
+                    } else {
+                        f[u] = 0u;
+                    }
+                }
+                cnt += d[u];
+            }
+            unsigned me = block_prefix(cnt);
+#pragma unroll
+            for (int u = 0; u < EC; ++u) {
+                if (EC * tid + u < na) pre[EC * tid + u] = me;
+                me += d[u];
+            }
+            // group ends look up pre one past the list's last index too; the
+            // position list follows at pre + na + 1
+            if (tid == 0) pre[na] = total;
+            __syncthreads();
+            bool left = false;
+#pragma unroll
+            for (int u = 0; u < EC; ++u) {
+                if (f[u] == 0u) continue;
+                const unsigned i = (unsigned)(EC * tid + u), g = v[u] >> 16, end = f[u] & 0xFFFFu, l = f[u] >> 16;
+                const unsigned pg = pre[g], tot = pre[end] - pg, mine = pre[i] - pg;
+                const unsigned L = tot & 0xFFFFu, Q = tot >> 16, ml = mine & 0xFFFFu, mq = mine >> 16;
+                unsigned ni, g2 = g, end2, l2 = l;
+                if (d[u] == 1u) { ni = g + ml; end2 = g + L; }
+                else if (d[u] != 0u) { g2 = g + L; ni = g2 + mq; end2 = g2 + Q; l2 = l + LW; }
+                else { g2 = g + L + Q; ni = g2 + (i - g - ml - mq); end2 = end; }
+                left = left || (end2 - g2 > 1u && (int)l2 < nlev);
+                ael[ni] = (v[u] & 0xFFFFu) | (g2 << 16);
+                fin[ap[ni]] = (v[u] & 0xFFFFu) | ((unsigned)ap[g2] << 16);
+                if (ni == g2) {
+                    ainf[g2] = end2 | (l2 << 16);
+                    if (g2 != g) bw[ap[g2]] = (unsigned short)l;
+                }
+            }
+            more = __syncthreads_or(left) != 0;
+        }
+    }
+    // run lengths: neighbours of one group share the whole history, others part
+    // in the word at which their boundary arose
+    const unsigned *elc = el + cur * n;
+    const unsigned pad_bi = 64u * (unsigned)w.a.W;
+    const int off0 = dir == 0 ? 31 - (int)kn : (int)kn;       // bits of word 0 nearer than `near`
+    for (int p = tid; p < np; p += T) {
+        unsigned M = 0u, bi = pad_bi;
+        if (p < n) {
+            const unsigned v = elc[p];
+            bi = v & 0xFFFFu;
+            if (p > 0) {
+                if ((int)(v >> 16) == p) {
+                    int l = bw[p];                // or one of the next LW - 1
+                    unsigned x = key(bi, l) ^ key(elc[p - 1] & 0xFFFFu, l);
+                    while (x == 0u && l + 1 < nlev) {
+                        ++l;
+                        x = key(bi, l) ^ key(elc[p - 1] & 0xFFFFu, l);
+                    }
+                    M = (unsigned)(32 * l - off0 + __clz((int)x));
+                } else {
+                    M = (unsigned)H;
+                }
+            }
+        }
+        st[p] = bi | (M << 16);
+    }
+}
+
+}  // namespace
+
+template <int T>
+__global__ void __launch_bounds__(T) start_kernel(SweepArgs w)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int dir = blockIdx.x / w.nch, c = blockIdx.x % w.nch;
+    const long long c0 = w.a.k0 + (long long)c * w.B;
+    if (c0 >= w.a.k1) return;
+    const long long c1 = c0 + w.B < w.a.k1 ? c0 + w.B : w.a.k1;
+    const int np = (int)sweep_elements(w.n, w.threads);
+    start_state<T>(w, smem, dir, c0, c1, (unsigned *)w.st + (size_t)blockIdx.x * np, np);
+}
+
 int split_walk_ctas(int n, int xpehh)
 {
     // resident CTAs of the persistent walker
@@ -1055,6 +1346,15 @@ cudaError_t launch_sweep_path(const SweepArgs &w0, cudaStream_t s)
     if ((e = cudaFuncSetAttribute(walk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wsm)) !=
         cudaSuccess)
         return e;
+    if (w.started) {
+        // narrow CTAs for small samples: a round is a few elements per thread
+        const int T = w.n <= 512 ? 128 : w.n <= 2048 ? 256 : 512;
+        void (*start)(SweepArgs) = T == 128 ? start_kernel<128> : T == 256 ? start_kernel<256> : start_kernel<512>;
+        const size_t smem = start_smem_bytes(w.n, T);
+        if ((e = cudaFuncSetAttribute(start, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
+            return e;
+        start<<<2 * w.nch, T, smem, s>>>(w);
+    }
     for (int st = 0; st < w.nstages; ++st) {
         w.stage = st;
         sweep<<<2 * w.nch, w.threads, ssm, s>>>(w);
