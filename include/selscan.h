@@ -101,12 +101,18 @@ typedef struct {
 
 /* Scheduling of the walk kernels.  Changes how the work runs, never the
  * results.  A NULL selscan_launch* selects the library defaults: the sorted
- * sweep for iHS / XPEHH scans of at least 131,072 markers and up to 16383
- * haplotypes, else the in-order persistent schedule; 8 warps per CTA and 512
+ * sweep for iHS / XPEHH scans of at least 32,768 + 4 n_total markers and up to
+ * 16383 haplotypes, else the in-order schedule; 8 warps per CTA and 512
  * on-chip group words per warp for the per-step kernels. */
 #define SELSCAN_SCHED_DEFAULT      -1  /* the library's choice (as for a NULL selscan_launch*) */
 #define SELSCAN_SCHED_LONGEST_FIRST 0  /* persistent kernel, probe pass + longest-first queue */
-#define SELSCAN_SCHED_IN_ORDER      1  /* persistent kernel, one queue in core order */
+#define SELSCAN_SCHED_IN_ORDER      1  /* one persistent launch in core order: a whole scan of at
+                                          most 65,000 markers and 6,144 haplotypes sorts and walks
+                                          chunks of cores; other scans, and launches that set a
+                                          field of the per-step kernels (warps_per_cta,
+                                          ctas_per_sm, smem_entries, probe_steps, window_rows,
+                                          cores_per_fetch, min_ctas_per_sm, big_group_entries),
+                                          walk every step from one queue */
 #define SELSCAN_SCHED_PLAIN         2  /* one CTA per core, no persistence, no ordering */
 #define SELSCAN_SCHED_SWEEP         3  /* sorted sweep: per chunk of cores the haplotypes are kept
                                           sorted by their sequence read outward from the core, and

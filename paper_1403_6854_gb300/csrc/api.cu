@@ -48,6 +48,7 @@ struct SweepPlan {
 
 struct Plan {
     int schedule;
+    bool chunked;       // in-order scan done by chunk_scan_kernel (sw holds its chunks)
     SweepPlan sw;
     int wpc;            // warps per CTA of the walk kernel
     int ctas;           // persistent grid size
@@ -126,6 +127,47 @@ SweepPlan make_sweep_plan(int n_total, long long m, int mode, const selscan_laun
     return w;
 }
 
+// A whole in-order scan in one launch of chunk_scan_kernel: any whole scan of
+// at most 65,000 markers (16-bit run lengths span it) and 6,144 haplotypes,
+// while its slots stay within 2 GiB, unless a field that shapes the per-step
+// walk is set.  As many chunks as the GPU holds CTAs at once, of at least 8
+// cores.
+constexpr long long kChunkMaxM = 65000;
+constexpr size_t kChunkSlotBudget = (size_t)2 << 30;
+bool chunk_plan(int n_total, long long m, int mode, const selscan_launch *L, SweepPlan *w)
+{
+    if (n_total < 2 || n_total > kChunkMaxN || m < 1 || m > kChunkMaxM || mode == SELSCAN_MODE_EHH) return false;
+    if (L && (L->warps_per_cta || L->ctas_per_sm || L->smem_entries || L->probe_steps || L->window_rows ||
+              L->cores_per_fetch || L->min_ctas_per_sm || L->big_group_entries))
+        return false;
+    const int xp = mode == SELSCAN_MODE_XPEHH;
+    memset(w, 0, sizeof(*w));
+    w->started = 1;
+    w->L = (int)kChunkMaxM;
+    w->threads = chunk_sort_threads(n_total, m);
+    w->state_bytes = sweep_state_bytes(n_total, w->threads);
+    w->slot_bytes = sweep_slot_bytes(n_total, xp);
+    w->split_bytes = (int)split_smem_per_warp(n_total, xp);
+    w->wscratch_bytes = split_scratch_per_warp(n_total);
+    // shared memory of rows one word wider (the plan does not depend on the
+    // row's split into populations) and of the longest chunk (one CTA per SM)
+    const int maxB = (int)(2 * m / device_sms() + 8);
+    const size_t smem = chunk_smem_bytes(n_total, m, (n_total + 63) / 64 + 1, maxB, xp);
+    if (smem > kMaxSmemPerCta || (w->slot_bytes & 15) || (size_t)2 * m * w->slot_bytes > kChunkSlotBudget)
+        return false;
+    int per_sm = chunk_ctas_per_sm(n_total, m, smem, xp);
+    if (per_sm < 1) per_sm = 1;
+    long long nch = (long long)per_sm * device_sms() / 2;
+    if (nch > (m + 1) / 2) nch = (m + 1) / 2;
+    if (nch < 1) nch = 1;
+    w->B = (m + nch - 1) / nch;
+    w->nch = (int)((m + w->B - 1) / w->B);
+    w->R = (int)w->B;
+    w->nstages = 1;
+    w->walk_ctas = (2 * w->nch * chunk_warps(n_total, m) + kSplitWarps - 1) / kSplitWarps;
+    return true;
+}
+
 // The schedule of a default launch: the sorted sweep once the chromosome is
 // long enough for its chunks' sequential sorts (each about B + warm-up
 // markers, n elements per marker) to cost less than walking every step, the
@@ -144,6 +186,7 @@ int default_schedule(int mode, long long n_total, long long m)
 Plan make_plan(int mode, long long ld, const selscan_launch *L, int n_total = 0, long long m = 0)
 {
     Plan p;
+    p.chunked = false;
     p.schedule = (L && L->schedule != SELSCAN_SCHED_DEFAULT) ? L->schedule
                                                               : default_schedule(mode, n_total, m);
     if (p.schedule < 0 || p.schedule > SELSCAN_SCHED_SWEEP) p.schedule = -1;
@@ -154,6 +197,7 @@ Plan make_plan(int mode, long long ld, const selscan_launch *L, int n_total = 0,
         else
             p.sw = make_sweep_plan(n_total, m, mode, L);
     }
+    if (p.schedule == SELSCAN_SCHED_IN_ORDER) p.chunked = chunk_plan(n_total, m, mode, L, &p.sw);
     p.cap_s = (L && L->smem_entries > 0) ? L->smem_entries : kDefaultSmemEntries;
     if (p.cap_s > 8192) p.cap_s = 8192;
     p.cap_s = (p.cap_s + 31) & ~31;
@@ -198,7 +242,7 @@ Plan make_plan(int mode, long long ld, const selscan_launch *L, int n_total = 0,
 }
 
 struct Layout {
-    size_t queue, slotmap, item_status, item_ihh, list2, key2, sorted2, bucket, scratch, total;
+    size_t queue, slotmap, heads, item_status, item_ihh, list2, key2, sorted2, bucket, scratch, total;
     size_t per_warp;
     size_t sweep_state, sweep_slots, sweep_head, sweep_wscratch, sweep_words;
 };
@@ -210,6 +254,7 @@ Layout make_layout(int n_total, long long m, int mode, int nslots, const SweepPl
     size_t o = 0;
     l.queue = o;        o += up256(sizeof(Queue));
     l.slotmap = o;      o += up256(((size_t)nslots + 31) / 32 * 4);
+    l.heads = o;        o += sw ? up256((size_t)(2 * sw->nch + 128) * 4) : 0;   // read 128 at a time
     l.item_status = o;  o += up256((size_t)items);
     l.item_ihh = o;     o += up256((size_t)items * 8 * (mode == SELSCAN_MODE_XPEHH ? 2 : 1));
     l.list2 = o;        o += up256((size_t)items * 4);
@@ -228,7 +273,7 @@ Layout make_layout(int n_total, long long m, int mode, int nslots, const SweepPl
         // 32-marker words of the cores and their histories (XPEHH: one more row
         // word when both populations end inside one)
         l.sweep_words = o;
-        if (sw->started) o += (size_t)((m + 2 * sw->L) / 32 + 2) * ((n_total + 63) / 64 + 1) * 256;
+        if (sw->started) o += (size_t)((m + 2 * (sw->L < kChunkMaxM ? sw->L : 0)) / 32 + 2) * ((n_total + 63) / 64 + 1) * 256;
     }
     l.total = o;
     return l;
@@ -308,7 +353,8 @@ int run_scan(int mode, const uint64_t *hap, int64_t ld, int32_t nA, int32_t nB, 
                   (size_t)plan.sw.split_bytes * kSplitWarps > kMaxSmemPerCta))
         return SELSCAN_ERR_UNSUPPORTED;
     if (sweep && (plan.sw.slot_bytes & 15)) return SELSCAN_ERR_UNSUPPORTED;   // slots are read in 16-byte units
-    const Layout l = make_layout(n_total, ncores, mode, plan.nslots, sweep ? &plan.sw : nullptr);
+    const Layout l = make_layout(n_total, ncores, mode, plan.nslots, sweep || plan.chunked ? &plan.sw : nullptr);
+    const bool chunked = plan.chunked && k0 == 0 && k1 == m;
     if (!workspace || ws_bytes < l.total || ((uintptr_t)workspace & 255)) return SELSCAN_ERR_WORKSPACE;
     cudaStream_t s = (cudaStream_t)stream;
     unsigned char *ws = (unsigned char *)workspace;
@@ -342,14 +388,13 @@ int run_scan(int mode, const uint64_t *hap, int64_t ld, int32_t nA, int32_t nB, 
 
     cudaError_t e;
     if ((e = cudaMemsetAsync(ws, 0, l.item_status, s)) != cudaSuccess) return SELSCAN_ERR_CUDA;
-    if ((e = cudaMemsetAsync(ws + l.bucket, 0, (NBUCKET + 1) * 4, s)) != cudaSuccess) return SELSCAN_ERR_CUDA;
     if ((e = cudaMemsetAsync(err, 0, sizeof(int32_t), s)) != cudaSuccess) return SELSCAN_ERR_CUDA;
     if (launch_validate((const long long *)pos, gmap, m, err, s, !p->use_physical_map) != cudaSuccess)
         return SELSCAN_ERR_CUDA;
     unsigned *words = (unsigned *)(ws + l.sweep_words);
     const long long x0 = k0 - plan.sw.L > 0 ? k0 - plan.sw.L : 0;     // markers the sweep's cores
     const long long x1 = k1 + plan.sw.L < m ? k1 + plan.sw.L : m;     // and histories span
-    if (sweep && plan.sw.started)
+    if ((sweep || chunked) && plan.sw.started)
         e = launch_core_select_words(a, sk.mode, p->maf_num, p->maf_den, p->xpehh_maf_filter, n1, status,
                                      x0, x1, words, s);
     else
@@ -359,7 +404,7 @@ int run_scan(int mode, const uint64_t *hap, int64_t ld, int32_t nA, int32_t nB, 
     if (launch && launch->walk_begin_event &&
         cudaEventRecord((cudaEvent_t)launch->walk_begin_event, s) != cudaSuccess)
         return SELSCAN_ERR_CUDA;
-    if (sweep) {
+    if (sweep || chunked) {
         SweepArgs w;
         w.a = a;
         w.sk = sk;
@@ -386,8 +431,9 @@ int run_scan(int mode, const uint64_t *hap, int64_t ld, int32_t nA, int32_t nB, 
         w.walk_head = (unsigned long long *)(ws + l.sweep_head);
         w.err = err;
         w.sweep_done_event = launch ? launch->sweep_done_event : nullptr;
-        if (launch_sweep_path(w, s) != cudaSuccess) return SELSCAN_ERR_CUDA;
-        if (launch_pass2(a, sk, sc, plan.wpc, plan.ctas, plan.minb, s) != cudaSuccess)
+        w.heads = (unsigned *)(ws + l.heads);
+        if ((sweep ? launch_sweep_path(w, s) : launch_chunk_scan(w, s)) != cudaSuccess) return SELSCAN_ERR_CUDA;
+        if (sweep && launch_pass2(a, sk, sc, plan.wpc, plan.ctas, plan.minb, s) != cudaSuccess)
             return SELSCAN_ERR_CUDA;
     } else if (launch_walk(a, sk, sc, plan.schedule, plan.wpc, ctas_or_slots, plan.probe, plan.fetch,
                            plan.minb, ncores, s) != cudaSuccess) {
@@ -476,7 +522,7 @@ size_t selscan_workspace_bytes(int32_t n_total, int64_t m, int32_t mode, const s
     const Plan p = make_plan(mode, (n_total + 63) / 64, launch, n_total, m);
     const int nslots = mode == SELSCAN_MODE_EHH ? p.nslots : device_sms() * 64;
     return make_layout(n_total, m, mode, nslots,
-                       p.schedule == SELSCAN_SCHED_SWEEP ? &p.sw : nullptr).total;
+                       p.schedule == SELSCAN_SCHED_SWEEP || p.chunked ? &p.sw : nullptr).total;
 }
 
 int32_t selscan_default_schedule(int32_t n_total, int64_t m, int32_t mode)

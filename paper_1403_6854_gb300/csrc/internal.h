@@ -147,10 +147,12 @@ struct SweepArgs {
     size_t slot_bytes;
     int split_bytes;         // shared memory of one split-walk warp
     int split_tile;          // lanes per split walk (32)
+    int split_off;           // one-launch scans: the walking warps' shared memory starts here
     unsigned char *wscratch; // per split-walk warp: window boundaries past the on-chip list
     size_t wscratch_bytes;
     int walk_ctas;           // persistent split-walk grid
     unsigned long long *walk_head;   // slot counter of the current walk launch
+    unsigned *heads;                 // one-launch scans: next slot of each chunk (0: not sorted yet)
     int32_t *err;                    // device error word of the call
     void *sweep_done_event;          // optional event after the first stage's sort
 };
@@ -164,5 +166,12 @@ size_t split_smem_per_warp(int n, int xpehh);
 size_t split_scratch_per_warp(int n);
 int split_walk_ctas(int n, int xpehh);
 cudaError_t launch_sweep_path(const SweepArgs &w, cudaStream_t s);
+// short scans in one launch (chunk_scan_kernel)
+constexpr int kChunkMaxN = 6144;     // 256 threads x 24 haplotypes
+int chunk_sort_threads(int n, long long m);      // threads that sort a chunk
+int chunk_warps(int n, long long m);             // warps of its CTA
+size_t chunk_smem_bytes(int n, long long m, int W, int R, int xpehh);
+int chunk_ctas_per_sm(int n, long long m, size_t smem, int xpehh);
+cudaError_t launch_chunk_scan(const SweepArgs &w, cudaStream_t s);
 
 }  // namespace selscan

@@ -141,10 +141,12 @@ __host__ __device__ size_t sweep_elements(int n, int T) { return (size_t)sweep_n
 // element's run length.  T threads (32 to 512); EMAX bounds the elements per
 // thread (at most 32, one allele bit each in a 32-bit mask), up to 24 stay in
 // registers between the two passes.
-template <int T, int EMAX, bool EXACT = false>
-__global__ void __launch_bounds__(T, T == 512 ? 2 : (T == 256 ? 3 : 512 / T)) sweep_kernel(SweepArgs w)
+// `sync` is a barrier of the T threads that sort; `done(r)` is called once every
+// thread has written its part of the slots of the stage's first r markers.
+template <int T, int EMAX, bool EXACT, class Sync, class Done>
+__device__ __forceinline__ void sort_chunk(const SweepArgs &w, unsigned char *smem, int dir, int c, Sync sync,
+                                           Done done)
 {
-    extern __shared__ __align__(16) unsigned char smem[];
     constexpr bool CACHE = EMAX <= 24;
     const int n = w.n;
     // EXACT: every thread holds exactly EMAX elements (no per-element guards)
@@ -160,8 +162,7 @@ __global__ void __launch_bounds__(T, T == 512 ? 2 : (T == 256 ? 3 : 512 / T)) sw
     unsigned *wsum = R0 + kRowRing * W32r;
     unsigned *cbits = wsum + 3 * NW;             // the stage's cores that pass the filter
 
-    const int dir = blockIdx.x / w.nch;          // 0: walks toward lower indices
-    const int c = blockIdx.x % w.nch;
+    // dir 0: walks toward lower indices
     const long long m = w.a.m;
     const long long c0 = w.a.k0 + (long long)c * w.B;   // chunk c covers cores [c0, c1) of [k0, k1)
     if (c0 >= w.a.k1) return;
@@ -188,9 +189,8 @@ __global__ void __launch_bounds__(T, T == 512 ? 2 : (T == 256 ? 3 : 512 / T)) sw
         xlast = klo;
     }
     const long long step = dir == 0 ? 1 : -1;
-    unsigned *st = (unsigned *)w.st + (size_t)blockIdx.x * np;
+    unsigned *st = (unsigned *)w.st + (size_t)(dir * w.nch + c) * np;
 
-    if (blockIdx.x == 0 && tid == 0) *w.walk_head = 0ull;   // the next walk launch's slot counter
     // ---- state in: the identity order, the chunk's starting state, or the last stage's
     if (w.stage == 0 && !w.started) {
         for (int t = tid; t < np; t += T) P0[t] = t < n ? bit_index(w, t) : pad_bi;
@@ -223,7 +223,7 @@ __global__ void __launch_bounds__(T, T == 512 ? 2 : (T == 256 ? 3 : 512 / T)) sw
         }
     }
     cp_async_wait<kRowRing - 1>();               // row 0
-    __syncthreads();
+    sync();
 
     int cur = 0;
     const int base = tid * E;
@@ -285,7 +285,8 @@ __global__ void __launch_bounds__(T, T == 512 ? 2 : (T == 256 ? 3 : 512 / T)) sw
         unsigned x2 = __shfl_up_sync(FULLMASK, p2, 1);
         if (lane == 0) { x0 = kIdA; x1 = kIdB; x2 = kIdC; }
         if (lane == 31) { wsum[3 * warp] = p0; wsum[3 * warp + 1] = p1; wsum[3 * warp + 2] = p2; }
-        __syncthreads();
+        sync();
+        if (is_core) done(dir == 0 ? (int)(x - klo) : (int)(khi - 1 - x));
         fetch_row(q + kRowRing);                  // every thread is done with this row's slot
         // every warp scans the warp totals: its own prefix and the block total
         unsigned q0 = lane < NW ? wsum[3 * lane] : kIdA;
@@ -363,7 +364,7 @@ __global__ void __launch_bounds__(T, T == 512 ? 2 : (T == 256 ? 3 : 512 / T)) sw
             }
         }
         cp_async_wait<kRowRing - 1>();           // row q + 1 has landed
-        __syncthreads();
+        sync();
         cur ^= 1;
 
         // ---- a core of this stage: hand its sorted state to the walk
@@ -409,6 +410,14 @@ __global__ void __launch_bounds__(T, T == 512 ? 2 : (T == 256 ? 3 : 512 / T)) sw
         const unsigned *Ps = P0 + cur * np;
         for (int t = tid; t < np; t += T) st[t] = Ps[t];
     }
+}
+
+template <int T, int EMAX, bool EXACT = false>
+__global__ void __launch_bounds__(T, T == 512 ? 2 : (T == 256 ? 3 : 512 / T)) sweep_kernel(SweepArgs w)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    if (blockIdx.x == 0 && threadIdx.x == 0) *w.walk_head = 0ull;   // the next walk launch's slot counter
+    sort_chunk<T, EMAX, EXACT>(w, smem, blockIdx.x / w.nch, blockIdx.x % w.nch, [] { __syncthreads(); }, [](int) {});
 }
 
 // ---- the split walk ----------------------------------------------------------
@@ -499,13 +508,14 @@ __device__ __forceinline__ unsigned count_a(const SplitSmem &s, int x)
 // first step).  Each lane turns 32 neighbouring run lengths into a bitmap word:
 // the 16x2 clamp to [hi, hi + 1] less hi leaves the bit "not yet parted", the
 // slot's layout puts the bits in position order.  `merge` first adds the
-// previous window's boundaries (N) to the older run starts (O).  Returns the
+// previous window's boundaries (N) to the older run starts (O).  Only positions
+// in [pa, pb) are looked at (the classes whose walks still run).  Returns the
 // number of boundaries, K0 of them before position n0; sup gets one bit per
 // summary word of O (at most 17 words: n <= 16383).
 template <int NPOP, typename Tile>
 __device__ __forceinline__ unsigned mark_window(const Tile &tile, const SplitSmem &s, const uint4 *M4,
                                                 int n, int n0, int hi, bool all, bool merge,
-                                                unsigned &K0, unsigned &sup)
+                                                int pa, int pb, unsigned &K0, unsigned &sup)
 {
     const int lane = tile.thread_rank();
     const unsigned short *M16 = (const unsigned short *)M4;
@@ -521,10 +531,10 @@ __device__ __forceinline__ unsigned mark_window(const Tile &tile, const SplitSme
                 o |= s.N[wd];
                 s.O[wd] = o;
             }
-            if (32 * wd < n) {
+            if (32 * wd < pb && 32 * wd + 32 > pa) {
                 uint4 q[4];
 #pragma unroll
-                for (int u = 0; u < 4; ++u) q[u] = __ldg(M4 + 4 * wd + u);
+                for (int u = 0; u < 4; ++u) q[u] = M4[4 * wd + u];
                 unsigned acc = 0u;               // word j's bits land at j and 16 + j
 #pragma unroll
                 for (int u = 3; u >= 0; --u) {
@@ -533,7 +543,8 @@ __device__ __forceinline__ unsigned mark_window(const Tile &tile, const SplitSme
                     acc = acc + acc + (__vmaxu2(__vminu2(q[u].y, PP), P1) - P1);
                     acc = acc + acc + (__vmaxu2(__vminu2(q[u].x, PP), P1) - P1);
                 }
-                hit = ~acc & (n - 32 * wd >= 32 ? 0xFFFFFFFFu : (1u << (n - 32 * wd)) - 1u);
+                hit = ~acc & (pb - 32 * wd >= 32 ? 0xFFFFFFFFu : (1u << (pb - 32 * wd)) - 1u);
+                if (pa > 32 * wd) hit &= 0xFFFFFFFFu << (pa - 32 * wd);
                 s.N[wd] = hit & ~o;
                 if (!all) hit &= ~o;
             }
@@ -555,7 +566,7 @@ __device__ __forceinline__ unsigned mark_window(const Tile &tile, const SplitSme
             const int b = __ffs(hit) - 1;
             hit &= hit - 1u;
             const int t = 32 * wd + b;
-            const unsigned tok = (unsigned)t | ((unsigned)__ldg(M16 + 32 * wd + ((b & 15) << 1 | b >> 4)) << 16);
+            const unsigned tok = (unsigned)t | ((unsigned)M16[32 * wd + ((b & 15) << 1 | b >> 4)] << 16);
             unsigned *dst = at < (unsigned)kTokSmem ? s.tk : s.gtk;
             if (NPOP == 2) *(uint2 *)(dst + 2 * at) = make_uint2(tok, count_a(s, t));
             else dst[at] = tok;
@@ -659,7 +670,7 @@ struct RunCut {
 // population the products of its members on either side.
 template <int NPOP, typename Tile>
 __device__ __forceinline__ void sparse_terms(const Tile &tile, const SplitSmem &s, unsigned K, int lo, int n0,
-                                             unsigned sup, bool act0, bool act1)
+                                             unsigned sup)
 {
     const int lane = tile.thread_rank();
     for (int q = lane; q < kWin * (NPOP == 2 ? 3 : 2); q += 32) s.dec[q] = 0u;
@@ -668,7 +679,6 @@ __device__ __forceinline__ void sparse_terms(const Tile &tile, const SplitSmem &
         const unsigned t = s.tk[NPOP * k];
         const int b = (int)(t & 0xFFFFu);
         const unsigned v = t >> 16;
-        if (NPOP == 1 && !(b < n0 ? act0 : act1)) continue;
         int p = prev_start(s.O, s.S, sup, b), e = next_start(s.O, s.S, sup, b);
         for (int q = (int)k - 1; q >= 0; --q) {
             const unsigned u = s.tk[NPOP * q];
@@ -706,20 +716,271 @@ size_t split_smem_per_warp(int n, int xpehh)
 
 size_t split_scratch_per_warp(int n) { return (((size_t)n * 8) + 255) & ~(size_t)255; }
 
-// Persistent: each warp takes slots of this stage (both directions) from a
-// counter and walks the cores in them.  The first window is the steps 1..32:
+// The walks of one core, by one warp.  The first window is the steps 1..32:
 // every lane runs over all boundaries with M <= 32 (shared memory, broadcast
 // reads) and cuts at those of its own step, so S(i) = (sum of squared run
 // lengths - haplotypes) / 2 of 32 steps costs about six instructions per
 // boundary, where a step at a time needs two bitmap searches, three shared
-// atomics and two warp sums per step with most lanes idle.  Later windows of
-// 64 steps hold few boundaries among many older run starts: there each lane
-// takes one boundary (sparse_terms); a window with more than kSparseMax of
-// them is cut like the first one, 32 steps at a time.
+// atomics and two warp sums per step with most lanes idle (1M iHS: 13.5 -> 8.4
+// ms).  The pooled XPEHH walk, three counts per boundary and few steps long,
+// takes 16 steps at a time, two lanes a step from both ends of the list (1M:
+// 17.2 ms against 24.1 with 32).  Later windows of 64 steps hold few boundaries
+// among many older run starts: there each lane takes one boundary
+// (sparse_terms); a window with more than kSparseMax of them is cut like the
+// first one.
 // Pair counts fit 32 bits (C(16383, 2) < 2^32); the digest is 64-bit.  Lane
 // (i - 1) mod 32 adds step i's trapezoid term to its own FP64 partial sum, and
 // the partial sums meet in a fixed butterfly when the walk ends: the order of
 // the per-step walk, so a walk handed over to it gives the same bits.
+template <int NPOP, typename Tile>
+__device__ __forceinline__ void walk_slot(const SweepArgs &w, const Tile &tile, const SplitSmem &s,
+                                          const unsigned char *slot, long long k, int dir)
+{
+    constexpr int G = 32;
+    constexpr int NV = NPOP == 2 ? 3 : 2;     // S values: class 0, class 1; or A, B, pooled
+    constexpr int NWK = NPOP == 2 ? 1 : 2;    // walks of a slot
+    constexpr int kDense = NPOP == 2 ? 16 : 32;   // steps of a window cut boundary by boundary
+    const int lane = tile.thread_rank();
+    const int n = w.n;
+    const long long m = w.a.m;
+    const int n0 = ((const int *)slot)[0];
+    const int hz = ((const int *)slot)[1];
+    const uint4 *M4 = (const uint4 *)(slot + 16);
+
+    for (int q = lane; q < s.nw; q += G) {   // run starts before step 1: 0, n0, n
+        unsigned o = q == 0 ? 1u : 0u;
+        if (q == n0 >> 5) o |= 1u << (n0 & 31);
+        if (q == n >> 5) o |= 1u << (n & 31);
+        s.O[q] = o;
+        s.N[q] = 0u;
+    }
+    if (NPOP == 2) {
+        const unsigned *isA = (const unsigned *)(slot + slot_isa_at(n));
+        unsigned carry = 0u;
+        for (int base = 0; base < s.nw; base += G) {
+            const int q = base + lane;
+            const unsigned v = q < s.nw ? isA[q] : 0u;
+            const unsigned pc = (unsigned)__popc(v);
+            unsigned incl = pc;
+#pragma unroll
+            for (int d = 1; d < G; d <<= 1) {
+                const unsigned u = tile.shfl_up(incl, d);
+                if (lane >= d) incl += u;
+            }
+            if (q < s.nw) { s.isA[q] = v; s.PA[q] = carry + incl - pc; }
+            carry += tile.shfl(incl, G - 1);
+        }
+    }
+    tile.sync();
+
+    // ---- step 0 (the core marker splits the sample into its allele classes)
+    unsigned S[NV], prev[NV];             // S of this lane's step; S of the step before the block
+    unsigned D[NV];                       // C(N, 2)
+    unsigned long long cutD[NWK];         // a walk stops at the first cut_den S < cut_num D
+    if (NPOP == 2) {
+        const unsigned nA = (unsigned)w.a.nA, nB = (unsigned)w.a.nB;
+        const unsigned a0 = count_a(s, n0), a1 = nA - a0;
+        const unsigned b0 = (unsigned)n0 - a0, b1 = nB - b0;
+        prev[0] = (unsigned)(c2i(a0) + c2i(a1));
+        prev[1] = (unsigned)(c2i(b0) + c2i(b1));
+        prev[NV - 1] = (unsigned)(c2i((unsigned)n0) + c2i((unsigned)(n - n0)));
+        D[0] = (unsigned)c2i(nA);
+        D[1] = (unsigned)c2i(nB);
+        D[NV - 1] = (unsigned)c2i((unsigned)n);
+    } else {
+        prev[0] = D[0] = (unsigned)c2i((unsigned)n0);             // allele 0: positions [0, n0)
+        prev[1] = D[1] = (unsigned)c2i((unsigned)(n - n0));       // allele 1: positions [n0, n)
+    }
+    unsigned long long dig[NV];           // this lane's part of the digests
+    double acc[2] = {0.0, 0.0};           // this lane's partial trapezoid sums
+    bool act[NWK];
+    int stop[NWK];
+    unsigned skey[NWK];                   // S where an unfinished walk left off
+    bool any = false;
+#pragma unroll
+    for (int q = 0; q < NV; ++q) dig[q] = lane == 0 ? prev[q] : 0u;
+#pragma unroll
+    for (int q = 0; q < NWK; ++q) {
+        const unsigned Dq = D[NPOP == 2 ? NV - 1 : q];
+        cutD[q] = (unsigned long long)w.a.cut_num * Dq;
+        stop[q] = 0;
+        skey[q] = 0u;
+        act[q] = Dq != 0u;
+        any |= act[q];
+    }
+    int fin = WALK_OK;                    // how the still-active walks end
+    int endstep = 0;
+    int lo = 1;                           // first step of the window
+    bool dense = true, merge = false;
+    while (any) {
+        unsigned K0, sup;
+        const int hi = lo + (dense ? kDense - 1 : kWin - 1);
+        const int pa = NPOP == 1 && !act[0] ? n0 : 0, pb = NPOP == 1 && !act[NWK - 1] ? n0 : n;
+        const unsigned K = mark_window<NPOP>(tile, s, M4, n, n0, hi, dense, merge, pa, pb, K0, sup);
+        if (!dense && K > (unsigned)kSparseMax) {    // redo as a window of 32 steps
+            dense = true;
+            merge = false;
+            continue;
+        }
+        if (!dense) sparse_terms<NPOP>(tile, s, K, lo, n0, sup);
+        for (int b0 = lo; b0 <= hi; b0 += 32) {
+            // the step of this lane: its map distance g, or how the walk ends
+            // there.  Step i belongs to lane (i - 1) mod 32; the block is the
+            // lanes [la, lb)
+            const int la = (b0 - 1) & 31, i0 = b0 - la, i = i0 + lane;
+            const int lb = la + (hi - b0 + 1 < 32 ? hi - b0 + 1 : 32);
+            const bool mine = lane >= la && lane < lb;
+            double gq = 0.0;
+            int gk = 0;                   // 0 a step, WALK_EDGE past the array end, WALK_GAP a gap abort
+            const long long step = dir ? 1 : -1;
+            const long long xl = k + step * i, xp = xl - step;
+            if (xl < 0 || xl >= m) gk = WALK_EDGE;
+            else {
+                const long long p1 = __ldg(w.a.pos + xl), p0 = __ldg(w.a.pos + xp);
+                const long long bp = dir ? p1 - p0 : p0 - p1;
+                if (bp > w.a.max_gap) gk = WALK_GAP;
+                else {
+                    double gg;
+                    if (w.a.physical) gg = (double)bp;
+                    else {
+                        const double g1 = __ldg(w.a.gmap + xl), g0 = __ldg(w.a.gmap + xp);
+                        gg = dir ? g1 - g0 : g0 - g1;
+                    }
+                    if (bp > w.a.gap_scale) gg = gg * ((double)w.a.gap_scale / (double)bp);
+                    gq = gg;
+                }
+            }
+            // S of this lane's step
+            if (dense) {
+                RunCut<NPOP> rc;
+                if (NPOP == 2) {
+                    // 16 steps, each by two lanes
+                    rc.lim = (unsigned)(i0 + la + (lane & 15) + 1) << 16;   // M <= i  <=>  token < lim
+                    rc.d[0] = rc.d[NPOP == 2 ? 1 : 0] = rc.d[NPOP == 2 ? 2 : 0] = 0u;
+                    rc.both_ends(tile, s, K, (unsigned)n, (unsigned)w.a.nA);
+                    S[0] = (rc.d[NPOP == 2 ? 1 : 0] - (unsigned)w.a.nA) >> 1;
+                    S[1] = (rc.d[NPOP == 2 ? 2 : 0] - (unsigned)w.a.nB) >> 1;
+                    S[NV - 1] = (rc.d[0] - (unsigned)n) >> 1;
+                } else {
+                    rc.lim = (unsigned)(i + 1) << 16;
+                    S[0] = S[1] = 0u;
+                    if (act[0]) {
+                        rc.last = 0u;
+                        rc.d[0] = 0u;
+                        rc.range(s, 0u, K0);
+                        rc.cut((unsigned)n0, 0u);
+                        S[0] = (rc.d[0] - (unsigned)n0) >> 1;
+                    }
+                    if (act[NWK - 1]) {
+                        rc.last = (unsigned)n0;
+                        rc.d[0] = 0u;
+                        rc.range(s, K0, K);
+                        rc.cut((unsigned)n, 0u);
+                        S[1] = (rc.d[0] - (unsigned)(n - n0)) >> 1;
+                    }
+                }
+            } else {
+#pragma unroll
+                for (int q = 0; q < NV; ++q) {
+                    unsigned dd = mine ? s.dec[q * kWin + (i - lo)] : 0u;
+#pragma unroll
+                    for (int d = 1; d < 32; d <<= 1) {
+                        const unsigned v = tile.shfl_up(dd, d);
+                        if (lane >= d) dd += v;
+                    }
+                    S[q] = prev[q] - dd;
+                }
+            }
+            // where the block ends for the walks still running: a gap or the
+            // array end (tested before a step's S), else the history's end
+            const unsigned km = tile.ballot(mine && gk != 0), hm = tile.ballot(mine && i > hz);
+            const int ke = km ? __ffs(km) - 1 : lb, he = hm ? __ffs(hm) - 1 : lb;
+            const int end = ke <= he ? ke : he;
+            const int kfin = tile.shfl(gk, ke & 31);
+            any = false;
+#pragma unroll
+            for (int q = 0; q < NWK; ++q) {
+                if (!act[q]) continue;
+                const int sd = NPOP == 2 ? NV - 1 : q;
+                const unsigned sm = tile.ballot(mine && (unsigned long long)w.a.cut_den * S[sd] < cutD[q]);
+                const int sl = sm ? __ffs(sm) - 1 : lb;
+                const bool stops = sl < end;
+                const int full = stops ? sl : end;       // lanes below: whole steps
+                const bool cnt = lane >= la && lane < full + (stops ? 1 : 0);
+                const bool term = lane >= la && lane < full + (stops && w.a.crossing ? 1 : 0);
+                if (end < lb) skey[q] = end > la ? tile.shfl(S[sd], (end - 1) & 31) : prev[sd];
+#pragma unroll
+                for (int v = NPOP == 2 ? 0 : q; v <= (NPOP == 2 ? NV - 1 : q); ++v) {
+                    unsigned sp = tile.shfl_up(S[v], 1);
+                    if (lane == la) sp = prev[v];
+                    if (cnt) dig[v] += (unsigned long long)(unsigned)(i + 1) * S[v];
+                    if (term && v < 2) acc[v < 2 ? v : 0] += (double)(sp + S[v]) * gq;
+                    prev[v] = tile.shfl(S[v], lb - 1);
+                }
+                if (stops) {
+                    stop[q] = i0 + sl;
+                    act[q] = false;
+                }
+                any |= act[q];
+            }
+            if (!any) break;
+            if (end < lb) {
+                fin = ke <= he ? kfin : WALK_UNFINISHED;
+                endstep = i0 + end;
+                any = false;
+                break;
+            }
+        }
+        lo = hi + 1;
+        dense = (lo & 31) != 1;           // whole blocks of 32 from here on
+        merge = true;
+    }
+    // ---- the lanes' partial sums, then the results (lane 0)
+#pragma unroll
+    for (int q = 0; q < 2; ++q) acc[q] = lane_sum_f64<G>(acc[q]);
+#pragma unroll
+    for (int q = 0; q < NV; ++q) {
+#pragma unroll
+        for (int d = G / 2; d > 0; d >>= 1) dig[q] += __shfl_xor_sync(0xFFFFFFFFu, dig[q], d);
+    }
+    if (lane == 0) {
+        const ItemSink &sk = w.sk;
+#pragma unroll
+        for (int q = 0; q < NWK; ++q) {
+            const unsigned Dq = D[NPOP == 2 ? NV - 1 : q];
+            // iHS items: (allele 1, down), (allele 1, up), (allele 0, down), (allele 0, up)
+            const uint32_t item = NPOP == 2 ? (uint32_t)(k * 2 + dir)
+                                            : (uint32_t)(k * 4 + (q == 1 ? 0 : 2) + dir);
+            int status = Dq == 0u ? WALK_UNDEFINED : WALK_OK;
+            if (act[q]) {
+                if (fin == WALK_UNFINISHED) {
+                    const unsigned long long slot2 = atomicAdd(&sk.q->n2, 1ull);
+                    sk.list2[slot2] = item;
+                    sk.key2[slot2] = bucket_of((float)((double)skey[q] / (double)Dq));
+                    continue;
+                }
+                status = fin;
+                stop[q] = endstep;
+            }
+            sk.item_status[item] = (int8_t)status;
+            sk.stop[item] = stop[q];
+            if (NPOP == 2) {
+                sk.item_ihh[2 * (size_t)item] = D[0] ? acc[0] / (2.0 * (double)D[0]) : 0.0;
+                sk.item_ihh[2 * (size_t)item + 1] = D[1] ? acc[1] / (2.0 * (double)D[1]) : 0.0;
+                sk.digest[3 * (size_t)item] = dig[0];
+                sk.digest[3 * (size_t)item + 1] = dig[1];
+                sk.digest[3 * (size_t)item + 2] = dig[NV - 1];
+            } else {
+                sk.item_ihh[item] = Dq ? acc[q] / (2.0 * (double)Dq) : 0.0;
+                sk.digest[item] = Dq ? dig[q] : 0ull;
+            }
+        }
+    }
+    tile.sync();
+}
+
+// Persistent: each warp takes slots of this stage (both directions) from a
+// counter.
 #ifndef SPLIT_MIN_CTAS
 #define SPLIT_MIN_CTAS 4
 #endif
@@ -730,16 +991,12 @@ __global__ void __launch_bounds__(kSplitWarps * 32, NPOP == 2 ? 3 : SPLIT_MIN_CT
     extern __shared__ __align__(16) unsigned char smem[];
     namespace cg = cooperative_groups;
     const cg::thread_block_tile<G> tile = cg::tiled_partition<G>(cg::this_thread_block());
-    constexpr int NV = NPOP == 2 ? 3 : 2;     // S values: class 0, class 1; or A, B, pooled
-    constexpr int NWK = NPOP == 2 ? 1 : 2;    // walks of a slot
-    constexpr int kDense = NPOP == 2 ? 16 : 32;   // steps of a window cut boundary by boundary
     const int lane = tile.thread_rank(), tix = threadIdx.x / G;
     const int n = w.n;
     const SplitSmem s = split_smem(smem + (size_t)tix * w.split_bytes,
                                    w.wscratch + ((size_t)blockIdx.x * kSplitWarps + tix) * w.wscratch_bytes,
                                    n, NPOP == 2);
     const long long per_dir = (long long)w.nch * w.R;
-    const long long m = w.a.m;
     unsigned long long nxt = 0;               // the slot after this one, fetched ahead
     if (lane == 0) nxt = atomicAdd(w.walk_head, 1ull);
     for (;;) {
@@ -770,241 +1027,7 @@ __global__ void __launch_bounds__(kSplitWarps * 32, NPOP == 2 ? 3 : SPLIT_MIN_CT
         }
         if (w.sk.core_status[k] == (int8_t)SELSCAN_LOCUS_MAF_FILTERED) continue;
 
-        const unsigned char *slot = w.slots + (size_t)gslot * w.slot_bytes;
-        const int n0 = ((const int *)slot)[0];
-        const int hz = ((const int *)slot)[1];
-        const uint4 *M4 = (const uint4 *)(slot + 16);
-
-        for (int q = lane; q < s.nw; q += G) {   // run starts before step 1: 0, n0, n
-            unsigned o = q == 0 ? 1u : 0u;
-            if (q == n0 >> 5) o |= 1u << (n0 & 31);
-            if (q == n >> 5) o |= 1u << (n & 31);
-            s.O[q] = o;
-            s.N[q] = 0u;
-        }
-        if (NPOP == 2) {
-            const unsigned *isA = (const unsigned *)(slot + slot_isa_at(n));
-            unsigned carry = 0u;
-            for (int base = 0; base < s.nw; base += G) {
-                const int q = base + lane;
-                const unsigned v = q < s.nw ? __ldg(isA + q) : 0u;
-                const unsigned pc = (unsigned)__popc(v);
-                unsigned incl = pc;
-#pragma unroll
-                for (int d = 1; d < G; d <<= 1) {
-                    const unsigned u = tile.shfl_up(incl, d);
-                    if (lane >= d) incl += u;
-                }
-                if (q < s.nw) { s.isA[q] = v; s.PA[q] = carry + incl - pc; }
-                carry += tile.shfl(incl, G - 1);
-            }
-        }
-        tile.sync();
-
-        // ---- step 0 (the core marker splits the sample into its allele classes)
-        unsigned S[NV], prev[NV];             // S of this lane's step; S of the step before the block
-        unsigned D[NV], thr[NWK];             // C(N, 2); a walk stops at the first S < thr
-        if (NPOP == 2) {
-            const unsigned nA = (unsigned)w.a.nA, nB = (unsigned)w.a.nB;
-            const unsigned a0 = count_a(s, n0), a1 = nA - a0;
-            const unsigned b0 = (unsigned)n0 - a0, b1 = nB - b0;
-            prev[0] = (unsigned)(c2i(a0) + c2i(a1));
-            prev[1] = (unsigned)(c2i(b0) + c2i(b1));
-            prev[NV - 1] = (unsigned)(c2i((unsigned)n0) + c2i((unsigned)(n - n0)));
-            D[0] = (unsigned)c2i(nA);
-            D[1] = (unsigned)c2i(nB);
-            D[NV - 1] = (unsigned)c2i((unsigned)n);
-        } else {
-            prev[0] = D[0] = (unsigned)c2i((unsigned)n0);             // allele 0: positions [0, n0)
-            prev[1] = D[1] = (unsigned)c2i((unsigned)(n - n0));       // allele 1: positions [n0, n)
-        }
-        unsigned long long dig[NV];           // this lane's part of the digests
-        double acc[2] = {0.0, 0.0};           // this lane's partial trapezoid sums
-        bool act[NWK];
-        int stop[NWK];
-        unsigned skey[NWK];                   // S where an unfinished walk left off
-        bool any = false;
-#pragma unroll
-        for (int q = 0; q < NV; ++q) dig[q] = lane == 0 ? prev[q] : 0u;
-#pragma unroll
-        for (int q = 0; q < NWK; ++q) {
-            const unsigned Dq = D[NPOP == 2 ? NV - 1 : q];
-            const unsigned long long t =
-                ((unsigned long long)w.a.cut_num * Dq + w.a.cut_den - 1u) / w.a.cut_den;
-            thr[q] = t < 0xFFFFFFFFull ? (unsigned)t : 0xFFFFFFFFu;
-            stop[q] = 0;
-            skey[q] = 0u;
-            act[q] = Dq != 0u;
-            any |= act[q];
-        }
-        int fin = WALK_OK;                    // how the still-active walks end
-        int endstep = 0;
-        int lo = 1;                           // first step of the window
-        bool dense = true, merge = false;
-        while (any) {
-            unsigned K0, sup;
-            const int hi = lo + (dense ? kDense - 1 : kWin - 1);
-            const unsigned K = mark_window<NPOP>(tile, s, M4, n, n0, hi, dense, merge, K0, sup);
-            if (!dense && K > (unsigned)kSparseMax) {    // redo as a window of 32 steps
-                dense = true;
-                merge = false;
-                continue;
-            }
-            if (!dense) sparse_terms<NPOP>(tile, s, K, lo, n0, sup, act[0], act[NWK - 1]);
-            for (int b0 = lo; b0 <= hi; b0 += 32) {
-                // the step of this lane: its map distance g, or how the walk ends
-                // there.  Step i belongs to lane (i - 1) mod 32; the block is the
-                // lanes [la, lb)
-                const int la = (b0 - 1) & 31, i0 = b0 - la, i = i0 + lane;
-                const int lb = la + (hi - b0 + 1 < 32 ? hi - b0 + 1 : 32);
-                const bool mine = lane >= la && lane < lb;
-                double gq = 0.0;
-                int gk = 0;                   // 0 a step, WALK_EDGE past the array end, WALK_GAP a gap abort
-                const long long step = dir ? 1 : -1;
-                const long long xl = k + step * i, xp = xl - step;
-                if (xl < 0 || xl >= m) gk = WALK_EDGE;
-                else {
-                    const long long p1 = __ldg(w.a.pos + xl), p0 = __ldg(w.a.pos + xp);
-                    const long long bp = dir ? p1 - p0 : p0 - p1;
-                    if (bp > w.a.max_gap) gk = WALK_GAP;
-                    else {
-                        double gg;
-                        if (w.a.physical) gg = (double)bp;
-                        else {
-                            const double g1 = __ldg(w.a.gmap + xl), g0 = __ldg(w.a.gmap + xp);
-                            gg = dir ? g1 - g0 : g0 - g1;
-                        }
-                        if (bp > w.a.gap_scale) gg = gg * ((double)w.a.gap_scale / (double)bp);
-                        gq = gg;
-                    }
-                }
-                // S of this lane's step
-                if (dense) {
-                    RunCut<NPOP> rc;
-                    if (NPOP == 2) {
-                        // 16 steps, each by two lanes
-                        rc.lim = (unsigned)(i0 + la + (lane & 15) + 1) << 16;   // M <= i  <=>  token < lim
-                        rc.d[0] = rc.d[NPOP == 2 ? 1 : 0] = rc.d[NPOP == 2 ? 2 : 0] = 0u;
-                        rc.both_ends(tile, s, K, (unsigned)n, (unsigned)w.a.nA);
-                        S[0] = (rc.d[NPOP == 2 ? 1 : 0] - (unsigned)w.a.nA) >> 1;
-                        S[1] = (rc.d[NPOP == 2 ? 2 : 0] - (unsigned)w.a.nB) >> 1;
-                        S[NV - 1] = (rc.d[0] - (unsigned)n) >> 1;
-                    } else {
-                        rc.lim = (unsigned)(i + 1) << 16;
-                        S[0] = S[1] = 0u;
-                        if (act[0]) {
-                            rc.last = 0u;
-                            rc.d[0] = 0u;
-                            rc.range(s, 0u, K0);
-                            rc.cut((unsigned)n0, 0u);
-                            S[0] = (rc.d[0] - (unsigned)n0) >> 1;
-                        }
-                        if (act[NWK - 1]) {
-                            rc.last = (unsigned)n0;
-                            rc.d[0] = 0u;
-                            rc.range(s, K0, K);
-                            rc.cut((unsigned)n, 0u);
-                            S[1] = (rc.d[0] - (unsigned)(n - n0)) >> 1;
-                        }
-                    }
-                } else {
-#pragma unroll
-                    for (int q = 0; q < NV; ++q) {
-                        unsigned dd = mine ? s.dec[q * kWin + (i - lo)] : 0u;
-#pragma unroll
-                        for (int d = 1; d < 32; d <<= 1) {
-                            const unsigned v = tile.shfl_up(dd, d);
-                            if (lane >= d) dd += v;
-                        }
-                        S[q] = prev[q] - dd;
-                    }
-                }
-                // where the block ends for the walks still running: a gap or the
-                // array end (tested before a step's S), else the history's end
-                const unsigned km = tile.ballot(mine && gk != 0), hm = tile.ballot(mine && i > hz);
-                const int ke = km ? __ffs(km) - 1 : lb, he = hm ? __ffs(hm) - 1 : lb;
-                const int end = ke <= he ? ke : he;
-                const int kfin = tile.shfl(gk, ke & 31);
-                any = false;
-#pragma unroll
-                for (int q = 0; q < NWK; ++q) {
-                    if (!act[q]) continue;
-                    const int sd = NPOP == 2 ? NV - 1 : q;
-                    const unsigned sm = tile.ballot(mine && S[sd] < thr[q]);
-                    const int sl = sm ? __ffs(sm) - 1 : lb;
-                    const bool stops = sl < end;
-                    const int full = stops ? sl : end;       // lanes below: whole steps
-                    const bool cnt = lane >= la && lane < full + (stops ? 1 : 0);
-                    const bool term = lane >= la && lane < full + (stops && w.a.crossing ? 1 : 0);
-                    if (end < lb) skey[q] = end > la ? tile.shfl(S[sd], (end - 1) & 31) : prev[sd];
-#pragma unroll
-                    for (int v = NPOP == 2 ? 0 : q; v <= (NPOP == 2 ? NV - 1 : q); ++v) {
-                        unsigned sp = tile.shfl_up(S[v], 1);
-                        if (lane == la) sp = prev[v];
-                        if (cnt) dig[v] += (unsigned long long)(unsigned)(i + 1) * S[v];
-                        if (term && v < 2) acc[v < 2 ? v : 0] += (double)(sp + S[v]) * gq;
-                        prev[v] = tile.shfl(S[v], lb - 1);
-                    }
-                    if (stops) {
-                        stop[q] = i0 + sl;
-                        act[q] = false;
-                    }
-                    any |= act[q];
-                }
-                if (!any) break;
-                if (end < lb) {
-                    fin = ke <= he ? kfin : WALK_UNFINISHED;
-                    endstep = i0 + end;
-                    any = false;
-                    break;
-                }
-            }
-            lo = hi + 1;
-            dense = (lo & 31) != 1;           // whole blocks of 32 from here on
-            merge = true;
-        }
-        // ---- the lanes' partial sums, then the results (lane 0)
-#pragma unroll
-        for (int q = 0; q < 2; ++q) acc[q] = lane_sum_f64<G>(acc[q]);
-#pragma unroll
-        for (int q = 0; q < NV; ++q) {
-#pragma unroll
-            for (int d = G / 2; d > 0; d >>= 1) dig[q] += __shfl_xor_sync(0xFFFFFFFFu, dig[q], d);
-        }
-        if (lane == 0) {
-            const ItemSink &sk = w.sk;
-#pragma unroll
-            for (int q = 0; q < NWK; ++q) {
-                const unsigned Dq = D[NPOP == 2 ? NV - 1 : q];
-                // iHS items: (allele 1, down), (allele 1, up), (allele 0, down), (allele 0, up)
-                const uint32_t item = NPOP == 2 ? (uint32_t)(k * 2 + dir)
-                                                : (uint32_t)(k * 4 + (q == 1 ? 0 : 2) + dir);
-                int status = Dq == 0u ? WALK_UNDEFINED : WALK_OK;
-                if (act[q]) {
-                    if (fin == WALK_UNFINISHED) {
-                        const unsigned long long slot2 = atomicAdd(&sk.q->n2, 1ull);
-                        sk.list2[slot2] = item;
-                        sk.key2[slot2] = bucket_of((float)((double)skey[q] / (double)Dq));
-                        continue;
-                    }
-                    status = fin;
-                    stop[q] = endstep;
-                }
-                sk.item_status[item] = (int8_t)status;
-                sk.stop[item] = stop[q];
-                if (NPOP == 2) {
-                    sk.item_ihh[2 * (size_t)item] = D[0] ? acc[0] / (2.0 * (double)D[0]) : 0.0;
-                    sk.item_ihh[2 * (size_t)item + 1] = D[1] ? acc[1] / (2.0 * (double)D[1]) : 0.0;
-                    sk.digest[3 * (size_t)item] = dig[0];
-                    sk.digest[3 * (size_t)item + 1] = dig[1];
-                    sk.digest[3 * (size_t)item + 2] = dig[NV - 1];
-                } else {
-                    sk.item_ihh[item] = Dq ? acc[q] / (2.0 * (double)Dq) : 0.0;
-                    sk.digest[item] = Dq ? dig[q] : 0ull;
-                }
-            }
-        }
-        tile.sync();
+        walk_slot<NPOP>(w, tile, s, w.slots + (size_t)gslot * w.slot_bytes, k, dir);
     }
 }
 
@@ -1301,6 +1324,200 @@ __global__ void __launch_bounds__(T) start_kernel(SweepArgs w)
     const long long c1 = c0 + w.B < w.a.k1 ? c0 + w.B : w.a.k1;
     const int np = (int)sweep_elements(w.n, w.threads);
     start_state<T>(w, smem, dir, c0, c1, (unsigned *)w.st + (size_t)blockIdx.x * np, np);
+}
+
+// ---- a whole short scan in one launch ----------------------------------------------
+// Short chromosomes (the in-order schedule): one CTA per chunk and direction.
+// All of its TC threads make the chunk's starting state (the whole arm as
+// history, so no walk is ever handed on); the first TS then sort the cores one
+// after the other into slots of their own, while the other warps walk each core
+// as soon as its slot is written.  When the sort is done its warps walk too, and
+// warps that run out of work take slots of any chunk whose sort is done.
+// Waits are inside the CTA only (a walking warp for its own sorting warps, with
+// a limit); a chunk that is not ready is left to its owner.
+// w.heads[chunk]: 0 until the chunk's sort is done, then 1 + the next slot.
+// Bound by latency (one chunk's serial chain of rounds, marker passes and walks),
+// so the chromosome is cut into as many chunks as the GPU holds CTAs at once.
+constexpr int kChunkClosed = 1 << 24;        // added to a chunk's own counter when its sort is done
+constexpr int kChunkPolls = 1 << 24;
+
+template <int TS>
+__device__ __forceinline__ void sort_barrier()
+{
+    if (TS == 32) __syncwarp();
+    else asm volatile("bar.sync 1, %0;" ::"n"(TS) : "memory");
+}
+
+template <int TS, int TC, int EMAX, int MINB, int NPOP>
+__global__ void __launch_bounds__(TC, MINB) chunk_scan_kernel(SweepArgs w)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ int own_next;                  // next slot of this chunk while it is being sorted
+    __shared__ volatile int own_ready;        // slots written
+    namespace cg = cooperative_groups;
+    const cg::thread_block_tile<32> tile = cg::tiled_partition<32>(cg::this_thread_block());
+    const int lane = tile.thread_rank(), warp = threadIdx.x >> 5;
+    const int nc = 2 * w.nch;
+    const int me = (int)blockIdx.x;
+    auto chunk = [&](int id, long long &c0, long long &c1) {
+        c0 = w.a.k0 + (long long)(id % w.nch) * w.B;
+        c1 = c0 + w.B < w.a.k1 ? c0 + w.B : w.a.k1;
+        return c0 < c1 ? (int)(c1 - c0) : 0;
+    };
+    const SplitSmem s = split_smem(smem + w.split_off + (size_t)warp * w.split_bytes,
+                                   w.wscratch + ((size_t)me * (TC / 32) + warp) * w.wscratch_bytes,
+                                   w.n, NPOP == 2);
+    auto walk_one = [&](int id, long long c0, long long c1, int r) {
+        const int dir = id / w.nch;
+        const long long k = dir == 0 ? c0 + r : c1 - 1 - r;
+        if (w.sk.core_status[k] == (int8_t)SELSCAN_LOCUS_MAF_FILTERED) return;
+        walk_slot<NPOP>(w, tile, s, w.slots + ((size_t)id * w.R + r) * w.slot_bytes, k, dir);
+    };
+    long long c0, c1;
+    const int cnt = chunk(me, c0, c1);
+    bool own = false;                         // this chunk's remaining slots are this warp's to drain
+    if (cnt > 0) {                            // uniform over the CTA
+        const int np = (int)sweep_elements(w.n, TS);
+        start_state<TC>(w, smem, me / w.nch, c0, c1, (unsigned *)w.st + (size_t)me * np, np);
+        if (threadIdx.x == 0) {
+            own_next = 0;
+            own_ready = 0;
+        }
+        __syncthreads();
+        if (threadIdx.x < TS) {
+            sort_chunk<TS, EMAX, false>(w, smem, me / w.nch, me % w.nch, [] { sort_barrier<TS>(); },
+                                        [&](int r) {
+                                            if (threadIdx.x == 0) {
+                                                __threadfence_block();
+                                                own_ready = r;
+                                            }
+                                        });
+            sort_barrier<TS>();
+            if (threadIdx.x == 0) {
+                __threadfence();              // the slots before the flags
+                own_ready = cnt;
+                const int next = atomicAdd(&own_next, kChunkClosed);
+                atomicExch(w.heads + me, 1u + (unsigned)(next < cnt ? next : cnt));
+            }
+            sort_barrier<TS>();
+            own = true;
+        } else {
+            for (;;) {
+                int r = 0;
+                if (lane == 0) r = atomicAdd(&own_next, 1);
+                r = __shfl_sync(FULLMASK, r, 0);
+                if (r >= cnt) break;
+                int polls = 0;
+                while (own_ready <= r && ++polls < kChunkPolls) __nanosleep(64);
+                if (polls >= kChunkPolls) {
+                    if (lane == 0) atomicExch(w.err, SELSCAN_ERR_TIMEOUT);
+                    break;
+                }
+                __threadfence_block();        // the flag before the slot
+                __syncwarp();
+                walk_one(me, c0, c1, r);
+            }
+        }
+    }
+    // own chunk first, then whatever is ready (128 chunks looked at per step,
+    // heads padded to a multiple of 128), until a full look finds nothing
+    int first = me & ~127;
+    const int span = (nc + 127) & ~127;
+    for (;;) {
+        int id = own ? me : -1;
+        own = false;
+        for (int q = 0; q < span && id < 0; q += 128) {
+            const int at = first + q < span ? first + q : first + q - span;
+            const volatile unsigned *h = w.heads + at + 4 * lane;
+            unsigned avail = 0u;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const unsigned v = h[u];
+                if (v != 0u && v <= (unsigned)w.R) avail |= 1u << u;
+            }
+            const unsigned any = __ballot_sync(FULLMASK, avail != 0u);
+            if (any) {
+                const int l = __ffs(any) - 1;
+                id = at + 4 * l + __ffs((int)__shfl_sync(FULLMASK, avail, l)) - 1;
+                first = at;
+                __threadfence();                  // the flag before the slots
+            }
+        }
+        if (id < 0) break;
+        long long d0, d1;
+        const int dcnt = chunk(id, d0, d1);
+        unsigned nxt = 0u;
+        if (lane == 0) nxt = atomicAdd(w.heads + id, 1u);
+        for (;;) {
+            const int r = (int)__shfl_sync(FULLMASK, nxt, 0) - 1;
+            if (r >= dcnt) break;
+            if (lane == 0) nxt = atomicAdd(w.heads + id, 1u);
+            walk_one(id, d0, d1, r);
+        }
+        // a short last chunk: mark it used up for the scan above
+        if (lane == 0) atomicMax(w.heads + id, (unsigned)w.R + 1u);
+    }
+}
+
+typedef void (*ChunkKernel)(SweepArgs);
+
+// Threads that sort a chunk, threads of its CTA, CTAs per SM.  Chunks of many
+// cores: a narrow sort with walking warps beside it (204 haplotypes x 22,147
+// markers 0.34 ms: one warp of six, four CTAs per SM; all four of four warps
+// sorting, then walking: 0.39).  Chunks of few cores: every warp sorts, then
+// walks (100 x 2,000: 0.127 ms, against 0.185 with one sorting warp of six).
+struct ChunkShape { int ts, tc, ctas; ChunkKernel ihs, xpehh; };
+static ChunkShape chunk_shape(int n, long long m)
+{
+    if (n <= 1024 && m < 16 * 2 * 152)
+        return {128, 128, 5, chunk_scan_kernel<128, 128, 8, 5, 1>, chunk_scan_kernel<128, 128, 8, 5, 2>};
+    if (n <= 256)
+        return {32, 192, 4, chunk_scan_kernel<32, 192, 8, 4, 1>, chunk_scan_kernel<32, 192, 8, 4, 2>};
+    if (n <= 512)
+        return {64, 192, 4, chunk_scan_kernel<64, 192, 8, 4, 1>, chunk_scan_kernel<64, 192, 8, 4, 2>};
+    if (n <= 2048)
+        return {128, 256, 2, chunk_scan_kernel<128, 256, 16, 2, 1>, chunk_scan_kernel<128, 256, 16, 2, 2>};
+    return {256, 320, 2, chunk_scan_kernel<256, 320, 24, 2, 1>, chunk_scan_kernel<256, 320, 24, 2, 2>};
+}
+int chunk_sort_threads(int n, long long m) { return chunk_shape(n, m).ts; }
+int chunk_warps(int n, long long m) { return chunk_shape(n, m).tc / 32; }
+
+// the walking warps' shared memory follows the sort's (they run side by side);
+// the starting state's is gone by then
+static int chunk_split_off(int n, int W, int ts, int R) { return (int)((sweep_smem_bytes(n, W, ts, R) + 15) & ~(size_t)15); }
+size_t chunk_smem_bytes(int n, long long m, int W, int R, int xpehh)
+{
+    const ChunkShape c = chunk_shape(n, m);
+    const size_t a = start_smem_bytes(n, c.tc);
+    const size_t b = (size_t)chunk_split_off(n, W, c.ts, R) + split_smem_per_warp(n, xpehh) * (size_t)(c.tc / 32);
+    return a > b ? a : b;
+}
+
+int chunk_ctas_per_sm(int n, long long m, size_t smem, int xpehh)
+{
+    const ChunkShape c = chunk_shape(n, m);
+    int per_sm = 0;
+    const ChunkKernel k = xpehh ? c.xpehh : c.ihs;
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, c.tc, smem) != cudaSuccess) {
+        cudaGetLastError();
+        return -1;
+    }
+    return per_sm < c.ctas ? per_sm : c.ctas;
+}
+
+cudaError_t launch_chunk_scan(const SweepArgs &w0, cudaStream_t s)
+{
+    SweepArgs w = w0;
+    const int xp = w.a.nB > 0;
+    const ChunkShape c = chunk_shape(w.n, w.a.m);
+    const size_t smem = chunk_smem_bytes(w.n, w.a.m, w.a.W, w.R, xp);
+    w.split_off = chunk_split_off(w.n, w.a.W, c.ts, w.R);
+    const ChunkKernel k = xp ? c.xpehh : c.ihs;
+    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    k<<<2 * w.nch, c.tc, smem, s>>>(w);
+    return cudaGetLastError();
 }
 
 int split_walk_ctas(int n, int xpehh)
