@@ -157,6 +157,26 @@ struct SweepArgs {
     void *sweep_done_event;          // optional event after the first stage's sort
 };
 
+// One tick of batched scans, chunk by chunk: the scans' arguments (slots, state
+// and 32-marker words in the tick's workspace), its core ranges ("units") and
+// how they are cut into tasks, a chunk and direction each.
+struct ChunkTick {
+    SweepArgs w[SELSCAN_BATCH_MAX_SCANS];
+    int boff[SELSCAN_BATCH_MAX_SCANS + 1];      // scan s's 32-marker blocks: [boff[s], boff[s + 1])
+    int nscans, nunits, B;                       // B: cores per chunk
+    unsigned *heads;                             // next slot of each task (0: not sorted yet)
+    short scan[SELSCAN_BATCH_MAX_UNITS];
+    int c0[SELSCAN_BATCH_MAX_UNITS], c1[SELSCAN_BATCH_MAX_UNITS];
+    int first[SELSCAN_BATCH_MAX_UNITS + 1];      // first task of unit u
+    int blk0[SELSCAN_BATCH_MAX_UNITS];           // its first task's place among its scan's slots
+};
+int tick_sort_threads(int max_n);                // threads that sort a chunk
+int tick_warps(int max_n);                       // warps of a task's CTA
+int tick_ctas(int max_n);                        // CTAs per SM
+size_t tick_smem_bytes(int max_n, int n, int W, int R, int xpehh, int *split_off);
+cudaError_t launch_tick_words(const ChunkTick &t, cudaStream_t s);   // kernels.cu
+cudaError_t launch_chunk_tick(const ChunkTick &t, int max_n, size_t smem, cudaStream_t s);
+
 size_t sweep_smem_bytes(int n, int W, int T, int R);
 size_t sweep_slot_bytes(int n, int xpehh);
 size_t sweep_state_bytes(int n, int T);

@@ -144,8 +144,8 @@ __host__ __device__ size_t sweep_elements(int n, int T) { return (size_t)sweep_n
 // `sync` is a barrier of the T threads that sort; `done(r)` is called once every
 // thread has written its part of the slots of the stage's first r markers.
 template <int T, int EMAX, bool EXACT, class Sync, class Done>
-__device__ __forceinline__ void sort_chunk(const SweepArgs &w, unsigned char *smem, int dir, int c, Sync sync,
-                                           Done done)
+__device__ __forceinline__ void sort_chunk(const SweepArgs &w, unsigned char *smem, int dir, long long c0,
+                                           long long c1, int blk, Sync sync, Done done)
 {
     constexpr bool CACHE = EMAX <= 24;
     const int n = w.n;
@@ -162,11 +162,9 @@ __device__ __forceinline__ void sort_chunk(const SweepArgs &w, unsigned char *sm
     unsigned *wsum = R0 + kRowRing * W32r;
     unsigned *cbits = wsum + 3 * NW;             // the stage's cores that pass the filter
 
-    // dir 0: walks toward lower indices
+    // dir 0: walks toward lower indices.  The chunk covers cores [c0, c1); blk is
+    // the index of its state and of its slots
     const long long m = w.a.m;
-    const long long c0 = w.a.k0 + (long long)c * w.B;   // chunk c covers cores [c0, c1) of [k0, k1)
-    if (c0 >= w.a.k1) return;
-    const long long c1 = c0 + w.B < w.a.k1 ? c0 + w.B : w.a.k1;
     long long klo, khi;                          // this stage's cores [klo, khi)
     if (dir == 0) {
         klo = c0 + (long long)w.stage * w.R;
@@ -189,7 +187,7 @@ __device__ __forceinline__ void sort_chunk(const SweepArgs &w, unsigned char *sm
         xlast = klo;
     }
     const long long step = dir == 0 ? 1 : -1;
-    unsigned *st = (unsigned *)w.st + (size_t)(dir * w.nch + c) * np;
+    unsigned *st = (unsigned *)w.st + (size_t)blk * np;
 
     // ---- state in: the identity order, the chunk's starting state, or the last stage's
     if (w.stage == 0 && !w.started) {
@@ -370,7 +368,7 @@ __device__ __forceinline__ void sort_chunk(const SweepArgs &w, unsigned char *sm
         // ---- a core of this stage: hand its sorted state to the walk
         if (wr) {
             const int r = dir == 0 ? (int)(x - klo) : (int)(khi - 1 - x);
-            unsigned char *slot = w.slots + ((size_t)(dir * w.nch + c) * w.R + r) * w.slot_bytes;
+            unsigned char *slot = w.slots + ((size_t)blk * w.R + r) * w.slot_bytes;
             const int xp = w.a.nB > 0;
             if (tid == 0) {
                 int *hdr = (int *)slot;
@@ -417,7 +415,11 @@ __global__ void __launch_bounds__(T, T == 512 ? 2 : (T == 256 ? 3 : 512 / T)) sw
 {
     extern __shared__ __align__(16) unsigned char smem[];
     if (blockIdx.x == 0 && threadIdx.x == 0) *w.walk_head = 0ull;   // the next walk launch's slot counter
-    sort_chunk<T, EMAX, EXACT>(w, smem, blockIdx.x / w.nch, blockIdx.x % w.nch, [] { __syncthreads(); }, [](int) {});
+    const int dir = blockIdx.x / w.nch, c = blockIdx.x % w.nch;
+    const long long c0 = w.a.k0 + (long long)c * w.B;   // chunk c of [k0, k1)
+    if (c0 >= w.a.k1) return;
+    const long long c1 = c0 + w.B < w.a.k1 ? c0 + w.B : w.a.k1;
+    sort_chunk<T, EMAX, EXACT>(w, smem, dir, c0, c1, blockIdx.x, [] { __syncthreads(); }, [](int) {});
 }
 
 // ---- the split walk ----------------------------------------------------------
@@ -714,7 +716,8 @@ size_t split_smem_per_warp(int n, int xpehh)
     return ((size_t)split_words(n, xpehh) * 4 + 15) & ~(size_t)15;
 }
 
-size_t split_scratch_per_warp(int n) { return (((size_t)n * 8) + 255) & ~(size_t)255; }
+// the list holds at most n boundaries, the first kTokSmem of them on chip
+size_t split_scratch_per_warp(int n) { return n <= kTokSmem ? 0 : (((size_t)n * 8) + 255) & ~(size_t)255; }
 
 // The walks of one core, by one warp.  The first window is the steps 1..32:
 // every lane runs over all boundaries with M <= 32 (shared memory, broadcast
@@ -1348,8 +1351,58 @@ __device__ __forceinline__ void sort_barrier()
     else asm volatile("bar.sync 1, %0;" ::"n"(TS) : "memory");
 }
 
-template <int TS, int TC, int EMAX, int MINB, int NPOP>
-__global__ void __launch_bounds__(TC, MINB) chunk_scan_kernel(SweepArgs w)
+// One chunk and direction of one scan.
+struct ChunkTask { const SweepArgs *w; long long c0, c1; int dir, blk, cnt; };
+
+// The chunks of one scan.
+struct ScanChunks {
+    SweepArgs w;
+    __device__ int count() const { return 2 * w.nch; }
+    __device__ int most() const { return w.R; }          // cores of a whole chunk
+    __device__ unsigned *heads() const { return w.heads; }
+    __device__ ChunkTask task(int id) const
+    {
+        ChunkTask t;
+        t.w = &w;
+        t.dir = id / w.nch;
+        t.blk = id;
+        t.c0 = w.a.k0 + (long long)(id % w.nch) * w.B;
+        t.c1 = t.c0 + w.B < w.a.k1 ? t.c0 + w.B : w.a.k1;
+        t.cnt = t.c0 < t.c1 ? (int)(t.c1 - t.c0) : 0;
+        return t;
+    }
+};
+
+// The chunks of a tick's units (ChunkTick): unit u's chunks are the tasks
+// [first[u], first[u + 1]), both directions.
+struct TickChunks {
+    ChunkTick t;
+    __device__ int count() const { return t.first[t.nunits]; }
+    __device__ int most() const { return t.B; }
+    __device__ unsigned *heads() const { return t.heads; }
+    __device__ ChunkTask task(int id) const
+    {
+        int lo = 0, hi = t.nunits - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (t.first[mid] <= id) lo = mid;
+            else hi = mid - 1;
+        }
+        const int local = id - t.first[lo], nch = (t.first[lo + 1] - t.first[lo]) >> 1;
+        ChunkTask r;
+        r.w = t.w + t.scan[lo];
+        r.dir = local >= nch;
+        r.blk = t.blk0[lo] + local;
+        r.c0 = t.c0[lo] + (long long)(local - r.dir * nch) * t.B;
+        r.c1 = r.c0 + t.B < t.c1[lo] ? r.c0 + t.B : t.c1[lo];
+        r.cnt = (int)(r.c1 - r.c0);
+        return r;
+    }
+};
+
+// NPOP 1: iHS scans, 2: XPEHH scans, 0: both kinds.
+template <int TS, int TC, int EMAX, int MINB, int NPOP, class Chunks>
+__global__ void __launch_bounds__(TC, MINB) chunk_scan_kernel(const __grid_constant__ Chunks ch)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int own_next;                  // next slot of this chunk while it is being sorted
@@ -1357,35 +1410,33 @@ __global__ void __launch_bounds__(TC, MINB) chunk_scan_kernel(SweepArgs w)
     namespace cg = cooperative_groups;
     const cg::thread_block_tile<32> tile = cg::tiled_partition<32>(cg::this_thread_block());
     const int lane = tile.thread_rank(), warp = threadIdx.x >> 5;
-    const int nc = 2 * w.nch;
     const int me = (int)blockIdx.x;
-    auto chunk = [&](int id, long long &c0, long long &c1) {
-        c0 = w.a.k0 + (long long)(id % w.nch) * w.B;
-        c1 = c0 + w.B < w.a.k1 ? c0 + w.B : w.a.k1;
-        return c0 < c1 ? (int)(c1 - c0) : 0;
-    };
-    const SplitSmem s = split_smem(smem + w.split_off + (size_t)warp * w.split_bytes,
-                                   w.wscratch + ((size_t)me * (TC / 32) + warp) * w.wscratch_bytes,
-                                   w.n, NPOP == 2);
-    auto walk_one = [&](int id, long long c0, long long c1, int r) {
-        const int dir = id / w.nch;
-        const long long k = dir == 0 ? c0 + r : c1 - 1 - r;
+    unsigned *heads = ch.heads();
+    auto walk_one = [&](const ChunkTask &t, int r) {
+        const SweepArgs &w = *t.w;
+        const long long k = t.dir == 0 ? t.c0 + r : t.c1 - 1 - r;
         if (w.sk.core_status[k] == (int8_t)SELSCAN_LOCUS_MAF_FILTERED) return;
-        walk_slot<NPOP>(w, tile, s, w.slots + ((size_t)id * w.R + r) * w.slot_bytes, k, dir);
+        const unsigned char *slot = w.slots + ((size_t)t.blk * w.R + r) * w.slot_bytes;
+        const bool xp = NPOP == 2 || (NPOP == 0 && w.a.nB > 0);
+        const SplitSmem s = split_smem(smem + w.split_off + (size_t)warp * w.split_bytes,
+                                       w.wscratch + ((size_t)me * (TC / 32) + warp) * w.wscratch_bytes, w.n, xp);
+        if (NPOP != 1 && xp) walk_slot<2>(w, tile, s, slot, k, t.dir);
+        if (NPOP != 2 && !xp) walk_slot<1>(w, tile, s, slot, k, t.dir);
     };
-    long long c0, c1;
-    const int cnt = chunk(me, c0, c1);
+    const ChunkTask mine = ch.task(me);
     bool own = false;                         // this chunk's remaining slots are this warp's to drain
-    if (cnt > 0) {                            // uniform over the CTA
+    if (mine.cnt > 0) {                       // uniform over the CTA
+        const SweepArgs &w = *mine.w;
         const int np = (int)sweep_elements(w.n, TS);
-        start_state<TC>(w, smem, me / w.nch, c0, c1, (unsigned *)w.st + (size_t)me * np, np);
+        start_state<TC>(w, smem, mine.dir, mine.c0, mine.c1, (unsigned *)w.st + (size_t)mine.blk * np, np);
         if (threadIdx.x == 0) {
             own_next = 0;
             own_ready = 0;
         }
         __syncthreads();
         if (threadIdx.x < TS) {
-            sort_chunk<TS, EMAX, false>(w, smem, me / w.nch, me % w.nch, [] { sort_barrier<TS>(); },
+            sort_chunk<TS, EMAX, false>(w, smem, mine.dir, mine.c0, mine.c1, mine.blk,
+                                        [] { sort_barrier<TS>(); },
                                         [&](int r) {
                                             if (threadIdx.x == 0) {
                                                 __threadfence_block();
@@ -1395,9 +1446,9 @@ __global__ void __launch_bounds__(TC, MINB) chunk_scan_kernel(SweepArgs w)
             sort_barrier<TS>();
             if (threadIdx.x == 0) {
                 __threadfence();              // the slots before the flags
-                own_ready = cnt;
+                own_ready = mine.cnt;
                 const int next = atomicAdd(&own_next, kChunkClosed);
-                atomicExch(w.heads + me, 1u + (unsigned)(next < cnt ? next : cnt));
+                atomicExch(heads + me, 1u + (unsigned)(next < mine.cnt ? next : mine.cnt));
             }
             sort_barrier<TS>();
             own = true;
@@ -1406,7 +1457,7 @@ __global__ void __launch_bounds__(TC, MINB) chunk_scan_kernel(SweepArgs w)
                 int r = 0;
                 if (lane == 0) r = atomicAdd(&own_next, 1);
                 r = __shfl_sync(FULLMASK, r, 0);
-                if (r >= cnt) break;
+                if (r >= mine.cnt) break;
                 int polls = 0;
                 while (own_ready <= r && ++polls < kChunkPolls) __nanosleep(64);
                 if (polls >= kChunkPolls) {
@@ -1415,25 +1466,26 @@ __global__ void __launch_bounds__(TC, MINB) chunk_scan_kernel(SweepArgs w)
                 }
                 __threadfence_block();        // the flag before the slot
                 __syncwarp();
-                walk_one(me, c0, c1, r);
+                walk_one(mine, r);
             }
         }
     }
     // own chunk first, then whatever is ready (128 chunks looked at per step,
     // heads padded to a multiple of 128), until a full look finds nothing
     int first = me & ~127;
-    const int span = (nc + 127) & ~127;
+    const int span = (ch.count() + 127) & ~127;
+    const unsigned most = (unsigned)ch.most();
     for (;;) {
         int id = own ? me : -1;
         own = false;
         for (int q = 0; q < span && id < 0; q += 128) {
             const int at = first + q < span ? first + q : first + q - span;
-            const volatile unsigned *h = w.heads + at + 4 * lane;
+            const volatile unsigned *h = heads + at + 4 * lane;
             unsigned avail = 0u;
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 const unsigned v = h[u];
-                if (v != 0u && v <= (unsigned)w.R) avail |= 1u << u;
+                if (v != 0u && v <= most) avail |= 1u << u;
             }
             const unsigned any = __ballot_sync(FULLMASK, avail != 0u);
             if (any) {
@@ -1444,22 +1496,21 @@ __global__ void __launch_bounds__(TC, MINB) chunk_scan_kernel(SweepArgs w)
             }
         }
         if (id < 0) break;
-        long long d0, d1;
-        const int dcnt = chunk(id, d0, d1);
+        const ChunkTask t = ch.task(id);
         unsigned nxt = 0u;
-        if (lane == 0) nxt = atomicAdd(w.heads + id, 1u);
+        if (lane == 0) nxt = atomicAdd(heads + id, 1u);
         for (;;) {
             const int r = (int)__shfl_sync(FULLMASK, nxt, 0) - 1;
-            if (r >= dcnt) break;
-            if (lane == 0) nxt = atomicAdd(w.heads + id, 1u);
-            walk_one(id, d0, d1, r);
+            if (r >= t.cnt) break;
+            if (lane == 0) nxt = atomicAdd(heads + id, 1u);
+            walk_one(t, r);
         }
-        // a short last chunk: mark it used up for the scan above
-        if (lane == 0) atomicMax(w.heads + id, (unsigned)w.R + 1u);
+        // a chunk shorter than the others: mark it used up for the scan above
+        if (lane == 0) atomicMax(heads + id, most + 1u);
     }
 }
 
-typedef void (*ChunkKernel)(SweepArgs);
+typedef void (*ChunkKernel)(ScanChunks);
 
 // Threads that sort a chunk, threads of its CTA, CTAs per SM.  Chunks of many
 // cores: a narrow sort with walking warps beside it (204 haplotypes x 22,147
@@ -1470,14 +1521,14 @@ struct ChunkShape { int ts, tc, ctas; ChunkKernel ihs, xpehh; };
 static ChunkShape chunk_shape(int n, long long m)
 {
     if (n <= 1024 && m < 16 * 2 * 152)
-        return {128, 128, 5, chunk_scan_kernel<128, 128, 8, 5, 1>, chunk_scan_kernel<128, 128, 8, 5, 2>};
+        return {128, 128, 5, chunk_scan_kernel<128, 128, 8, 5, 1, ScanChunks>, chunk_scan_kernel<128, 128, 8, 5, 2, ScanChunks>};
     if (n <= 256)
-        return {32, 192, 4, chunk_scan_kernel<32, 192, 8, 4, 1>, chunk_scan_kernel<32, 192, 8, 4, 2>};
+        return {32, 192, 4, chunk_scan_kernel<32, 192, 8, 4, 1, ScanChunks>, chunk_scan_kernel<32, 192, 8, 4, 2, ScanChunks>};
     if (n <= 512)
-        return {64, 192, 4, chunk_scan_kernel<64, 192, 8, 4, 1>, chunk_scan_kernel<64, 192, 8, 4, 2>};
+        return {64, 192, 4, chunk_scan_kernel<64, 192, 8, 4, 1, ScanChunks>, chunk_scan_kernel<64, 192, 8, 4, 2, ScanChunks>};
     if (n <= 2048)
-        return {128, 256, 2, chunk_scan_kernel<128, 256, 16, 2, 1>, chunk_scan_kernel<128, 256, 16, 2, 2>};
-    return {256, 320, 2, chunk_scan_kernel<256, 320, 24, 2, 1>, chunk_scan_kernel<256, 320, 24, 2, 2>};
+        return {128, 256, 2, chunk_scan_kernel<128, 256, 16, 2, 1, ScanChunks>, chunk_scan_kernel<128, 256, 16, 2, 2, ScanChunks>};
+    return {256, 320, 2, chunk_scan_kernel<256, 320, 24, 2, 1, ScanChunks>, chunk_scan_kernel<256, 320, 24, 2, 2, ScanChunks>};
 }
 int chunk_sort_threads(int n, long long m) { return chunk_shape(n, m).ts; }
 int chunk_warps(int n, long long m) { return chunk_shape(n, m).tc / 32; }
@@ -1508,7 +1559,9 @@ int chunk_ctas_per_sm(int n, long long m, size_t smem, int xpehh)
 
 cudaError_t launch_chunk_scan(const SweepArgs &w0, cudaStream_t s)
 {
-    SweepArgs w = w0;
+    ScanChunks sc;
+    sc.w = w0;
+    SweepArgs &w = sc.w;
     const int xp = w.a.nB > 0;
     const ChunkShape c = chunk_shape(w.n, w.a.m);
     const size_t smem = chunk_smem_bytes(w.n, w.a.m, w.a.W, w.R, xp);
@@ -1516,7 +1569,44 @@ cudaError_t launch_chunk_scan(const SweepArgs &w0, cudaStream_t s)
     const ChunkKernel k = xp ? c.xpehh : c.ihs;
     const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k<<<2 * w.nch, c.tc, smem, s>>>(w);
+    k<<<2 * w.nch, c.tc, smem, s>>>(sc);
+    return cudaGetLastError();
+}
+
+// ---- a tick's core ranges (batched scans) -----------------------------------------
+// Shapes by the largest sample of the tick: a scan's smaller sample sorts on the
+// same threads.
+struct TickShape { int ts, tc, ctas; void (*kernel)(TickChunks); };
+static TickShape tick_shape(int max_n)
+{
+    if (max_n <= 512) return {64, 192, 4, chunk_scan_kernel<64, 192, 8, 4, 0, TickChunks>};
+    if (max_n <= 1024) return {128, 256, 2, chunk_scan_kernel<128, 256, 8, 2, 0, TickChunks>};
+    if (max_n <= 2048) return {128, 320, 2, chunk_scan_kernel<128, 320, 16, 2, 0, TickChunks>};
+    return {256, 320, 2, chunk_scan_kernel<256, 320, 24, 2, 0, TickChunks>};
+}
+int tick_sort_threads(int max_n) { return tick_shape(max_n).ts; }
+int tick_warps(int max_n) { return tick_shape(max_n).tc / 32; }
+int tick_ctas(int max_n) { return tick_shape(max_n).ctas; }
+
+size_t tick_smem_bytes(int max_n, int n, int W, int R, int xpehh, int *split_off)
+{
+    const TickShape c = tick_shape(max_n);
+    *split_off = chunk_split_off(n, W, c.ts, R);
+    const size_t a = start_smem_bytes(n, c.tc);
+    const size_t b = (size_t)*split_off + split_smem_per_warp(n, xpehh) * (size_t)(c.tc / 32);
+    return a > b ? a : b;
+}
+
+cudaError_t launch_chunk_tick(const ChunkTick &t, int max_n, size_t smem, cudaStream_t s)
+{
+    static_assert(sizeof(TickChunks) <= 32000, "tick parameter block too large");
+    const TickShape c = tick_shape(max_n);
+    const cudaError_t e = cudaFuncSetAttribute(c.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    // static: the block is large, and the launch consumes it before this returns
+    static thread_local TickChunks tc;
+    tc.t = t;
+    c.kernel<<<t.first[t.nunits], c.tc, smem, s>>>(tc);
     return cudaGetLastError();
 }
 

@@ -54,3 +54,59 @@ def test_equals_per_step_walk(sg, nA, nB, m):
     a = scan(sg, rows, pos, gmap, nA, nB, sg.make_launch(sg.SCHED_IN_ORDER))
     b = scan(sg, rows, pos, gmap, nA, nB, sg.make_launch(sg.SCHED_IN_ORDER, warps_per_cta=8))
     assert_bitwise_equal(b, a)
+
+
+def batch_scan(sg, rows, pos, gmap, nA, nB):
+    import torch
+    hap, p, g = sg.to_device(rows, pos, gmap)
+    m, mode = hap.shape[0], sg.MODE_XPEHH if nB else sg.MODE_IHS
+    ipc, nd = (2, 6) if nB else (4, 4)
+    e = lambda shape, dt: torch.empty(shape, dtype=dt, device="cuda")
+    t = dict(status=e(m, torch.int8), n1=e(m, torch.int32), ihh_a=e(m, torch.float64), ihh_b=e(m, torch.float64),
+             lnratio=e(m, torch.float64), stop=e((m, ipc), torch.int32), digest=e((m, nd), torch.int64),
+             error=torch.zeros(1, dtype=torch.int32, device="cuda"))
+    raw = e(sg.selscan_batch_item_bytes(m, mode) + 256, torch.uint8)
+    s = sg.selscan_scan()
+    s.mode, s.nA, s.nB, s.m, s.ld, s.params = mode, nA, nB, m, hap.shape[1], sg.selscan_default_params()
+    s.hap, s.pos_bp, s.gmap = hap.data_ptr(), p.data_ptr(), g.data_ptr()
+    s.items = raw.data_ptr() + (-raw.data_ptr()) % 256
+    for f, v in t.items():
+        setattr(s, f, v.data_ptr())
+    return s, t, (hap, p, g, raw)
+
+
+@pytest.mark.parametrize("sizes", [[(30, 0, 900), (200, 250, 1300), (512, 0, 700)],
+                                   [(1000, 0, 800), (40, 33, 2100), (2, 0, 5)],
+                                   [(100, 0, 1500), (900, 800, 600), (1500, 0, 333), (64, 0, 64)],
+                                   [(2300, 0, 400), (77, 0, 1000), (1200, 1300, 350)]])
+def test_ticks_equal_scans_alone(sg, sizes):
+    """Two ticks over uneven core ranges of scans of different samples and both
+    kinds (empty ranges among them): every output bit of the scan alone."""
+    import torch
+    scans, alone = [], []
+    for i, (nA, nB, m) in enumerate(sizes):
+        hap, pos, gmap = synth.tiny_mosaic(nA + nB, m, 77 + i, founders=6, switch=0.02, flip=0.004)
+        parts = [synth.pack(hap[:, :nA])] + ([synth.pack(hap[:, nA:])] if nB else [])
+        rows = np.concatenate(parts, 1)
+        scans.append(batch_scan(sg, rows, pos, gmap, nA, nB))
+        alone.append(scan(sg, rows, pos, gmap, nA, nB, sg.make_launch(sg.SCHED_IN_ORDER, warps_per_cta=8)))
+    max_n, max_ld = max(s.nA + s.nB for s, _, _ in scans), max(s.ld for s, _, _ in scans)
+    nb = sg.selscan_batch_workspace_bytes(max_n, max_ld, len(scans), 256)
+    raw = torch.empty(nb + 256, dtype=torch.uint8, device="cuda")
+    off = (-raw.data_ptr()) % 256
+    units = [[], []]
+    for i, (s, _, _) in enumerate(scans):
+        sg.selscan_batch_prepare(s)
+        cuts = sorted({0, s.m // 7, s.m // 3, s.m // 3 + 1, s.m})
+        for q, (a, b) in enumerate(zip(cuts, cuts[1:])):
+            units[q % 2].append((i, a, b))
+        units[i % 2].append((i, s.m // 2, s.m // 2))
+    for us in units:
+        sg.selscan_batch_run([s for s, _, _ in scans], *zip(*us), max_n, max_ld, raw[off:off + nb])
+    for (s, t, _), ref in zip(scans, alone):
+        sg.selscan_batch_finalize(s)
+        got = to_np(t)
+        assert int(t["error"].item()) == 0
+        a, b = ("ihhA", "ihhB") if s.nB else ("ihh1", "ihh0")
+        ref = {**ref, "ihh_a": ref.pop(a), "ihh_b": ref.pop(b)}
+        assert_bitwise_equal(got, ref)
