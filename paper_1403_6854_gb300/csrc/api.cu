@@ -279,6 +279,32 @@ Layout make_layout(int n_total, long long m, int mode, int nslots, const SweepPl
     return l;
 }
 
+// Workspace of a single-locus report after the per-step walks' scratch: the
+// locus' 32-marker words, both directions' states and slots, the counts.
+struct ReportLayout {
+    bool on;
+    int threads;
+    size_t words, state, slots, scratch, S, ctl, total;
+};
+ReportLayout report_layout(int n, size_t from)
+{
+    ReportLayout l;
+    memset(&l, 0, sizeof(l));
+    l.total = from;
+    l.on = start_smem_bytes(n, 512) <= kMaxSmemPerCta;
+    if (!l.on) return l;
+    l.threads = n <= 1024 ? 128 : n <= 6144 ? 256 : 512;
+    size_t o = up256(from);
+    l.words = o;   o += (size_t)(2 * kReportSteps / 32 + 2) * ((n + 63) / 64) * 256;
+    l.state = o;   o += up256(2 * sweep_state_bytes(n, l.threads));
+    l.slots = o;   o += up256(2 * sweep_slot_bytes(n, 0));
+    l.scratch = o; o += up256((size_t)2 * (kReportSteps / 32) * split_scratch_per_warp(n));
+    l.S = o;       o += up256((size_t)4 * kReportSteps * 4);
+    l.ctl = o;     o += 256;             // counters and flags, zeroed
+    l.total = o;
+    return l;
+}
+
 inline unsigned long long last_mask(int n)
 {
     return (n % 64) ? ((1ull << (n % 64)) - 1ull) : ~0ull;
@@ -477,19 +503,61 @@ int ehh_prepare(const uint64_t *hap, int64_t ld, int32_t n, int64_t m, const int
     sc->base = nullptr;
     sc->err = out->error;
     *scratch_off = l.scratch;
-    *ws_need = l.total;
+    *ws_need = report_layout(n, l.total).total;
     return SELSCAN_OK;
 }
 
 int ehh_run(const ScanArgs &a, int64_t locus, const selscan_params *p, const Scratch &sc,
-            const selscan_ehh_out *out, int64_t capacity, void *stream)
+            const selscan_ehh_out *out, int64_t capacity, unsigned char *ws, void *stream)
 {
     cudaStream_t s = (cudaStream_t)stream;
     if (cudaMemsetAsync(out->error, 0, sizeof(int32_t), s) != cudaSuccess) return SELSCAN_ERR_CUDA;
     if (launch_validate(a.pos, a.gmap, a.m, out->error, s, !p->use_physical_map) != cudaSuccess)
         return SELSCAN_ERR_CUDA;
+    const int *rest = nullptr;
+    const ReportLayout l = report_layout(a.nA, make_layout(a.nA, a.m, SELSCAN_MODE_EHH, 6).total);
+    if (ws && l.on) {
+        ReportArgs r;
+        memset(&r, 0, sizeof(r));
+        SweepArgs &w = r.w;
+        w.a = a;
+        w.a.k0 = locus;
+        w.a.k1 = locus + 1;
+        w.n = a.nA;
+        w.threads = l.threads;
+        w.nch = 1;
+        w.B = w.R = 1;
+        w.nstages = 1;
+        w.L = kReportSteps;
+        w.started = 1;
+        w.tw = (unsigned *)(ws + l.words);
+        const long long x0 = locus - w.L > 0 ? locus - w.L : 0, x1 = locus + 1 + w.L < a.m ? locus + 1 + w.L : a.m;
+        w.tb0 = x0 >> 5;
+        w.tld = 64 * a.W;
+        w.st = (unsigned short *)(ws + l.state);
+        w.slots = ws + l.slots;
+        w.slot_bytes = sweep_slot_bytes(w.n, 0);
+        w.split_bytes = (int)split_smem_per_warp(w.n, 0);
+        w.wscratch = ws + l.scratch;
+        w.wscratch_bytes = split_scratch_per_warp(w.n);
+        w.walk_head = (unsigned long long *)(ws + l.ctl);            // not used: no walk kernel takes slots
+        w.sk.core_status = at_core((int8_t *)(ws + l.ctl + 128), locus);   // 0: the locus is walked
+        w.err = out->error;
+        r.out = *out;
+        r.capacity = capacity;
+        r.S = (unsigned *)(ws + l.S);
+        r.done = (unsigned *)(ws + l.ctl + 8);
+        r.rest = (int *)(ws + l.ctl + 16);
+        rest = r.rest;
+        // the words of the locus' surroundings (its count and status go to the control block)
+        if (cudaMemsetAsync(ws + l.ctl, 0, 256, s) != cudaSuccess ||
+            launch_core_select_words(w.a, 0, 0, 1, 0, at_core((int32_t *)(ws + l.ctl + 192), locus),
+                                     w.sk.core_status, x0, x1, (unsigned *)(ws + l.words), s) != cudaSuccess ||
+            launch_report(r, s) != cudaSuccess)
+            return SELSCAN_ERR_CUDA;
+    }
     if (launch_ehh(a, locus, sc, (unsigned long long *)out->S, capacity, (long long *)out->len,
-                   out->stop, out->status, out->ihh, (unsigned long long *)out->denom, s) !=
+                   out->stop, out->status, out->ihh, (unsigned long long *)out->denom, rest, s) !=
         cudaSuccess)
         return SELSCAN_ERR_CUDA;
     return SELSCAN_OK;
@@ -521,8 +589,9 @@ size_t selscan_workspace_bytes(int32_t n_total, int64_t m, int32_t mode, const s
     // not depend on the row stride, registers or shared memory of the call
     const Plan p = make_plan(mode, (n_total + 63) / 64, launch, n_total, m);
     const int nslots = mode == SELSCAN_MODE_EHH ? p.nslots : device_sms() * 64;
-    return make_layout(n_total, m, mode, nslots,
-                       p.schedule == SELSCAN_SCHED_SWEEP || p.chunked ? &p.sw : nullptr).total;
+    const size_t total = make_layout(n_total, m, mode, nslots,
+                                     p.schedule == SELSCAN_SCHED_SWEEP || p.chunked ? &p.sw : nullptr).total;
+    return mode == SELSCAN_MODE_EHH ? report_layout(n_total, total).total : total;
 }
 
 int32_t selscan_default_schedule(int32_t n_total, int64_t m, int32_t mode)
@@ -635,7 +704,7 @@ int selscan_ehh(const uint64_t *hap, int64_t ld, int32_t n, int64_t m, const int
     if (rc != SELSCAN_OK) return rc;
     if (!workspace || ws_bytes < need || ((uintptr_t)workspace & 255)) return SELSCAN_ERR_WORKSPACE;
     sc.base = (unsigned char *)workspace + scratch_off;
-    return ehh_run(a, locus, p, sc, out, capacity, stream);
+    return ehh_run(a, locus, p, sc, out, capacity, (unsigned char *)workspace, stream);
 }
 
 int selscan_pack(const uint8_t *hap01, int32_t n, int64_t m, int32_t hap_major, uint64_t *rows,

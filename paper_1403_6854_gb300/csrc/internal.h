@@ -96,9 +96,11 @@ cudaError_t launch_finalize_ihs(const ItemSink &sink, long long k0, long long k1
                                 double *ihh0, double *lnratio, int8_t *status, cudaStream_t s);
 cudaError_t launch_finalize_xpehh(const ItemSink &sink, long long k0, long long k1, double *ihhA,
                                   double *ihhB, double *lnratio, int8_t *status, cudaStream_t s);
+// rest (may be null): only the walks q with rest[q] != 0
 cudaError_t launch_ehh(const ScanArgs &a, long long locus, const Scratch &sc,
                        unsigned long long *S, long long cap, long long *len, int32_t *stop,
-                       int8_t *status, double *ihh, unsigned long long *denom, cudaStream_t s);
+                       int8_t *status, double *ihh, unsigned long long *denom, const int *rest,
+                       cudaStream_t s);
 cudaError_t launch_pack(const uint8_t *hap01, int n, long long m, int hap_major,
                         unsigned long long *rows, long long ld, cudaStream_t s);
 int max_ctas_per_sm(int schedule, int warps_per_cta, size_t smem_bytes, int minb);
@@ -121,8 +123,9 @@ int ehh_prepare(const uint64_t *hap, int64_t ld, int32_t n, int64_t m, const int
                 const selscan_ehh_out *out, int64_t capacity, int32_t max_n, ScanArgs *a,
                 Scratch *sc, size_t *scratch_off, size_t *ws_need);
 // Clears the error word, validates positions / map and launches the report.
+// ws (may be null): a report workspace (ehh_workspace), for the sorted form.
 int ehh_run(const ScanArgs &a, int64_t locus, const selscan_params *p, const Scratch &sc,
-            const selscan_ehh_out *out, int64_t capacity, void *stream);
+            const selscan_ehh_out *out, int64_t capacity, unsigned char *ws, void *stream);
 
 // ---- sorted-sweep walks (sweep.cu)
 constexpr int kSplitWarps = 8;       // warps of one split-walk CTA
@@ -186,6 +189,17 @@ size_t split_smem_per_warp(int n, int xpehh);
 size_t split_scratch_per_warp(int n);
 int split_walk_ctas(int n, int xpehh);
 cudaError_t launch_sweep_path(const SweepArgs &w, cudaStream_t s);
+// the single-locus report from the sorted state (report_kernel)
+constexpr int kReportSteps = 2048;   // steps per direction, a multiple of 32 x kSplitWarps
+struct ReportArgs {
+    SweepArgs w;                     // one core, the locus; its words, state and slots
+    selscan_ehh_out out;
+    long long capacity;
+    unsigned *S;                     // [2 directions][class 0, 1][kReportSteps]: S of steps 1 ..
+    unsigned *done;                  // zero
+    int *rest;                       // [6] 1: the walk outlived the history
+};
+cudaError_t launch_report(const ReportArgs &r, cudaStream_t s);
 // short scans in one launch (chunk_scan_kernel)
 constexpr int kChunkMaxN = 6144;     // 256 threads x 24 haplotypes
 int chunk_sort_threads(int n, long long m);      // threads that sort a chunk

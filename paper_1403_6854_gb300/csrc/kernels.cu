@@ -550,11 +550,12 @@ __global__ void __launch_bounds__(192) ehh_trace_kernel(ScanArgs a, long long lo
                                                         unsigned long long *S, long long cap,
                                                         long long *len, int32_t *stop,
                                                         int8_t *status, double *ihh,
-                                                        unsigned long long *denom)
+                                                        unsigned long long *denom, const int *rest)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31;
     const int q = threadIdx.x >> 5;           // walk w = q / 2, direction q % 2
+    if (rest && rest[q] == 0) return;         // done from the sorted state (warps do not meet)
     WarpBufs b = make_bufs(smem + (size_t)q * slice_bytes(sc),
                            sc.base + (size_t)q * sc.per_warp, sc);
     init_window(b);
@@ -584,13 +585,14 @@ __global__ void __launch_bounds__(192) ehh_trace_kernel(ScanArgs a, long long lo
 
 cudaError_t launch_ehh(const ScanArgs &a, long long locus, const Scratch &sc,
                        unsigned long long *S, long long cap, long long *len, int32_t *stop,
-                       int8_t *status, double *ihh, unsigned long long *denom, cudaStream_t s)
+                       int8_t *status, double *ihh, unsigned long long *denom, const int *rest,
+                       cudaStream_t s)
 {
     const size_t smem = slice_bytes(sc) * 6;
     cudaError_t e = cudaFuncSetAttribute(ehh_trace_kernel,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    ehh_trace_kernel<<<1, 192, smem, s>>>(a, locus, sc, S, cap, len, stop, status, ihh, denom);
+    ehh_trace_kernel<<<1, 192, smem, s>>>(a, locus, sc, S, cap, len, stop, status, ihh, denom, rest);
     return cudaGetLastError();
 }
 

@@ -109,5 +109,5 @@ extern "C" int selscan_ehh_noalloc(const uint64_t *hap, int64_t ld, int32_t n, i
     void *base = nullptr;
     if ((rc = scratch_address(&base)) != SELSCAN_OK) return rc;
     sc.base = (unsigned char *)base;
-    return ehh_run(a, locus, p, sc, out, capacity, stream);
+    return ehh_run(a, locus, p, sc, out, capacity, nullptr, stream);
 }

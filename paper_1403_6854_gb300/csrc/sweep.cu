@@ -1625,27 +1625,43 @@ int split_walk_ctas(int n, int xpehh)
     return per_sm * (sms > 0 ? sms : 1);
 }
 
+// The sorting kernel of a sample and CTA width.
+static void (*sort_kernel(int n, int threads))(SweepArgs)
+{
+    const int E = sweep_e(n, threads);
+    if (threads == 256)
+        return E == 4 ? sweep_kernel<256, 4, true> : E == 8 ? sweep_kernel<256, 8, true>
+             : E == 12 ? sweep_kernel<256, 12, true> : E == 16 ? sweep_kernel<256, 16, true>
+             : E == 20 ? sweep_kernel<256, 20, true> : E == 24 ? sweep_kernel<256, 24, true>
+             : sweep_kernel<256, 32>;
+    if (threads == 512)
+        return E <= 4 ? sweep_kernel<512, 4> : E <= 8 ? sweep_kernel<512, 8>
+             : E <= 16 ? sweep_kernel<512, 16> : E <= 24 ? sweep_kernel<512, 24>
+             : sweep_kernel<512, 32>;
+    if (threads == 128)
+        return E <= 8 ? sweep_kernel<128, 8> : E <= 16 ? sweep_kernel<128, 16> : sweep_kernel<128, 32>;
+    if (threads == 64)
+        return E <= 8 ? sweep_kernel<64, 8> : E <= 16 ? sweep_kernel<64, 16> : sweep_kernel<64, 32>;
+    return E <= 8 ? sweep_kernel<32, 8> : E <= 16 ? sweep_kernel<32, 16> : sweep_kernel<32, 32>;
+}
+
+static cudaError_t launch_start(const SweepArgs &w, cudaStream_t s)
+{
+    // narrow CTAs for small samples: a round is a few elements per thread
+    const int T = w.n <= 512 ? 128 : w.n <= 2048 ? 256 : 512;
+    void (*start)(SweepArgs) = T == 128 ? start_kernel<128> : T == 256 ? start_kernel<256> : start_kernel<512>;
+    const size_t smem = start_smem_bytes(w.n, T);
+    const cudaError_t e = cudaFuncSetAttribute(start, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    start<<<2 * w.nch, T, smem, s>>>(w);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_sweep_path(const SweepArgs &w0, cudaStream_t s)
 {
     SweepArgs w = w0;
     const size_t ssm = sweep_smem_bytes(w.n, w.a.W, w.threads, w.R);
-    const int E = sweep_e(w.n, w.threads);
-    void (*sweep)(SweepArgs);
-    if (w.threads == 256)
-        sweep = E == 4 ? sweep_kernel<256, 4, true> : E == 8 ? sweep_kernel<256, 8, true>
-              : E == 12 ? sweep_kernel<256, 12, true> : E == 16 ? sweep_kernel<256, 16, true>
-              : E == 20 ? sweep_kernel<256, 20, true> : E == 24 ? sweep_kernel<256, 24, true>
-              : sweep_kernel<256, 32>;
-    else if (w.threads == 512)
-        sweep = E <= 4 ? sweep_kernel<512, 4> : E <= 8 ? sweep_kernel<512, 8>
-              : E <= 16 ? sweep_kernel<512, 16> : E <= 24 ? sweep_kernel<512, 24>
-              : sweep_kernel<512, 32>;
-    else if (w.threads == 128)
-        sweep = E <= 8 ? sweep_kernel<128, 8> : E <= 16 ? sweep_kernel<128, 16> : sweep_kernel<128, 32>;
-    else if (w.threads == 64)
-        sweep = E <= 8 ? sweep_kernel<64, 8> : E <= 16 ? sweep_kernel<64, 16> : sweep_kernel<64, 32>;
-    else
-        sweep = E <= 8 ? sweep_kernel<32, 8> : E <= 16 ? sweep_kernel<32, 16> : sweep_kernel<32, 32>;
+    void (*sweep)(SweepArgs) = sort_kernel(w.n, w.threads);
     cudaError_t e = cudaFuncSetAttribute(sweep, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssm);
     if (e != cudaSuccess) return e;
     const size_t wsm = (size_t)w.split_bytes * kSplitWarps;
@@ -1653,15 +1669,7 @@ cudaError_t launch_sweep_path(const SweepArgs &w0, cudaStream_t s)
     if ((e = cudaFuncSetAttribute(walk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wsm)) !=
         cudaSuccess)
         return e;
-    if (w.started) {
-        // narrow CTAs for small samples: a round is a few elements per thread
-        const int T = w.n <= 512 ? 128 : w.n <= 2048 ? 256 : 512;
-        void (*start)(SweepArgs) = T == 128 ? start_kernel<128> : T == 256 ? start_kernel<256> : start_kernel<512>;
-        const size_t smem = start_smem_bytes(w.n, T);
-        if ((e = cudaFuncSetAttribute(start, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
-            return e;
-        start<<<2 * w.nch, T, smem, s>>>(w);
-    }
+    if (w.started && (e = launch_start(w, s)) != cudaSuccess) return e;
     for (int st = 0; st < w.nstages; ++st) {
         w.stage = st;
         sweep<<<2 * w.nch, w.threads, ssm, s>>>(w);
@@ -1672,6 +1680,151 @@ cudaError_t launch_sweep_path(const SweepArgs &w0, cudaStream_t s)
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     return cudaSuccess;
+}
+
+// ---- the single-locus report --------------------------------------------------------
+// The locus is a chunk of one core with kReportSteps markers of history on either
+// side: its starting states and one marker of the sort give the run lengths of
+// both directions, and then every step's S is independent of the others: a warp
+// counts 32 steps from the boundaries with M up to its last one (RunCut).  The CTA
+// that finishes last runs the six walks over those counts, 32 steps a turn, with
+// the rules of walk_slot (the whole sample's S is the sum of the two classes').
+// A walk that outlives the history is left to the per-step kernel (rest[q] = 1).
+// Bound by the chain of launches and rounds, not by a step at a time (204
+// haplotypes, 22,147 markers, a locus in a sweep: 269 us by the per-step kernel).
+__global__ void __launch_bounds__(kSplitWarps * 32) report_kernel(ReportArgs r)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ bool last;
+    namespace cg = cooperative_groups;
+    const cg::thread_block_tile<32> tile = cg::tiled_partition<32>(cg::this_thread_block());
+    const int lane = tile.thread_rank(), warp = threadIdx.x >> 5;
+    const SweepArgs &w = r.w;
+    const int n = w.n;
+    const long long m = w.a.m, x0 = w.a.k0;
+    {
+        const int dir = blockIdx.y;
+        const int blk = blockIdx.x * kSplitWarps + warp, lo = 32 * blk + 1;
+        const long long most = dir ? m - 1 - x0 : x0;            // steps inside the array
+        if (lo <= most && lo <= kReportSteps) {                  // uniform over the warp
+            const unsigned char *slot = w.slots + (size_t)dir * w.slot_bytes;
+            const int n0 = ((const int *)slot)[0];
+            const SplitSmem s = split_smem(smem + (size_t)warp * w.split_bytes,
+                                           w.wscratch + ((size_t)(dir * gridDim.x + blockIdx.x) * kSplitWarps + warp) *
+                                                            w.wscratch_bytes, n, false);
+            for (int q = lane; q < s.nw; q += 32) s.O[q] = s.N[q] = 0u;
+            tile.sync();
+            unsigned K0, sup;
+            const unsigned K = mark_window<1>(tile, s, (const uint4 *)(slot + 16), n, n0, lo + 31, true, false, 0, n,
+                                              K0, sup);
+            RunCut<1> rc;
+            rc.lim = (unsigned)(lo + lane + 1) << 16;
+            rc.last = 0u;
+            rc.d[0] = 0u;
+            rc.range(s, 0u, K0);
+            rc.cut((unsigned)n0, 0u);
+            r.S[(size_t)(2 * dir) * kReportSteps + lo - 1 + lane] = (rc.d[0] - (unsigned)n0) >> 1;
+            rc.last = (unsigned)n0;
+            rc.d[0] = 0u;
+            rc.range(s, K0, K);
+            rc.cut((unsigned)n, 0u);
+            r.S[(size_t)(2 * dir + 1) * kReportSteps + lo - 1 + lane] = (rc.d[0] - (unsigned)(n - n0)) >> 1;
+        }
+    }
+    __threadfence();                              // the counts before the tally
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(r.done, 1u) == gridDim.x * gridDim.y - 1u;
+    __syncthreads();
+    if (!last || warp >= 6) return;
+    __threadfence();
+    // ---- walk w = q / 2 (allele 1, allele 0, the whole sample), direction q % 2
+    const int q = warp, wk = q >> 1, dir = q & 1;
+    const unsigned n0 = ((const unsigned *)(w.slots + (size_t)dir * w.slot_bytes))[0], n1 = (unsigned)n - n0;
+    const int hz = ((const int *)(w.slots + (size_t)dir * w.slot_bytes))[1];
+    const unsigned D = (unsigned)c2i(wk == 0 ? n1 : wk == 1 ? n0 : (unsigned)n);
+    if (q < 3 && lane == 0) r.out.denom[q] = (uint64_t)(unsigned)c2i(q == 0 ? n1 : q == 1 ? n0 : (unsigned)n);
+    int status = D == 0u ? WALK_UNDEFINED : WALK_OK, stop = 0;
+    double acc = 0.0;
+    if (D != 0u) {
+        const unsigned long long cutD = (unsigned long long)w.a.cut_num * D;
+        unsigned prev = wk == 2 ? (unsigned)(c2i(n0) + c2i(n1)) : D;
+        uint64_t *trace = r.out.S + (size_t)q * r.capacity;
+        if (lane == 0 && r.capacity > 0) trace[0] = prev;
+        const unsigned *Sd = r.S + (size_t)(2 * dir) * kReportSteps;
+        bool walking = true;
+        for (int i0 = 1; walking; i0 += 32) {
+            const int i = i0 + lane;
+            double gq = 0.0;
+            int gk = 0;
+            const long long step = dir ? 1 : -1, xl = x0 + step * i, xp = xl - step;
+            if (xl < 0 || xl >= m) gk = WALK_EDGE;
+            else {
+                const long long p1 = __ldg(w.a.pos + xl), p0 = __ldg(w.a.pos + xp);
+                const long long bp = dir ? p1 - p0 : p0 - p1;
+                if (bp > w.a.max_gap) gk = WALK_GAP;
+                else {
+                    double gg;
+                    if (w.a.physical) gg = (double)bp;
+                    else {
+                        const double g1 = __ldg(w.a.gmap + xl), g0 = __ldg(w.a.gmap + xp);
+                        gg = dir ? g1 - g0 : g0 - g1;
+                    }
+                    if (bp > w.a.gap_scale) gg = gg * ((double)w.a.gap_scale / (double)bp);
+                    gq = gg;
+                }
+            }
+            unsigned S = 0u;
+            if (gk != WALK_EDGE && i <= kReportSteps) {
+                const unsigned s0 = __ldcg(Sd + i - 1), s1 = __ldcg(Sd + kReportSteps + i - 1);
+                S = wk == 0 ? s1 : wk == 1 ? s0 : s0 + s1;
+            }
+            const unsigned km = tile.ballot(gk != 0), hm = tile.ballot(i > hz || i > kReportSteps);
+            const int ke = km ? __ffs(km) - 1 : 32, he = hm ? __ffs(hm) - 1 : 32;
+            const int end = ke <= he ? ke : he;
+            const unsigned sm = tile.ballot((unsigned long long)w.a.cut_den * S < cutD);
+            const int sl = sm ? __ffs(sm) - 1 : 32;
+            const bool stops = sl < end;
+            const int full = stops ? sl : end;
+            unsigned sp = tile.shfl_up(S, 1);
+            if (lane == 0) sp = prev;
+            if (lane < full + (stops ? 1 : 0) && i < r.capacity) trace[i] = S;
+            if (lane < full + (stops && w.a.crossing ? 1 : 0)) acc += (double)(sp + S) * gq;
+            prev = tile.shfl(S, 31);
+            if (stops) {
+                stop = i0 + sl;
+                walking = false;
+            } else if (end < 32) {
+                status = ke <= he ? tile.shfl(gk, ke & 31) : WALK_UNFINISHED;
+                stop = i0 + end;
+                walking = false;
+            }
+        }
+    }
+    acc = lane_sum_f64<32>(acc);
+    if (lane != 0) return;
+    r.rest[q] = status == WALK_UNFINISHED ? 1 : 0;
+    if (status == WALK_UNFINISHED) return;
+    r.out.len[q] = status == WALK_OK ? stop + 1 : status == WALK_UNDEFINED ? 0 : stop;
+    r.out.stop[q] = stop;
+    r.out.status[q] = (int8_t)status;
+    r.out.ihh[q] = D ? acc / (2.0 * (double)D) : 0.0;
+}
+
+cudaError_t launch_report(const ReportArgs &r, cudaStream_t s)
+{
+    const SweepArgs &w = r.w;
+    cudaError_t e = launch_start(w, s);
+    if (e != cudaSuccess) return e;
+    void (*sweep)(SweepArgs) = sort_kernel(w.n, w.threads);
+    const size_t ssm = sweep_smem_bytes(w.n, w.a.W, w.threads, 1);
+    if ((e = cudaFuncSetAttribute(sweep, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssm)) != cudaSuccess)
+        return e;
+    sweep<<<2, w.threads, ssm, s>>>(w);
+    const size_t wsm = (size_t)w.split_bytes * kSplitWarps;
+    if ((e = cudaFuncSetAttribute(report_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wsm)) != cudaSuccess)
+        return e;
+    report_kernel<<<dim3(kReportSteps / 32 / kSplitWarps, 2), kSplitWarps * 32, wsm, s>>>(r);
+    return cudaGetLastError();
 }
 
 }  // namespace selscan
