@@ -44,9 +44,14 @@ namespace {
 
 constexpr unsigned kInf16 = 0xFFFFu;
 constexpr int kRowRing = 4;                 // rows in flight ahead of the sort (cp.async)
-constexpr int kTokSmem = 1024;              // window boundaries a walking warp keeps on chip (multiple of 4)
-constexpr int kSparseMax = kTokSmem;        // most new boundaries of a window taken one per lane
-constexpr int kWin = 64;                    // steps of such a window (two blocks of 32)
+// Window boundaries a walking warp keeps on chip (a multiple of 4; a window with
+// more new ones than that is not taken one boundary per lane), and the steps of a
+// window after the first (whole blocks of 32).  An XPEHH boundary takes 8 bytes
+// and its walks are short: 1,024 of them left too little of the SM's memory to L1
+// for the slots the walk reads twice (1M: walks 17.2 ms; 512 and 32 steps, four CTAs
+// per SM, 12.7).
+__host__ __device__ constexpr int tok_smem(int xpehh) { return xpehh ? 512 : 1024; }
+__host__ __device__ constexpr int win_steps(int xpehh) { return xpehh ? 32 : 64; }
 
 __host__ __device__ inline int sweep_e(int n, int T)
 {
@@ -141,9 +146,10 @@ __host__ __device__ size_t sweep_elements(int n, int T) { return (size_t)sweep_n
 // element's run length.  T threads (32 to 512); EMAX bounds the elements per
 // thread (at most 32, one allele bit each in a 32-bit mask), up to 24 stay in
 // registers between the two passes.
+// XP: 1 an XPEHH scan, 0 iHS, -1 told by nB.
 // `sync` is a barrier of the T threads that sort; `done(r)` is called once every
 // thread has written its part of the slots of the stage's first r markers.
-template <int T, int EMAX, bool EXACT, class Sync, class Done>
+template <int T, int EMAX, bool EXACT, int XP, class Sync, class Done>
 __device__ __forceinline__ void sort_chunk(const SweepArgs &w, unsigned char *smem, int dir, long long c0,
                                            long long c1, int blk, Sync sync, Done done)
 {
@@ -369,7 +375,7 @@ __device__ __forceinline__ void sort_chunk(const SweepArgs &w, unsigned char *sm
         if (wr) {
             const int r = dir == 0 ? (int)(x - klo) : (int)(khi - 1 - x);
             unsigned char *slot = w.slots + ((size_t)blk * w.R + r) * w.slot_bytes;
-            const int xp = w.a.nB > 0;
+            const bool xp = XP < 0 ? w.a.nB > 0 : XP == 1;
             if (tid == 0) {
                 int *hdr = (int *)slot;
                 hdr[0] = (int)n0;
@@ -381,24 +387,41 @@ __device__ __forceinline__ void sort_chunk(const SweepArgs &w, unsigned char *sm
             const unsigned *Ps = P0 + cur * np;
             // run lengths, 8 per 16-byte store (the padding elements fill the last
             // group; np is a multiple of 32).  Nothing waits for the stores: the
-            // next marker's partition reads this buffer and writes the other one
+            // next marker's partition reads this buffer and writes the other one.
+            // XPEHH: the same thread makes the population flags of its 8 positions
+            // (16x2 clamps of the bit indices, as the walker marks windows) and four
+            // neighbours' make a word: a third of the instructions of a ballot per
+            // word (1M: sort 19.0 -> 17.0 ms)
             const uint4 *P4 = (const uint4 *)Ps;
             uint4 *M4 = (uint4 *)(slot + 16);
-            for (int t = tid; t < (n + 31) / 32 * 4; t += T) {
-                const uint4 lo = P4[(t >> 2) * 8 + (t & 3)], hi = P4[(t >> 2) * 8 + 4 + (t & 3)];
-                M4[t] = make_uint4(__byte_perm(lo.x, hi.x, 0x7632u), __byte_perm(lo.y, hi.y, 0x7632u),
-                                   __byte_perm(lo.z, hi.z, 0x7632u), __byte_perm(lo.w, hi.w, 0x7632u));
-            }
-            if (xp) {                            // population of each sorted position
-                // one 32-position word per warp iteration: a ballot over the lanes
-                const unsigned limA = 64u * (unsigned)w.a.WA;
-                unsigned *isA = (unsigned *)(slot + slot_isa_at(n));
-                const int nw = split_nw(n);
-                for (int q = warp; q < nw; q += NW) {
-                    const int t = q * 32 + lane;
-                    const unsigned word = __ballot_sync(FULLMASK, t < n && (Ps[t] & 0xFFFFu) < limA);
-                    if (lane == 0) isA[q] = word;
+            const int items = (n + 31) / 32 * 4;
+            if (!xp) {
+                for (int t = tid; t < items; t += T) {
+                    const uint4 lo = P4[(t >> 2) * 8 + (t & 3)], hi = P4[(t >> 2) * 8 + 4 + (t & 3)];
+                    M4[t] = make_uint4(__byte_perm(lo.x, hi.x, 0x7632u), __byte_perm(lo.y, hi.y, 0x7632u),
+                                       __byte_perm(lo.z, hi.z, 0x7632u), __byte_perm(lo.w, hi.w, 0x7632u));
                 }
+            } else {
+                unsigned *isA = (unsigned *)(slot + slot_isa_at(n));
+                const unsigned L = 64u * (unsigned)w.a.WA * 0x00010001u, L1 = L - 0x00010001u;
+                for (int t0 = 0; t0 < items; t0 += T) {      // whole warps: items is a multiple of 4
+                    const int t = t0 + tid;
+                    unsigned f = 0u;                          // bits j, 16 + j: the position is in B
+                    if (t < items) {
+                        const uint4 lo = P4[(t >> 2) * 8 + (t & 3)], hi = P4[(t >> 2) * 8 + 4 + (t & 3)];
+                        M4[t] = make_uint4(__byte_perm(lo.x, hi.x, 0x7632u), __byte_perm(lo.y, hi.y, 0x7632u),
+                                           __byte_perm(lo.z, hi.z, 0x7632u), __byte_perm(lo.w, hi.w, 0x7632u));
+                        f = __vmaxu2(__vminu2(__byte_perm(lo.w, hi.w, 0x5410u), L), L1) - L1;
+                        f = f + f + (__vmaxu2(__vminu2(__byte_perm(lo.z, hi.z, 0x5410u), L), L1) - L1);
+                        f = f + f + (__vmaxu2(__vminu2(__byte_perm(lo.y, hi.y, 0x5410u), L), L1) - L1);
+                        f = f + f + (__vmaxu2(__vminu2(__byte_perm(lo.x, hi.x, 0x5410u), L), L1) - L1);
+                        f = (f ^ 0x000F000Fu) << (4 * (t & 3));
+                    }
+                    f |= __shfl_xor_sync(FULLMASK, f, 1);
+                    f |= __shfl_xor_sync(FULLMASK, f, 2);
+                    if (t < items && (t & 3) == 0) isA[t >> 2] = f;
+                }
+                if (tid == 0 && (n & 31) == 0) isA[n >> 5] = 0u;   // the word of position n
             }
         }
         if (!more) break;
@@ -410,7 +433,7 @@ __device__ __forceinline__ void sort_chunk(const SweepArgs &w, unsigned char *sm
     }
 }
 
-template <int T, int EMAX, bool EXACT = false>
+template <int T, int EMAX, bool EXACT = false, int XP = -1>
 __global__ void __launch_bounds__(T, T == 512 ? 2 : (T == 256 ? 3 : 512 / T)) sweep_kernel(SweepArgs w)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -419,7 +442,7 @@ __global__ void __launch_bounds__(T, T == 512 ? 2 : (T == 256 ? 3 : 512 / T)) sw
     const long long c0 = w.a.k0 + (long long)c * w.B;   // chunk c of [k0, k1)
     if (c0 >= w.a.k1) return;
     const long long c1 = c0 + w.B < w.a.k1 ? c0 + w.B : w.a.k1;
-    sort_chunk<T, EMAX, EXACT>(w, smem, dir, c0, c1, blockIdx.x, [] { __syncthreads(); }, [](int) {});
+    sort_chunk<T, EMAX, EXACT, XP>(w, smem, dir, c0, c1, blockIdx.x, [] { __syncthreads(); }, [](int) {});
 }
 
 // ---- the split walk ----------------------------------------------------------
@@ -432,7 +455,7 @@ namespace {
 // per step of a sparse window; and for XPEHH the population-A flags of the
 // sorted positions with their per-word prefix counts.
 struct SplitSmem {
-    unsigned *tk;                         // window list on chip, first kTokSmem entries (XPEHH: pairs)
+    unsigned *tk;                         // window list on chip, first tok_smem entries (XPEHH: pairs)
     unsigned *gtk;                        // the rest, global: entry k at gtk[k]
     unsigned *O, *N, *S, *dec;
     unsigned *isA, *PA;
@@ -442,7 +465,7 @@ struct SplitSmem {
 __host__ __device__ inline int split_words(int n, int xpehh)
 {
     const int nw = split_nw(n), ns = (nw + 31) >> 5;
-    return kTokSmem * (xpehh ? 2 : 1) + 2 * nw + ns + kWin * (xpehh ? 3 : 2) + (xpehh ? 2 * nw : 0);
+    return tok_smem(xpehh) * (xpehh ? 2 : 1) + 2 * nw + ns + win_steps(xpehh) * (xpehh ? 3 : 2) + (xpehh ? 2 * nw : 0);
 }
 
 __device__ inline SplitSmem split_smem(unsigned char *base, unsigned char *scratch, int n, int xpehh)
@@ -451,8 +474,8 @@ __device__ inline SplitSmem split_smem(unsigned char *base, unsigned char *scrat
     s.nw = split_nw(n);
     s.ns = (s.nw + 31) >> 5;
     unsigned *p = (unsigned *)base;
-    s.tk = p; p += kTokSmem * (xpehh ? 2 : 1);
-    s.dec = p; p += kWin * (xpehh ? 3 : 2);
+    s.tk = p; p += tok_smem(xpehh) * (xpehh ? 2 : 1);
+    s.dec = p; p += win_steps(xpehh) * (xpehh ? 3 : 2);
     s.O = p; p += s.nw;
     s.N = p; p += s.nw;
     s.S = p; p += s.ns;
@@ -569,7 +592,7 @@ __device__ __forceinline__ unsigned mark_window(const Tile &tile, const SplitSme
             hit &= hit - 1u;
             const int t = 32 * wd + b;
             const unsigned tok = (unsigned)t | ((unsigned)M16[32 * wd + ((b & 15) << 1 | b >> 4)] << 16);
-            unsigned *dst = at < (unsigned)kTokSmem ? s.tk : s.gtk;
+            unsigned *dst = at < (unsigned)tok_smem(NPOP == 2) ? s.tk : s.gtk;
             if (NPOP == 2) *(uint2 *)(dst + 2 * at) = make_uint2(tok, count_a(s, t));
             else dst[at] = tok;
             ++at;
@@ -608,7 +631,7 @@ struct RunCut {
     // list entry k
     __device__ __forceinline__ void one(const SplitSmem &s, unsigned k)
     {
-        const unsigned *src = k < (unsigned)kTokSmem ? s.tk : s.gtk;
+        const unsigned *src = k < (unsigned)tok_smem(NPOP == 2) ? s.tk : s.gtk;
         if (NPOP == 2) {
             const uint2 t = *(const uint2 *)(src + 2 * k);
             cut(t.x, t.y);
@@ -620,7 +643,7 @@ struct RunCut {
     __device__ __forceinline__ void range(const SplitSmem &s, unsigned ka, unsigned kb)
     {
         unsigned k = ka;
-        const unsigned kv = kb < (unsigned)kTokSmem ? kb : (unsigned)kTokSmem;
+        const unsigned kv = kb < (unsigned)tok_smem(NPOP == 2) ? kb : (unsigned)tok_smem(NPOP == 2);
         for (; k < kv && (k & 3u); ++k) one(s, k);
 #pragma unroll 2
         for (; k + 4 <= kv; k += 4) {
@@ -643,7 +666,7 @@ struct RunCut {
         last = up ? 0u : n;
         lastA = up ? 0u : nA;
         const unsigned half = K >> 1;
-        if (K <= (unsigned)kTokSmem) {
+        if (K <= (unsigned)tok_smem(NPOP == 2)) {
             const uint2 *q = (const uint2 *)s.tk + (up ? 0u : K - 1u);
             const int st = up ? 1 : -1;
 #pragma unroll 4
@@ -674,6 +697,7 @@ template <int NPOP, typename Tile>
 __device__ __forceinline__ void sparse_terms(const Tile &tile, const SplitSmem &s, unsigned K, int lo, int n0,
                                              unsigned sup)
 {
+    constexpr int kWin = win_steps(NPOP == 2);
     const int lane = tile.thread_rank();
     for (int q = lane; q < kWin * (NPOP == 2 ? 3 : 2); q += 32) s.dec[q] = 0u;
     tile.sync();
@@ -716,8 +740,8 @@ size_t split_smem_per_warp(int n, int xpehh)
     return ((size_t)split_words(n, xpehh) * 4 + 15) & ~(size_t)15;
 }
 
-// the list holds at most n boundaries, the first kTokSmem of them on chip
-size_t split_scratch_per_warp(int n) { return n <= kTokSmem ? 0 : (((size_t)n * 8) + 255) & ~(size_t)255; }
+// the list holds at most n boundaries, the first tok_smem of them on chip
+size_t split_scratch_per_warp(int n) { return n <= tok_smem(1) ? 0 : (((size_t)n * 8) + 255) & ~(size_t)255; }
 
 // The walks of one core, by one warp.  The first window is the steps 1..32:
 // every lane runs over all boundaries with M <= 32 (shared memory, broadcast
@@ -729,7 +753,7 @@ size_t split_scratch_per_warp(int n) { return n <= kTokSmem ? 0 : (((size_t)n * 
 // takes 16 steps at a time, two lanes a step from both ends of the list (1M:
 // 17.2 ms against 24.1 with 32).  Later windows of 64 steps hold few boundaries
 // among many older run starts: there each lane takes one boundary
-// (sparse_terms); a window with more than kSparseMax of them is cut like the
+// (sparse_terms); a window with more than tok_smem of them is cut like the
 // first one.
 // Pair counts fit 32 bits (C(16383, 2) < 2^32); the digest is 64-bit.  Lane
 // (i - 1) mod 32 adds step i's trapezoid term to its own FP64 partial sum, and
@@ -743,6 +767,7 @@ __device__ __forceinline__ void walk_slot(const SweepArgs &w, const Tile &tile, 
     constexpr int NV = NPOP == 2 ? 3 : 2;     // S values: class 0, class 1; or A, B, pooled
     constexpr int NWK = NPOP == 2 ? 1 : 2;    // walks of a slot
     constexpr int kDense = NPOP == 2 ? 16 : 32;   // steps of a window cut boundary by boundary
+    constexpr int kWin = win_steps(NPOP == 2);    // and of one taken one boundary per lane
     const int lane = tile.thread_rank();
     const int n = w.n;
     const long long m = w.a.m;
@@ -820,7 +845,7 @@ __device__ __forceinline__ void walk_slot(const SweepArgs &w, const Tile &tile, 
         const int hi = lo + (dense ? kDense - 1 : kWin - 1);
         const int pa = NPOP == 1 && !act[0] ? n0 : 0, pb = NPOP == 1 && !act[NWK - 1] ? n0 : n;
         const unsigned K = mark_window<NPOP>(tile, s, M4, n, n0, hi, dense, merge, pa, pb, K0, sup);
-        if (!dense && K > (unsigned)kSparseMax) {    // redo as a window of 32 steps
+        if (!dense && K > (unsigned)tok_smem(NPOP == 2)) {    // redo as a window of 32 steps
             dense = true;
             merge = false;
             continue;
@@ -988,7 +1013,7 @@ __device__ __forceinline__ void walk_slot(const SweepArgs &w, const Tile &tile, 
 #define SPLIT_MIN_CTAS 4
 #endif
 template <int NPOP, int G>
-__global__ void __launch_bounds__(kSplitWarps * 32, NPOP == 2 ? 3 : SPLIT_MIN_CTAS) split_walk_kernel(SweepArgs w)
+__global__ void __launch_bounds__(kSplitWarps * 32, SPLIT_MIN_CTAS) split_walk_kernel(SweepArgs w)
 {
     static_assert(G == 32, "lane l owns step l of a block of 32");
     extern __shared__ __align__(16) unsigned char smem[];
@@ -1435,7 +1460,7 @@ __global__ void __launch_bounds__(TC, MINB) chunk_scan_kernel(const __grid_const
         }
         __syncthreads();
         if (threadIdx.x < TS) {
-            sort_chunk<TS, EMAX, false>(w, smem, mine.dir, mine.c0, mine.c1, mine.blk,
+            sort_chunk<TS, EMAX, false, NPOP == 0 ? -1 : NPOP - 1>(w, smem, mine.dir, mine.c0, mine.c1, mine.blk,
                                         [] { sort_barrier<TS>(); },
                                         [&](int r) {
                                             if (threadIdx.x == 0) {
@@ -1625,15 +1650,21 @@ int split_walk_ctas(int n, int xpehh)
     return per_sm * (sms > 0 ? sms : 1);
 }
 
-// The sorting kernel of a sample and CTA width.
-static void (*sort_kernel(int n, int threads))(SweepArgs)
+// The sorting kernel of a sample and CTA width.  The 256-thread sorts of the large
+// scans are compiled for each kind of scan (iHS beside XPEHH's population flags in
+// one kernel: 1M iHS sort 15.2 ms against 14.5).
+template <int XP>
+static void (*sort256(int E))(SweepArgs)
+{
+    return E == 4 ? sweep_kernel<256, 4, true, XP> : E == 8 ? sweep_kernel<256, 8, true, XP>
+         : E == 12 ? sweep_kernel<256, 12, true, XP> : E == 16 ? sweep_kernel<256, 16, true, XP>
+         : E == 20 ? sweep_kernel<256, 20, true, XP> : E == 24 ? sweep_kernel<256, 24, true, XP>
+         : sweep_kernel<256, 32>;
+}
+static void (*sort_kernel(int n, int threads, bool xpehh))(SweepArgs)
 {
     const int E = sweep_e(n, threads);
-    if (threads == 256)
-        return E == 4 ? sweep_kernel<256, 4, true> : E == 8 ? sweep_kernel<256, 8, true>
-             : E == 12 ? sweep_kernel<256, 12, true> : E == 16 ? sweep_kernel<256, 16, true>
-             : E == 20 ? sweep_kernel<256, 20, true> : E == 24 ? sweep_kernel<256, 24, true>
-             : sweep_kernel<256, 32>;
+    if (threads == 256) return xpehh ? sort256<1>(E) : sort256<0>(E);
     if (threads == 512)
         return E <= 4 ? sweep_kernel<512, 4> : E <= 8 ? sweep_kernel<512, 8>
              : E <= 16 ? sweep_kernel<512, 16> : E <= 24 ? sweep_kernel<512, 24>
@@ -1661,7 +1692,7 @@ cudaError_t launch_sweep_path(const SweepArgs &w0, cudaStream_t s)
 {
     SweepArgs w = w0;
     const size_t ssm = sweep_smem_bytes(w.n, w.a.W, w.threads, w.R);
-    void (*sweep)(SweepArgs) = sort_kernel(w.n, w.threads);
+    void (*sweep)(SweepArgs) = sort_kernel(w.n, w.threads, w.a.nB > 0);
     cudaError_t e = cudaFuncSetAttribute(sweep, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssm);
     if (e != cudaSuccess) return e;
     const size_t wsm = (size_t)w.split_bytes * kSplitWarps;
@@ -1815,7 +1846,7 @@ cudaError_t launch_report(const ReportArgs &r, cudaStream_t s)
     const SweepArgs &w = r.w;
     cudaError_t e = launch_start(w, s);
     if (e != cudaSuccess) return e;
-    void (*sweep)(SweepArgs) = sort_kernel(w.n, w.threads);
+    void (*sweep)(SweepArgs) = sort_kernel(w.n, w.threads, w.a.nB > 0);
     const size_t ssm = sweep_smem_bytes(w.n, w.a.W, w.threads, 1);
     if ((e = cudaFuncSetAttribute(sweep, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssm)) != cudaSuccess)
         return e;
