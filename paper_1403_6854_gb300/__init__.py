@@ -365,6 +365,18 @@ def _workspace(nbytes: int, device, workspace: Optional[torch.Tensor]):
     return ws[off:off + max(nbytes, 256)]
 
 
+def _scan_workspace(n: int, k: int, mode: int, launch, device, workspace: Optional[torch.Tensor]):
+    need = selscan_workspace_bytes(n, k, mode, launch)
+    if workspace is not None:
+        # an in-order scan also runs step by step, in less
+        step = selscan_launch.from_buffer_copy(launch) if launch is not None else selscan_launch()
+        if launch is None:
+            step.schedule = SCHED_DEFAULT
+        step.warps_per_cta = step.warps_per_cta or 8
+        need = min(need, selscan_workspace_bytes(n, k, mode, step))
+    return _workspace(need, device, workspace)
+
+
 def _as_rows(hap: torch.Tensor) -> torch.Tensor:
     if hap.dim() != 2 or hap.element_size() != 8 or not hap.is_cuda or not hap.is_contiguous():
         raise ValueError("hap must be a contiguous 2-D 64-bit CUDA tensor [m, ld]")
@@ -416,7 +428,7 @@ def selscan_ihs_range(hap: torch.Tensor, n: int, pos: torch.Tensor, gmap: torch.
     if out is None:
         out = _ihs_outputs(max(k1 - k0, 0), dev)
     p = params if params is not None else selscan_default_params()
-    ws = _workspace(selscan_workspace_bytes(n, max(k1 - k0, 1), MODE_IHS, launch), dev, workspace)
+    ws = _scan_workspace(n, max(k1 - k0, 1), MODE_IHS, launch, dev, workspace)
     o = selscan_ihs_out(*(_ptr(out[f]) for f in ("status", "n1", "ihh1", "ihh0", "lnratio",
                                                   "stop", "digest", "error")))
     rc = lib.selscan_ihs_range(_ptr(hap), ld, n, m, k0, k1, _ptr(pos), _ptr(gmap), ctypes.byref(p),
@@ -453,8 +465,7 @@ def selscan_xpehh_range(hap: torch.Tensor, nA: int, nB: int, pos: torch.Tensor,
     if out is None:
         out = _xpehh_outputs(max(k1 - k0, 0), dev)
     p = params if params is not None else selscan_default_params()
-    ws = _workspace(selscan_workspace_bytes(nA + nB, max(k1 - k0, 1), MODE_XPEHH, launch), dev,
-                    workspace)
+    ws = _scan_workspace(nA + nB, max(k1 - k0, 1), MODE_XPEHH, launch, dev, workspace)
     o = selscan_xpehh_out(*(_ptr(out[f]) for f in ("status", "n1", "ihhA", "ihhB", "lnratio",
                                                     "stop", "digest", "error")))
     rc = lib.selscan_xpehh_range(_ptr(hap), ld, nA, nB, m, k0, k1, _ptr(pos), _ptr(gmap),

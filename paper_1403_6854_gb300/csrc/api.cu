@@ -64,13 +64,13 @@ struct Plan {
 inline size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 
-SweepPlan make_sweep_plan(int n_total, long long m, int mode, const selscan_launch *L)
+SweepPlan make_sweep_plan(int n_total, long long m, int mode, const selscan_launch *L, bool start = true)
 {
     SweepPlan w;
     // chunks start from a sorted state made directly from the history's 32-marker
     // words where one CTA's shared memory holds the sort (n up to about 10,500);
     // larger samples sweep the history marker by marker
-    w.started = start_smem_bytes(n_total, 512) <= kMaxSmemPerCta;
+    w.started = start && start_smem_bytes(n_total, 512) <= kMaxSmemPerCta;
     w.L = (L && L->sweep_warmup > 0) ? L->sweep_warmup : (w.started ? kDefaultSweepHistory : kDefaultSweepWarmup);
     if (w.L < 16) w.L = 16;
     if (w.L > 16384) w.L = 16384;
@@ -169,13 +169,12 @@ bool chunk_plan(int n_total, long long m, int mode, const selscan_launch *L, Swe
 }
 
 // The schedule of a default launch: the sorted sweep once the chromosome is
-// long enough for its chunks' sequential sorts (each about B + warm-up
-// markers, n elements per marker) to cost less than walking every step, the
-// in-order per-step schedule otherwise.  The crossover depends on the walk
-// lengths: on mosaics of n / 25 founders (long walks) about 7k markers at
-// n = 100, 12k at 1,000, 23k at 2,000 and 30k at 5,000; on a 22k-marker
-// chromosome with short walks the per-step walk is still 2-4x faster.  The
-// rule sits above both.
+// long, the in-order schedule otherwise.  Both sort (chunk_plan) wherever the
+// line runs below 65,000 markers and 6,144 haplotypes, and the line only
+// decides between one launch and several; it was drawn against the per-step
+// walk, which above it loses on mosaics of n / 25 founders (it lost from about
+// 7k markers at n = 100, 30k at 5,000), and is kept so that saved plans and
+// callers that ask for the schedule see the same answer.
 int default_schedule(int mode, long long n_total, long long m)
 {
     if (mode == SELSCAN_MODE_EHH || n_total < 2 || n_total > kSweepMaxN) return SELSCAN_SCHED_IN_ORDER;
@@ -370,17 +369,24 @@ int run_scan(int mode, const uint64_t *hap, int64_t ld, int32_t nA, int32_t nB, 
 {
     const int n_total = nA + nB;
     const long long ncores = k1 - k0;
-    const Plan plan = make_plan(mode, ld, launch, n_total, ncores);
+    Plan plan = make_plan(mode, ld, launch, n_total, ncores);
+    const bool sweep = plan.schedule == SELSCAN_SCHED_SWEEP;
+    bool chunked = plan.chunked && k0 == 0 && k1 == m;
+    Layout l = make_layout(n_total, ncores, mode, plan.nslots, sweep || chunked ? &plan.sw : nullptr);
+    if (workspace && ws_bytes < l.total) {
+        // a workspace sized for another shape still serves: the in-order scan
+        // step by step, the sweep without the words of the starting states
+        chunked = false;
+        if (sweep) plan.sw = make_sweep_plan(n_total, ncores, mode, launch, false);
+        l = make_layout(n_total, ncores, mode, plan.nslots, sweep ? &plan.sw : nullptr);
+    }
     if (plan.schedule < 0 || (launch && launch->warps_per_cta < 0)) return SELSCAN_ERR_INVALID_ARG;
     if (smem_per_warp(plan.cap_s, plan.tcap_s, plan.rowcap, plan.poscap) * (size_t)plan.wpc > kMaxSmemPerCta)
         return SELSCAN_ERR_UNSUPPORTED;
-    const bool sweep = plan.schedule == SELSCAN_SCHED_SWEEP;
     if (sweep && (sweep_smem_bytes(n_total, (nA + 63) / 64 + (nB + 63) / 64, plan.sw.threads, plan.sw.R) > kMaxSmemPerCta ||
                   (size_t)plan.sw.split_bytes * kSplitWarps > kMaxSmemPerCta))
         return SELSCAN_ERR_UNSUPPORTED;
     if (sweep && (plan.sw.slot_bytes & 15)) return SELSCAN_ERR_UNSUPPORTED;   // slots are read in 16-byte units
-    const Layout l = make_layout(n_total, ncores, mode, plan.nslots, sweep || plan.chunked ? &plan.sw : nullptr);
-    const bool chunked = plan.chunked && k0 == 0 && k1 == m;
     if (!workspace || ws_bytes < l.total || ((uintptr_t)workspace & 255)) return SELSCAN_ERR_WORKSPACE;
     cudaStream_t s = (cudaStream_t)stream;
     unsigned char *ws = (unsigned char *)workspace;
@@ -503,7 +509,7 @@ int ehh_prepare(const uint64_t *hap, int64_t ld, int32_t n, int64_t m, const int
     sc->base = nullptr;
     sc->err = out->error;
     *scratch_off = l.scratch;
-    *ws_need = report_layout(n, l.total).total;
+    *ws_need = l.total;
     return SELSCAN_OK;
 }
 
@@ -704,7 +710,9 @@ int selscan_ehh(const uint64_t *hap, int64_t ld, int32_t n, int64_t m, const int
     if (rc != SELSCAN_OK) return rc;
     if (!workspace || ws_bytes < need || ((uintptr_t)workspace & 255)) return SELSCAN_ERR_WORKSPACE;
     sc.base = (unsigned char *)workspace + scratch_off;
-    return ehh_run(a, locus, p, sc, out, capacity, (unsigned char *)workspace, stream);
+    // a workspace without room for the sorted form: the per-step walks alone
+    const bool sorted = ws_bytes >= report_layout(n, need).total;
+    return ehh_run(a, locus, p, sc, out, capacity, sorted ? (unsigned char *)workspace : nullptr, stream);
 }
 
 int selscan_pack(const uint8_t *hap01, int32_t n, int64_t m, int32_t hap_major, uint64_t *rows,

@@ -748,11 +748,11 @@ size_t split_scratch_per_warp(int n) { return n <= tok_smem(1) ? 0 : (((size_t)n
 // reads) and cuts at those of its own step, so S(i) = (sum of squared run
 // lengths - haplotypes) / 2 of 32 steps costs about six instructions per
 // boundary, where a step at a time needs two bitmap searches, three shared
-// atomics and two warp sums per step with most lanes idle (1M iHS: 13.5 -> 8.4
-// ms).  The pooled XPEHH walk, three counts per boundary and few steps long,
+// atomics and two warp sums per step with most lanes idle (1M iHS: 13.5 ms ->
+// 7.4).  The pooled XPEHH walk, three counts per boundary and few steps long,
 // takes 16 steps at a time, two lanes a step from both ends of the list (1M:
-// 17.2 ms against 24.1 with 32).  Later windows of 64 steps hold few boundaries
-// among many older run starts: there each lane takes one boundary
+// 17.2 ms against 24.1 with 32; 12.7 since its list is shorter, tok_smem).  Later
+// windows (win_steps) hold few boundaries among many older run starts: there each lane takes one boundary
 // (sparse_terms); a window with more than tok_smem of them is cut like the
 // first one.
 // Pair counts fit 32 bits (C(16383, 2) < 2^32); the digest is 64-bit.  Lane

@@ -110,3 +110,32 @@ def test_ticks_equal_scans_alone(sg, sizes):
         a, b = ("ihhA", "ihhB") if s.nB else ("ihh1", "ihh0")
         ref = {**ref, "ihh_a": ref.pop(a), "ihh_b": ref.pop(b)}
         assert_bitwise_equal(got, ref)
+
+
+@pytest.mark.parametrize("n,m", [(513, 2400), (600, 40_000)])
+def test_smaller_workspaces_same_bits(sg, n, m):
+    """Workspaces one percent smaller each time, down to the first that is
+    refused: those without room for the chunks' slots (in-order) or for the
+    starting states' words (sweep) take the per-step walk or swept histories,
+    with the same bits."""
+    import torch
+    hap, pos, gmap = synth.tiny_mosaic(n, m, n + m, founders=8, switch=0.02, flip=0.002)
+    h, p, g = sg.to_device(synth.pack(hap), pos, gmap)
+    full = sg.selscan_workspace_bytes(n, m, sg.MODE_IHS)
+    ws = torch.empty(full + 256, dtype=torch.uint8, device="cuda")
+    ws = ws[(-ws.data_ptr()) % 256:][:full]
+    lib, first = sg.load_library(), None
+    for pct in range(100, 0, -1):
+        out = sg._ihs_outputs(m, h.device)
+        o = sg.selscan_ihs_out(*(out[f].data_ptr() for f in ("status", "n1", "ihh1", "ihh0", "lnratio",
+                                                             "stop", "digest", "error")))
+        rc = lib.selscan_ihs(h.data_ptr(), h.shape[1], n, m, p.data_ptr(), g.data_ptr(),
+                             sg.selscan_default_params(), o, ws.data_ptr(), full * pct // 100, None, None)
+        if rc == sg.ERR_WORKSPACE:
+            break
+        assert rc == sg.OK
+        torch.cuda.synchronize()
+        sg.check(out)
+        first = first or to_np(out)
+        assert_bitwise_equal(first, to_np(out))
+    assert 1 < pct < 99

@@ -51,3 +51,34 @@ def test_equals_per_step_report(sg, n, m, kind):
     for f in ("len", "stop", "status", "denom"):
         assert np.array_equal(a[f], ref[f]), f
     np.testing.assert_allclose(a["ihh"], ref["ihh"], rtol=1e-12, atol=0)
+
+
+def test_smaller_workspaces_same_bits(sg):
+    """Down to the first workspace that is refused; those without room for the
+    sorted form take the per-step walks."""
+    import torch
+    n, m, locus = 300, 900, 450
+    hap, pos, gmap = synth.tiny_mosaic(n, m, 5, founders=6, switch=0.02, flip=0.003)
+    h, p, g = sg.to_device(synth.pack(hap), pos, gmap)
+    full = sg.selscan_workspace_bytes(n, m, sg.MODE_EHH)
+    ws = torch.empty(full + 256, dtype=torch.uint8, device="cuda")
+    ws = ws[(-ws.data_ptr()) % 256:][:full]
+    lib, first = sg.load_library(), None
+    for pct in range(100, 0, -1):
+        out = dict(S=torch.zeros((3, 2, 64), dtype=torch.int64, device="cuda"),
+                   **{f: torch.empty((3, 2), dtype=d, device="cuda") for f, d in
+                      (("len", torch.int64), ("stop", torch.int32), ("status", torch.int8), ("ihh", torch.float64))},
+                   denom=torch.empty(3, dtype=torch.int64, device="cuda"),
+                   error=torch.zeros(1, dtype=torch.int32, device="cuda"))
+        o = sg.selscan_ehh_out(*(out[f].data_ptr() for f in ("S", "len", "stop", "status", "ihh", "denom", "error")))
+        rc = lib.selscan_ehh(h.data_ptr(), h.shape[1], n, m, p.data_ptr(), g.data_ptr(), locus,
+                             sg.selscan_default_params(), o, 64, ws.data_ptr(), full * pct // 100, None)
+        if rc == sg.ERR_WORKSPACE:
+            break
+        assert rc == sg.OK
+        torch.cuda.synchronize()
+        sg.check(out)
+        first = first or to_np(out)
+        for f, v in to_np(out).items():
+            assert np.array_equal(first[f], v), f
+    assert 1 < pct < 99
