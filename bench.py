@@ -210,16 +210,17 @@ def run_reference(args, rank, world):
     }), flush=True)
 
 
-SWEEP_DRAM_BYTES_PER_CORE = 4.6139e9 / 125020
 # ncu capture of the 250k case (5,000 x 250,000, default sweep shape; summarised
-# in profiles/sweep_split_walk_ihs250k_full.md): sweep_kernel alone read + wrote
-# 3.489 GB (125,020 core loci) and issued 7.164e9 warp instructions over
-# 997,618 marker passes of 5,120 elements, i.e. 44.88 thread instructions per
-# sorted element and marker pass, 19.80 of them on the ALU pipe
-# (sm__inst_executed_pipe_alu 3.161e9 warp instructions)
-SORT_DRAM_BYTES_PER_CORE = 3.4889e9 / 125020
-SORT_INSTR_PER_ELEMENT_PASS = 44.88
-SORT_ALU_OPS_PER_ELEMENT_PASS = 19.80
+# in profiles/sweep_split_walk_ihs250k_full.md): thread instructions of
+# sweep_kernel per sorted element and marker pass (500,000 passes of 5,120
+# elements), and of start_kernel per element and 32-marker word of history
+# (114,541 words), in all and on the ALU pipe; and both kernels' DRAM
+# traffic over 125,020 core loci
+SORT_DRAM_BYTES_PER_CORE = 3.2546e9 / 125020
+SORT_INSTR_PER_ELEMENT_PASS = 39.11
+SORT_ALU_OPS_PER_ELEMENT_PASS = 20.53
+START_INSTR_PER_ELEMENT_WORD = 21.32
+START_ALU_OPS_PER_ELEMENT_WORD = 9.59
 
 
 def main():
@@ -492,21 +493,27 @@ def main():
             pk = int_peak.measure()
             issue_peak = float(np.median([pk[o]["ops_per_s"] for o in ("IADD3", "IMNMX")]))
             alu_peak = float(np.median([pk[o]["ops_per_s"] for o in ("LOP3", "PRMT", "SHF")]))
-            element_passes = work[0] * work[1]
-            ops = element_passes * SORT_INSTR_PER_ELEMENT_PASS / (sort_ms / 1e3)
-            alu = element_passes * SORT_ALU_OPS_PER_ELEMENT_PASS / (sort_ms / 1e3)
-            roofline = {"bound": "alu", "kernel": "sweep_kernel (the sort; first stage)",
+            # one marker pass per core and direction; the rest of the library's count
+            # are the 32-marker words of the chunks' histories (start_kernel)
+            marker_passes = 2 * (k1 - k0)
+            words = work[0] - marker_passes
+            ops = work[1] * (marker_passes * SORT_INSTR_PER_ELEMENT_PASS +
+                             words * START_INSTR_PER_ELEMENT_WORD) / (sort_ms / 1e3)
+            alu = work[1] * (marker_passes * SORT_ALU_OPS_PER_ELEMENT_PASS +
+                             words * START_ALU_OPS_PER_ELEMENT_WORD) / (sort_ms / 1e3)
+            roofline = {"bound": "alu", "kernel": "start_kernel + sweep_kernel (the sort; first stage)",
                         "achieved": ops / 1e9, "peak": issue_peak / 1e9, "unit": "Gop/s",
                         "frac": ops / issue_peak,
                         "traffic": cores * SORT_DRAM_BYTES_PER_CORE,
-                        "traffic_note": "ncu capture of the 250k case (3.489 GB of sweep_kernel "
-                                        "DRAM traffic over 125,020 core loci), scaled by core loci",
+                        "traffic_note": "ncu capture of the 250k case (DRAM traffic of both "
+                                        "kernels over 125,020 core loci), scaled by core loci",
                         "kernel_ms": sort_ms, "split_walk_ms": walk_ms - sort_ms,
-                        "element_passes": element_passes, "marker_passes": work[0],
+                        "elements": work[1], "marker_passes": marker_passes, "history_words": words,
                         "ops_per_element_pass": SORT_INSTR_PER_ELEMENT_PASS,
+                        "ops_per_element_word": START_INSTR_PER_ELEMENT_WORD,
                         "ops_note": "integer thread instructions (all pipes) per sorted element and "
-                                    "marker pass from the ncu capture of the 250k case, times the "
-                                    "passes of this launch",
+                                    "marker pass, and per element and 32-marker history word, from "
+                                    "the ncu capture of the 250k case, times those of this launch",
                         "peak_source": "integer issue rate (IADD3 / IMNMX chains: 128 thread "
                                        "operations = 4 warp instructions per SM cycle) measured "
                                        "in this run by libselscan_peak",
@@ -651,7 +658,7 @@ def run_complexity(args):
     import __graft_entry__
     __graft_entry__.build()
     import paper_1403_6854_gb300 as sg
-    shapes = [("per_step", sg.make_launch(sg.SCHED_IN_ORDER)), ("sorted_sweep", sg.make_launch(sg.SCHED_SWEEP))]
+    shapes = [("per_step", sg.make_launch(sg.SCHED_IN_ORDER, warps_per_cta=8)), ("sorted_sweep", sg.make_launch(sg.SCHED_SWEEP))]
 
     def point(n, dens):
         sp = synth.complexity_spec(n, dens)

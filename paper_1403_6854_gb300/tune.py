@@ -24,10 +24,10 @@ SHAPE_FIELDS = ("schedule", "warps_per_cta", "smem_entries", "window_rows", "cor
 
 SWEEP_MAX_N = 16383
 SWEEP_CANDIDATES: List[Dict] = [
-    dict(schedule=1, warps_per_cta=4),          # per-step in-order, for short chromosomes
+    dict(schedule=1, warps_per_cta=4),          # per-step in-order
     dict(schedule=3),
-    dict(schedule=3, sweep_warmup=2048),        # longer histories: fewer walks handed to
-    dict(schedule=3, sweep_warmup=4096),        # the per-step second pass
+    dict(schedule=3, sweep_warmup=2048),        # shorter histories: less to sort, more walks
+    dict(schedule=3, sweep_warmup=4096),        # handed to the per-step second pass
     dict(schedule=3, sweep_threads=512),
 ]
 
