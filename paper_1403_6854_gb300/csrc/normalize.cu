@@ -280,7 +280,9 @@ __global__ void norm_finish_kernel(int nbins, int pass, const long long *bin_cou
 // cycle) and the divide is what the kernel spends its time on: the bin's
 // reciprocal is taken once per CTA, and a quotient is one product corrected by
 // its exact remainder (Markstein's method: correctly rounded, like the divide);
-// quotients that are not in the ordinary range take the divide.
+// quotients that are not in the ordinary range, and bins whose reciprocal is not
+// (an SD that overflowed to infinity has 0, a subnormal one infinity), take the
+// divide.
 __device__ __forceinline__ bool ordinary(double v)
 {
     // 2^-767 <= |v| < 2^768, on the integer pipe: a compare would take the FP64 pipe
@@ -300,13 +302,14 @@ __global__ void __launch_bounds__(kApplyThreads) norm_apply_kernel(const double 
                                                                    const double *bin_sd,
                                                                    const long long *bin_count, double *out)
 {
-    extern __shared__ double tab[];              // per bin: mean, SD, 1 / SD (0: no score)
+    extern __shared__ double tab[];              // per bin: mean, SD, 1 / SD (0: no score; NaN: divide)
     for (int b = threadIdx.x; b < nbins; b += kApplyThreads) {
         const double sd = bin_sd[b];
         const bool ok = bin_count[b] >= 2 && sd > 0.0;
         tab[3 * b] = bin_mean[b];
         tab[3 * b + 1] = sd;
-        tab[3 * b + 2] = ok ? 1.0 / sd : 0.0;
+        const double inv = 1.0 / sd;
+        tab[3 * b + 2] = !ok ? 0.0 : ordinary(inv) ? inv : __longlong_as_double(0x7ff8000000000000ll);
     }
     __syncthreads();
     const bool small = (unsigned long long)n * (unsigned long long)nbins < (1ull << 32);
