@@ -1376,6 +1376,20 @@ __device__ __forceinline__ void sort_barrier()
     else asm volatile("bar.sync 1, %0;" ::"n"(TS) : "memory");
 }
 
+// Waits until the CTA's sorting warps have written slot r, `limit` looks at the
+// most.  Each lane looks, the warp decides together: lanes that left on their own
+// count could part when the slot is written around the last look.  (One lane
+// looking for its warp takes chr22 iHS from 0.33 to 0.62 ms.)
+__device__ __forceinline__ bool wait_slot(const volatile int *ready, int r, int limit)
+{
+    int looks = 0;
+    while (*ready <= r && ++looks < limit) __nanosleep(64);
+    const bool ok = !__any_sync(FULLMASK, looks >= limit);
+    __threadfence_block();                    // the flag before the slot
+    __syncwarp();
+    return ok;
+}
+
 // One chunk and direction of one scan.
 struct ChunkTask { const SweepArgs *w; long long c0, c1; int dir, blk, cnt; };
 
@@ -1483,14 +1497,10 @@ __global__ void __launch_bounds__(TC, MINB) chunk_scan_kernel(const __grid_const
                 if (lane == 0) r = atomicAdd(&own_next, 1);
                 r = __shfl_sync(FULLMASK, r, 0);
                 if (r >= mine.cnt) break;
-                int polls = 0;
-                while (own_ready <= r && ++polls < kChunkPolls) __nanosleep(64);
-                if (polls >= kChunkPolls) {
+                if (!wait_slot(&own_ready, r, kChunkPolls)) {
                     if (lane == 0) atomicExch(w.err, SELSCAN_ERR_TIMEOUT);
                     break;
                 }
-                __threadfence_block();        // the flag before the slot
-                __syncwarp();
                 walk_one(mine, r);
             }
         }
