@@ -35,7 +35,6 @@ constexpr int kDefaultSweepHistory = 8192;
 constexpr size_t kSweepSlotBudget = (size_t)24 << 30;  // bytes of sweep slots per scan
 constexpr long long kSweepMinMarkers = 32768;          // default sweep: m >= this +
 constexpr long long kSweepMinPerHaplotype = 4;         // this x n
-constexpr size_t kMaxSmemPerCta = 227 * 1024;
 
 struct SweepPlan {
     int nch, L, R, nstages, threads, started;
@@ -153,7 +152,7 @@ bool chunk_plan(int n_total, long long m, int mode, const selscan_launch *L, Swe
     // row's split into populations) and of the longest chunk (one CTA per SM)
     const int maxB = (int)(2 * m / device_sms() + 8);
     const size_t smem = chunk_smem_bytes(n_total, m, (n_total + 63) / 64 + 1, maxB, xp);
-    if (smem > kMaxSmemPerCta || (w->slot_bytes & 15) || (size_t)2 * m * w->slot_bytes > kChunkSlotBudget)
+    if (smem > kMaxSmemPerCta - kFixedSmem || (w->slot_bytes & 15) || (size_t)2 * m * w->slot_bytes > kChunkSlotBudget)
         return false;
     int per_sm = chunk_ctas_per_sm(n_total, m, smem, xp);
     if (per_sm < 1) per_sm = 1;

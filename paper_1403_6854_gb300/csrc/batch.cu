@@ -253,7 +253,7 @@ bool chunk_tick(const selscan_scan *scans, const BatchDesc *d, int nscans, const
         t.w[i].wscratch_bytes = per_warp;
     }
     o += (size_t)tasks * (size_t)nw * per_warp;
-    return o <= ws_bytes && smem <= 227 * 1024;
+    return o <= ws_bytes && smem <= kMaxSmemPerCta - kFixedSmem;
 }
 
 }  // namespace
@@ -385,8 +385,7 @@ int selscan_batch_run(const selscan_scan *scans, int32_t nscans, const int32_t *
     t.sc = plan.sc;
     t.head = (unsigned long long *)(ws + l.head);
     if (cudaMemsetAsync(ws + l.head, 0, 256, st) != cudaSuccess) return SELSCAN_ERR_CUDA;
-    if (cudaFuncSetAttribute(walk_batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)plan.smem) != cudaSuccess ||
+    if (allow_smem(walk_batch_kernel) != cudaSuccess ||
         cudaFuncSetAttribute(walk_batch_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
                              plan.carveout) != cudaSuccess)
         return SELSCAN_ERR_CUDA;

@@ -78,6 +78,18 @@ __host__ __device__ constexpr size_t scratch_per_warp(int n_total)
     return ((size_t)list_cap(n_total) * 8 + (size_t)table_cap(n_total) * 10 + 255) & ~(size_t)255;
 }
 
+// Lets `kernel` be launched with any dynamic shared memory a CTA can have.  The
+// limit belongs to the kernel, not to a launch: every thread and every size sets
+// the same one (with a limit of its own size, a call lowered it under another's
+// launch, which then failed).  `fixed`: room left for the kernel's static shared
+// memory.
+constexpr size_t kMaxSmemPerCta = 227 * 1024;
+constexpr size_t kFixedSmem = 1024;
+template <class K> inline cudaError_t allow_smem(K kernel, size_t fixed = 0)
+{
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kMaxSmemPerCta - fixed));
+}
+
 // kernel launchers (kernels.cu)
 cudaError_t launch_validate(const long long *pos, const double *gmap, long long m, int32_t *err,
                             cudaStream_t s, int check_map = 1);

@@ -189,8 +189,7 @@ cudaError_t launch_tick_words(const ChunkTick &t, cudaStream_t s)
     int W = 1;
     for (int i = 0; i < t.nscans; ++i) W = t.w[i].a.W > W ? t.w[i].a.W : W;
     const size_t smem = (size_t)32 * (W | 1) * 8;
-    const cudaError_t e = cudaFuncSetAttribute(tick_words_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)smem);
+    const cudaError_t e = allow_smem(tick_words_kernel);
     if (e != cudaSuccess) return e;
     tick_words_kernel<<<t.boff[t.nscans], 256, smem, s>>>(t);
     return cudaGetLastError();
@@ -201,8 +200,7 @@ cudaError_t launch_core_select_words(const ScanArgs &a, int mode, unsigned maf_n
                                      long long x1, unsigned *tw, cudaStream_t s)
 {
     const size_t smem = (size_t)32 * (a.W | 1) * 8;
-    const cudaError_t e = cudaFuncSetAttribute(core_select_words_kernel,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_smem(core_select_words_kernel);
     if (e != cudaSuccess) return e;
     const long long blocks = ((x1 - 1) >> 5) - (x0 >> 5) + 1;
     core_select_words_kernel<<<(unsigned)blocks, 256, smem, s>>>(a, mode, maf_num, maf_den, maf_filter, n1,
@@ -344,7 +342,7 @@ template <typename K>
 static int occupancy_of(K kernel, int warps_per_cta, size_t smem_bytes, bool carve)
 {
     int nb = 0;
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
+    allow_smem(kernel);
     if (carve) cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, warps_per_cta * 32, smem_bytes) !=
         cudaSuccess) {
@@ -391,8 +389,7 @@ static cudaError_t persistent_impl(const ScanArgs &a, const ItemSink &sk, const 
                                    long long n_cores, cudaStream_t s)
 {
     const size_t smem = slice_bytes(sc) * (size_t)wpc;
-    cudaError_t e = cudaFuncSetAttribute(walk_persistent_kernel<NPOP, MINB>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(walk_persistent_kernel<NPOP, MINB>);
     if (e != cudaSuccess) return e;
     // shared memory as large as the resident CTAs need; the rest stays L1
     e = cudaFuncSetAttribute(walk_persistent_kernel<NPOP, MINB>,
@@ -418,8 +415,7 @@ static cudaError_t walk_impl(const ScanArgs &a, const ItemSink &sk, const Scratc
     if (schedule == SELSCAN_SCHED_PLAIN) {
         const int ipc = NPOP == 2 ? 2 : 4;
         const size_t smem_p = slice_bytes(sc) * (size_t)ipc;
-        cudaError_t e = cudaFuncSetAttribute(walk_plain_kernel<NPOP>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_p);
+        cudaError_t e = allow_smem(walk_plain_kernel<NPOP>);
         if (e != cudaSuccess) return e;
         // `ctas` carries the number of scratch slots; the bitmap was reset by the caller
         walk_plain_kernel<NPOP><<<(unsigned)n_cores, ipc * 32, smem_p, s>>>(a, sk, sc, sk.slotmap,
@@ -436,8 +432,7 @@ static cudaError_t pass2_impl(const ScanArgs &a, const ItemSink &sk, const Scrat
                               int ctas, cudaStream_t s)
 {
     const size_t smem = slice_bytes(sc) * (size_t)wpc;
-    cudaError_t e = cudaFuncSetAttribute(walk_persistent_kernel<NPOP, MINB>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(walk_persistent_kernel<NPOP, MINB>);
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(walk_persistent_kernel<NPOP, MINB>,
                              cudaFuncAttributePreferredSharedMemoryCarveout, carveout_pct(smem, ctas));
@@ -589,8 +584,7 @@ cudaError_t launch_ehh(const ScanArgs &a, long long locus, const Scratch &sc,
                        cudaStream_t s)
 {
     const size_t smem = slice_bytes(sc) * 6;
-    cudaError_t e = cudaFuncSetAttribute(ehh_trace_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(ehh_trace_kernel);
     if (e != cudaSuccess) return e;
     ehh_trace_kernel<<<1, 192, smem, s>>>(a, locus, sc, S, cap, len, stop, status, ihh, denom, rest);
     return cudaGetLastError();

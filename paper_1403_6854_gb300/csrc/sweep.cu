@@ -1584,7 +1584,7 @@ int chunk_ctas_per_sm(int n, long long m, size_t smem, int xpehh)
     const ChunkShape c = chunk_shape(n, m);
     int per_sm = 0;
     const ChunkKernel k = xpehh ? c.xpehh : c.ihs;
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+    if (allow_smem(k, kFixedSmem) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, c.tc, smem) != cudaSuccess) {
         cudaGetLastError();
         return -1;
@@ -1602,7 +1602,7 @@ cudaError_t launch_chunk_scan(const SweepArgs &w0, cudaStream_t s)
     const size_t smem = chunk_smem_bytes(w.n, w.a.m, w.a.W, w.R, xp);
     w.split_off = chunk_split_off(w.n, w.a.W, c.ts, w.R);
     const ChunkKernel k = xp ? c.xpehh : c.ihs;
-    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_smem(k, kFixedSmem);
     if (e != cudaSuccess) return e;
     k<<<2 * w.nch, c.tc, smem, s>>>(sc);
     return cudaGetLastError();
@@ -1636,7 +1636,7 @@ cudaError_t launch_chunk_tick(const ChunkTick &t, int max_n, size_t smem, cudaSt
 {
     static_assert(sizeof(TickChunks) <= 32000, "tick parameter block too large");
     const TickShape c = tick_shape(max_n);
-    const cudaError_t e = cudaFuncSetAttribute(c.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_smem(c.kernel, kFixedSmem);
     if (e != cudaSuccess) return e;
     // static: the block is large, and the launch consumes it before this returns
     static thread_local TickChunks tc;
@@ -1650,7 +1650,7 @@ int split_walk_ctas(int n, int xpehh)
     // resident CTAs of the persistent walker
     int per_sm = 0;
     const size_t smem = split_smem_per_warp(n, xpehh) * kSplitWarps;
-    cudaFuncSetAttribute(walk_kernel_for<32>(xpehh), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    allow_smem(walk_kernel_for<32>(xpehh));
     const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
         &per_sm, walk_kernel_for<32>(xpehh), kSplitWarps * 32, smem);
     if (e != cudaSuccess || per_sm < 1) per_sm = 1;
@@ -1692,7 +1692,7 @@ static cudaError_t launch_start(const SweepArgs &w, cudaStream_t s)
     const int T = w.n <= 512 ? 128 : w.n <= 2048 ? 256 : 512;
     void (*start)(SweepArgs) = T == 128 ? start_kernel<128> : T == 256 ? start_kernel<256> : start_kernel<512>;
     const size_t smem = start_smem_bytes(w.n, T);
-    const cudaError_t e = cudaFuncSetAttribute(start, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_smem(start);
     if (e != cudaSuccess) return e;
     start<<<2 * w.nch, T, smem, s>>>(w);
     return cudaGetLastError();
@@ -1703,13 +1703,11 @@ cudaError_t launch_sweep_path(const SweepArgs &w0, cudaStream_t s)
     SweepArgs w = w0;
     const size_t ssm = sweep_smem_bytes(w.n, w.a.W, w.threads, w.R);
     void (*sweep)(SweepArgs) = sort_kernel(w.n, w.threads, w.a.nB > 0);
-    cudaError_t e = cudaFuncSetAttribute(sweep, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssm);
+    cudaError_t e = allow_smem(sweep);
     if (e != cudaSuccess) return e;
     const size_t wsm = (size_t)w.split_bytes * kSplitWarps;
     void (*walk)(SweepArgs) = walk_kernel_for<32>(w.a.nB > 0);
-    if ((e = cudaFuncSetAttribute(walk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wsm)) !=
-        cudaSuccess)
-        return e;
+    if ((e = allow_smem(walk)) != cudaSuccess) return e;
     if (w.started && (e = launch_start(w, s)) != cudaSuccess) return e;
     for (int st = 0; st < w.nstages; ++st) {
         w.stage = st;
@@ -1858,12 +1856,10 @@ cudaError_t launch_report(const ReportArgs &r, cudaStream_t s)
     if (e != cudaSuccess) return e;
     void (*sweep)(SweepArgs) = sort_kernel(w.n, w.threads, w.a.nB > 0);
     const size_t ssm = sweep_smem_bytes(w.n, w.a.W, w.threads, 1);
-    if ((e = cudaFuncSetAttribute(sweep, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssm)) != cudaSuccess)
-        return e;
+    if ((e = allow_smem(sweep)) != cudaSuccess) return e;
     sweep<<<2, w.threads, ssm, s>>>(w);
     const size_t wsm = (size_t)w.split_bytes * kSplitWarps;
-    if ((e = cudaFuncSetAttribute(report_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wsm)) != cudaSuccess)
-        return e;
+    if ((e = allow_smem(report_kernel, kFixedSmem)) != cudaSuccess) return e;
     report_kernel<<<dim3(kReportSteps / 32 / kSplitWarps, 2), kSplitWarps * 32, wsm, s>>>(r);
     return cudaGetLastError();
 }
