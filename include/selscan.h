@@ -68,7 +68,7 @@ extern "C" {
 #define SELSCAN_OK                 0
 #define SELSCAN_ERR_INVALID_ARG   -1  /* null pointer, n < 2, m < 1, bad rational, ld < W, limits */
 #define SELSCAN_ERR_UNSORTED      -2  /* (device error word) positions or map decrease */
-#define SELSCAN_ERR_WORKSPACE     -3  /* ws_bytes < selscan_workspace_bytes(...) */
+#define SELSCAN_ERR_WORKSPACE     -3  /* ws_bytes too small (selscan_workspace_min_bytes) */
 #define SELSCAN_ERR_CUDA          -4  /* a kernel launch or CUDA runtime call failed */
 #define SELSCAN_ERR_TIMEOUT       -5  /* (device error word) a bounded device wait gave up */
 #define SELSCAN_ERR_UNSUPPORTED   -6  /* no sm_103a device, or a launch shape it cannot run */
@@ -208,6 +208,14 @@ void selscan_default_params(selscan_params *p);
  * The workspace must be 256-byte aligned. */
 size_t selscan_workspace_bytes(int32_t n_total, int64_t m, int32_t mode,
                                const selscan_launch *launch);
+
+/* The least workspace bytes that such a call surely runs in: a workspace sized
+ * for another shape may have room for no more than the forms that need less
+ * (the in-order scan and the single-locus report step by step, the sweep with
+ * its chunks' histories swept marker by marker), whose results are the same
+ * and which take longer. */
+size_t selscan_workspace_min_bytes(int32_t n_total, int64_t m, int32_t mode,
+                                   const selscan_launch *launch);
 
 /* iHS at every marker (Eq. 3, Eq. 4, Section 1.2).  hap/pos/gmap: device
  * inputs as described above; out: device outputs of length m. */

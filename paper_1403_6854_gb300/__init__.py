@@ -77,7 +77,8 @@ class selscan_scan(ctypes.Structure):
                 ("error", _P), ("items", _P)]
 
 
-EXPORTS = ("selscan_default_params", "selscan_workspace_bytes", "selscan_ihs", "selscan_xpehh",
+EXPORTS = ("selscan_default_params", "selscan_workspace_bytes", "selscan_workspace_min_bytes",
+           "selscan_ihs", "selscan_xpehh",
            "selscan_ihs_range", "selscan_xpehh_range", "selscan_normalize_bin_sums",
            "selscan_normalize_finish", "selscan_normalize_apply",
            "selscan_ehh", "selscan_ehh_noalloc", "selscan_pack", "selscan_strerror",
@@ -104,6 +105,8 @@ def load_library():
     lib.selscan_workspace_bytes.restype = ctypes.c_size_t
     lib.selscan_workspace_bytes.argtypes = [ctypes.c_int32, ctypes.c_int64, ctypes.c_int32,
                                             ctypes.POINTER(selscan_launch)]
+    lib.selscan_workspace_min_bytes.restype = ctypes.c_size_t
+    lib.selscan_workspace_min_bytes.argtypes = lib.selscan_workspace_bytes.argtypes
     lib.selscan_ihs.restype = ctypes.c_int
     lib.selscan_ihs.argtypes = [_P, ctypes.c_int64, ctypes.c_int32, ctypes.c_int64, _P, _P,
                                 ctypes.POINTER(selscan_params), ctypes.POINTER(selscan_ihs_out),
@@ -346,6 +349,14 @@ def selscan_workspace_bytes(n_total: int, m: int, mode: int,
                                            ctypes.byref(launch) if launch is not None else None))
 
 
+def selscan_workspace_min_bytes(n_total: int, m: int, mode: int,
+                                launch: Optional[selscan_launch] = None) -> int:
+    """The least workspace that a call runs in (selscan_workspace_bytes: the one in
+    which it is fastest)."""
+    return int(load_library().selscan_workspace_min_bytes(
+        n_total, m, mode, ctypes.byref(launch) if launch is not None else None))
+
+
 def _ptr(t: Optional[torch.Tensor]):
     return None if t is None else ctypes.c_void_p(t.data_ptr())
 
@@ -366,15 +377,9 @@ def _workspace(nbytes: int, device, workspace: Optional[torch.Tensor]):
 
 
 def _scan_workspace(n: int, k: int, mode: int, launch, device, workspace: Optional[torch.Tensor]):
-    need = selscan_workspace_bytes(n, k, mode, launch)
-    if workspace is not None:
-        # an in-order scan also runs step by step, in less
-        step = selscan_launch.from_buffer_copy(launch) if launch is not None else selscan_launch()
-        if launch is None:
-            step.schedule = SCHED_DEFAULT
-        step.warps_per_cta = step.warps_per_cta or 8
-        need = min(need, selscan_workspace_bytes(n, k, mode, step))
-    return _workspace(need, device, workspace)
+    # a workspace that is passed may have been sized for another shape
+    size = selscan_workspace_bytes if workspace is None else selscan_workspace_min_bytes
+    return _workspace(size(n, k, mode, launch), device, workspace)
 
 
 def _as_rows(hap: torch.Tensor) -> torch.Tensor:
@@ -494,7 +499,7 @@ def selscan_ehh(hap: torch.Tensor, n: int, pos: torch.Tensor, gmap: torch.Tensor
                denom=torch.empty(3, dtype=torch.int64, device=dev),
                error=torch.zeros(1, dtype=torch.int32, device=dev))
     p = params if params is not None else selscan_default_params()
-    ws = _workspace(selscan_workspace_bytes(n, m, MODE_EHH, None), dev, workspace)
+    ws = _scan_workspace(n, m, MODE_EHH, None, dev, workspace)
     o = selscan_ehh_out(*(_ptr(out[f]) if out[f].numel() else None
                           for f in ("S", "len", "stop", "status", "ihh", "denom", "error")))
     rc = lib.selscan_ehh(_ptr(hap), ld, n, m, _ptr(pos), _ptr(gmap), locus, ctypes.byref(p),

@@ -606,6 +606,20 @@ size_t selscan_workspace_bytes(int32_t n_total, int64_t m, int32_t mode, const s
     return mode == SELSCAN_MODE_EHH ? report_layout(n_total, total).total : total;
 }
 
+size_t selscan_workspace_min_bytes(int32_t n_total, int64_t m, int32_t mode, const selscan_launch *launch)
+{
+    const size_t full = selscan_workspace_bytes(n_total, m, mode, launch);
+    if (full == 0) return 0;
+    // the layouts that run_scan and selscan_ehh fall back to
+    const Plan p = make_plan(mode, (n_total + 63) / 64, launch, n_total, m);
+    const int nslots = mode == SELSCAN_MODE_EHH ? p.nslots : device_sms() * 64;
+    const bool sweep = p.schedule == SELSCAN_SCHED_SWEEP;
+    SweepPlan sw;
+    if (sweep) sw = make_sweep_plan(n_total, m, mode, launch, false);
+    const size_t least = make_layout(n_total, m, mode, nslots, sweep ? &sw : nullptr).total;
+    return least < full ? least : full;
+}
+
 int32_t selscan_default_schedule(int32_t n_total, int64_t m, int32_t mode)
 {
     if (n_total < 2 || m < 1 || (mode != SELSCAN_MODE_IHS && mode != SELSCAN_MODE_XPEHH)) return -1;
