@@ -161,26 +161,31 @@ BatchDesc make_desc(const selscan_scan *s)
     return d;
 }
 
-// A tick whose scans all have at most 65,000 markers (16-bit run lengths span the
-// whole arm) and 6,144 haplotypes, and whose chunks' slots, states and words fit
-// the tick's workspace, sorts and walks chunks of its core ranges
-// (chunk_scan_kernel) instead of walking every step (six scans of 100 to 1,000
-// haplotypes x about 10,000 markers: 24.0 -> 2.0 ms).  Chunks: one task per
-// resident CTA, of at least 16 cores; a short chunk costs as much for its
-// starting state as for its cores (twice as many tasks: 2.7 ms).  Fills t; false: take the per-step walk.
+// A tick whose scans (those with cores in it) all have at most 65,000 markers
+// (16-bit run lengths span the whole arm) and 6,144 haplotypes, and whose chunks'
+// slots, states and words fit the tick's workspace, sorts and walks chunks of its
+// core ranges (chunk_scan_kernel) instead of walking every step (six scans of 100
+// to 1,000 haplotypes x about 10,000 markers: 24.0 -> 1.7 ms).  Chunks: one task
+// per resident CTA, of at least 16 cores; a short chunk costs as much for its
+// starting state as for its cores (twice as many tasks: 2.7 ms).  Fills t; false:
+// take the per-step walk.
 bool chunk_tick(const selscan_scan *scans, const BatchDesc *d, int nscans, const int32_t *unit_scan,
                 const int64_t *unit_c0, const int64_t *unit_c1, int nunits, unsigned char *ws, size_t ws_bytes,
                 ChunkTick &t, int &max_n, size_t &smem, size_t &head_bytes)
 {
     max_n = 0;
-    long long cores = 0;
+    long long cores = 0, of_scan[SELSCAN_BATCH_MAX_SCANS] = {0};   // the tick's cores; 0: no part in it
+    for (int u = 0; u < nunits; ++u) {
+        cores += unit_c1[u] - unit_c0[u];
+        of_scan[unit_scan[u]] += unit_c1[u] - unit_c0[u];
+    }
+    if (cores < 1) return false;
     for (int i = 0; i < nscans; ++i) {
+        if (of_scan[i] == 0) continue;
         const int n = d[i].a.nA + d[i].a.nB;
         if (n > kChunkMaxN || d[i].a.m > 65000) return false;
         max_n = n > max_n ? n : max_n;
     }
-    for (int u = 0; u < nunits; ++u) cores += unit_c1[u] - unit_c0[u];
-    if (cores < 1) return false;
     const int ts = tick_sort_threads(max_n), nw = tick_warps(max_n);
     const long long want = (long long)tick_ctas(max_n) * device_sms();
     long long B = (2 * cores + want - 1) / want;
@@ -210,6 +215,8 @@ bool chunk_tick(const selscan_scan *scans, const BatchDesc *d, int nscans, const
     for (int i = 0; i < nscans; ++i) {
         SweepArgs &w = t.w[i];
         memset(&w, 0, sizeof(w));
+        t.boff[i] = blocks;
+        if (of_scan[i] == 0) continue;       // no unit: no words, no room
         w.a = d[i].a;
         w.sk = d[i].sk;
         w.n = d[i].a.nA + d[i].a.nB;
@@ -237,7 +244,6 @@ bool chunk_tick(const selscan_scan *scans, const BatchDesc *d, int nscans, const
         smem = sm > smem ? sm : smem;
         split_off = so > split_off ? so : split_off;
         split_bytes = w.split_bytes > split_bytes ? w.split_bytes : split_bytes;
-        t.boff[i] = blocks;
         blocks += (int)((w.a.m + 31) / 32);
     }
     t.boff[nscans] = blocks;

@@ -187,7 +187,7 @@ __global__ void __launch_bounds__(256) tick_words_kernel(const __grid_constant__
 cudaError_t launch_tick_words(const ChunkTick &t, cudaStream_t s)
 {
     int W = 1;
-    for (int i = 0; i < t.nscans; ++i) W = t.w[i].a.W > W ? t.w[i].a.W : W;
+    for (int i = 0; i < t.nscans; ++i) W = t.w[i].a.W > W ? t.w[i].a.W : W;     // 0: no part in the tick
     const size_t smem = (size_t)32 * (W | 1) * 8;
     const cudaError_t e = allow_smem(tick_words_kernel);
     if (e != cudaSuccess) return e;
