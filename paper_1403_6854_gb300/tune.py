@@ -1,9 +1,9 @@
 """Autotuner for the walk kernels' launch shape.
 
 The shape changes how the walks run, never their results.  Samples of up to
-16383 haplotypes use the sorted sweep: its cost depends on the chromosome's
-length (chunking, warm-up, walks that outrun a chunk's history), so its few
-candidates are timed on the whole scan.  Larger samples use the per-step
+16383 haplotypes use the sorted forms: their cost depends on the chromosome's
+length (chunking, warm-up, walks that outrun a chunk's history), so the few
+candidates, the default launch's form among them, are timed on the whole scan.  Larger samples use the per-step
 schedules (warps per CTA, on-chip group words per warp, rows per TMA window
 buffer, cores per queue fetch), timed on a prefix of the scan (the first
 `sample_markers` markers, a view, no copy).  Timing is CUDA events around
@@ -24,6 +24,7 @@ SHAPE_FIELDS = ("schedule", "warps_per_cta", "smem_entries", "window_rows", "cor
 
 SWEEP_MAX_N = 16383
 SWEEP_CANDIDATES: List[Dict] = [
+    dict(schedule=1),                           # a default launch's choice for short chromosomes
     dict(schedule=1, warps_per_cta=4),          # per-step in-order
     dict(schedule=3),
     dict(schedule=3, sweep_warmup=2048),        # shorter histories: less to sort, more walks
