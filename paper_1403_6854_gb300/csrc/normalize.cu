@@ -6,16 +6,17 @@
 // segment s of the markers once; each of its threads adds its markers (thread
 // stride) into its own per-bin accumulators in shared memory, then one thread
 // per bin adds the threads' values (from thread b on, so that the threads read
-// distinct banks).  More bins: CTA (b, s) sums bin b over segment s (thread
-// stride, then a fixed tree).  Either way the CTA that finishes last adds the
-// segments (first the last CTA of each dozen those of its dozen) and, for a whole
-// standardisation, makes the bin's mean or SD.  FP64 additions are slow here (two
-// lanes per SM cycle, some hundred cycles for a dependent one), so every sum is
-// short or runs in several chains.  Every order is fixed, so
-// the results are the same whichever CTA is last.  Two passes: the mean, then the
-// sum of squared deviations about it (no cancellation of E[x^2] - E[x]^2).  Three
-// launches; with one kernel per step there were seven, and one thread per bin
-// added 304 segments one after the other (1M scores, 100 bins: 0.142 ms).
+// distinct banks), and the CTA that finishes last adds the segments (first the
+// last CTA of each dozen those of its dozen) and, for a whole standardisation,
+// makes the bin's mean or SD: three launches (one kernel per step took seven, and
+// one thread per bin added 304 segments one after the other; 1M scores, 100 bins:
+// 0.142 ms, now 0.078).  More bins: CTA (b, s) sums bin b over segment s (thread
+// stride, then a fixed tree), and a second launch adds the segments.  FP64
+// additions are slow here (two lanes per SM cycle, some hundred cycles for a
+// dependent one), so every sum is short or runs in several chains.  Every order
+// is fixed (the segments' number too, whatever the GPU), so the results are the
+// same whichever CTA is last.  Two passes: the mean, then the sum of squared
+// deviations about it (no cancellation of E[x^2] - E[x]^2).
 #include <limits.h>
 #include <math.h>
 
@@ -113,11 +114,11 @@ __device__ __forceinline__ void sum_parts(int nbins, int pass, int b, int q0, in
     c = k[0];
 }
 
-// The totals of bin b, from its parts [q0, q1).
-__device__ __forceinline__ void put_totals(int nbins, int pass, int q0, int q1, const double *part_sum,
-                                           const long long *part_cnt, const BinOut &out)
+// The totals of the bins first, first + step, ..., from their parts [q0, q1).
+__device__ __forceinline__ void put_totals(int first, int step, int nbins, int pass, int q0, int q1,
+                                           const double *part_sum, const long long *part_cnt, const BinOut &out)
 {
-    for (int b = threadIdx.x; b < nbins; b += blockDim.x) {
+    for (int b = first; b < nbins; b += step) {
         double s;
         long long c;
         sum_parts(nbins, pass, b, q0, q1, part_sum, part_cnt, s, c);
@@ -140,7 +141,7 @@ __device__ __forceinline__ void bin_interval(int b, int n, int nbins, long long 
 // pass 0: count and sum per (bin, segment); pass 1: squared deviations about mean[bin]
 __global__ void __launch_bounds__(kNormThreads) norm_partial_kernel(
     const double *score, const int8_t *status, const int32_t *n1, long long m, int n, int nbins,
-    int pass, const double *mean, double *part_sum, long long *part_cnt, BinOut out)
+    int pass, const double *mean, double *part_sum, long long *part_cnt)
 {
     __shared__ double red_d[kNormThreads / 32];
     __shared__ long long red_c[kNormThreads / 32];
@@ -166,12 +167,22 @@ __global__ void __launch_bounds__(kNormThreads) norm_partial_kernel(
         part_sum[(size_t)seg * nbins + b] = s;
         if (pass == 0) part_cnt[(size_t)seg * nbins + b] = c;
     }
+}
+
+// The totals of every bin from its segments, after norm_partial_kernel.  A launch
+// of its own: there are 16 CTAs a bin, and a tally in each of them cost more than
+// it saved (1,024 bins, 1,000 scores, whole call: 0.242 ms against 0.159).
+__global__ void __launch_bounds__(32) norm_totals_kernel(int nbins, int pass, const double *part_sum,
+                                                         const long long *part_cnt, BinOut out)
+{
     static_assert(kNormSegments <= 16, "one sum of the parts");
-    if (last_of(out.done, gridDim.x)) put_totals(nbins, pass, 0, kNormSegments, part_sum, part_cnt, out);
+    put_totals(blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, nbins, pass, 0, kNormSegments, part_sum,
+               part_cnt, out);
 }
 
 // pass 0: count and sum per (segment, bin); pass 1: squared deviations about
-// mean[bin].  Shared memory: sums [nbins][64] (double), counts [nbins][64].
+// mean[bin].  Shared memory: sums [nbins + 1][128] (double), counts [nbins + 1][128]
+// (the last row takes the markers that count in no bin).
 __global__ void __launch_bounds__(kNormPrivThreads) norm_partial_private_kernel(
     const double *score, const int8_t *status, const int32_t *n1, long long m, int n, int nbins,
     int pass, const double *mean, double *part_sum, long long *part_cnt, BinOut out)
@@ -264,7 +275,8 @@ __global__ void __launch_bounds__(kNormPrivThreads) norm_partial_private_kernel(
         if (pass == 0) part_cnt[(size_t)(kNormPrivSegments + dz) * nbins + b] = c;
     }
     if (last_of(out.done, kNormDozens))
-        put_totals(nbins, pass, kNormPrivSegments, kNormPrivSegments + kNormDozens, part_sum, part_cnt, out);
+        put_totals(t, kNormPrivThreads, nbins, pass, kNormPrivSegments, kNormPrivSegments + kNormDozens, part_sum,
+                   part_cnt, out);
 }
 
 // Mean (pass 0) or sample SD (pass 1) of each bin from its totals.
@@ -378,7 +390,8 @@ void launch_bin_sums(const double *score, const int8_t *status, const int32_t *n
     } else {
         const unsigned grid = (unsigned)(nbins * kNormSegments);
         norm_partial_kernel<<<grid, kNormThreads, 0, s>>>(score, status, n1, m, n, nbins, pass,
-                                                          bin_mean, part_sum, part_cnt, out);
+                                                          bin_mean, part_sum, part_cnt);
+        norm_totals_kernel<<<(nbins + 31) / 32, 32, 0, s>>>(nbins, pass, part_sum, part_cnt, out);
     }
 }
 
