@@ -295,7 +295,7 @@ ReportLayout report_layout(int n, size_t from)
     ReportLayout l;
     memset(&l, 0, sizeof(l));
     l.total = from;
-    l.on = start_smem_bytes(n, 512) <= kMaxSmemPerCta;
+    l.on = report_start_smem(n, 512) <= kMaxSmemPerCta;
     if (!l.on) return l;
     l.threads = n <= 1024 ? 128 : n <= 6144 ? 256 : 512;
     size_t o = up256(from);
@@ -467,6 +467,7 @@ int run_scan(int mode, const uint64_t *hap, int64_t ld, int32_t nA, int32_t nB, 
         w.walk_ctas = plan.sw.walk_ctas;
         w.walk_head = (unsigned long long *)(ws + l.sweep_head);
         w.err = err;
+        w.quit = nullptr;
         w.sweep_done_event = launch ? launch->sweep_done_event : nullptr;
         w.heads = (unsigned *)(ws + l.heads);
         if ((sweep ? launch_sweep_path(w, s) : launch_chunk_scan(w, s)) != cudaSuccess) return SELSCAN_ERR_CUDA;
@@ -559,12 +560,15 @@ int ehh_run(const ScanArgs &a, int64_t locus, const selscan_params *p, const Scr
         r.S = (unsigned *)(ws + l.S);
         r.done = (unsigned *)(ws + l.ctl + 8);
         r.rest = (int *)(ws + l.ctl + 16);
+        r.walked = (int *)(ws + l.ctl + 48);
+        r.started = (int *)(ws + l.ctl + 64);
+        w.quit = r.walked;
         rest = r.rest;
         // the words of the locus' surroundings (its count and status go to the control block)
         if (cudaMemsetAsync(ws + l.ctl, 0, 256, s) != cudaSuccess ||
             launch_core_select_words(w.a, 0, 0, 1, 0, at_core((int32_t *)(ws + l.ctl + 192), locus),
                                      w.sk.core_status, x0, x1, (unsigned *)(ws + l.words), s) != cudaSuccess ||
-            launch_report(r, s) != cudaSuccess)
+            launch_report(r, sc, s) != cudaSuccess)
             return SELSCAN_ERR_CUDA;
     }
     if (launch_ehh(a, locus, sc, (unsigned long long *)out->S, capacity, (long long *)out->len,

@@ -95,4 +95,41 @@ __device__ __forceinline__ bool run_item(const ScanArgs &a, const ItemSink &sk, 
     return go_on;
 }
 
+// Walk q of a single-locus report (walk q / 2, direction q % 2) by one warp, with
+// its results, the traces at S + q cap; the first walk's warp makes the
+// denominators.  False if `quit` ended it (no results then).
+template <class Quit = NeverQuit>
+__device__ __forceinline__ bool trace_walk(const ScanArgs &a, long long locus, const Scratch &sc, unsigned char *slice,
+                                           int q, unsigned long long *S, long long cap, long long *len, int32_t *stop,
+                                           int8_t *status, double *ihh, unsigned long long *denom, Quit quit = Quit())
+{
+    const int lane = threadIdx.x & 31;
+    WarpBufs b = make_bufs(slice, sc.base + (size_t)q * sc.per_warp, sc);
+    init_window(b);
+    unsigned wpar[2] = {0u, 0u};
+    const int w = q >> 1, dir = q & 1;
+    const WalkOut o = walk<1>(a, locus, dir, w, b, S + (size_t)q * cap, cap, 0, wpar, quit);
+    if (q == 0 && lane == 0) {
+        // denominators from the core row
+        const unsigned int *row = (const unsigned int *)(a.hap + locus * a.ld);
+        unsigned long long c1 = 0;
+        for (int k = 0; k < 2 * a.W; ++k) c1 += (unsigned long long)__popc(row[k] & valid32(a, k));
+        const unsigned long long n = (unsigned long long)a.nA;
+        denom[0] = choose2(c1);
+        denom[1] = choose2(n - c1);
+        denom[2] = choose2(n);
+    }
+    if (o.status == WALK_UNFINISHED) return false;
+    if (lane == 0) {
+        long long steps = 0;
+        if (o.status == WALK_OK) steps = o.stop + 1;
+        else if (o.status == WALK_EDGE || o.status == WALK_GAP) steps = o.stop;
+        len[q] = steps;
+        stop[q] = o.stop;
+        status[q] = (int8_t)o.status;
+        ihh[q] = o.ihh[0];
+    }
+    return true;
+}
+
 }  // namespace selscan

@@ -170,6 +170,7 @@ struct SweepArgs {
     unsigned *heads;                 // one-launch scans: next slot of each chunk (0: not sorted yet)
     int32_t *err;                    // device error word of the call
     void *sweep_done_event;          // optional event after the first stage's sort
+    const int *quit;                 // report: walks done step by step, all six end the sort (else null)
 };
 
 // One tick of batched scans, chunk by chunk: the scans' arguments (slots, state
@@ -196,7 +197,7 @@ size_t sweep_smem_bytes(int n, int W, int T, int R);
 size_t sweep_slot_bytes(int n, int xpehh);
 size_t sweep_state_bytes(int n, int T);
 __host__ __device__ size_t sweep_elements(int n, int T);     // sorted elements of one CTA (n and its padding)
-size_t start_smem_bytes(int n, int T);   // shared memory of a starting state's sort
+__host__ __device__ size_t start_smem_bytes(int n, int T);   // shared memory of a starting state's sort
 size_t split_smem_per_warp(int n, int xpehh);
 size_t split_scratch_per_warp(int n);
 int split_walk_ctas(int n, int xpehh);
@@ -209,9 +210,12 @@ struct ReportArgs {
     long long capacity;
     unsigned *S;                     // [2 directions][class 0, 1][kReportSteps]: S of steps 1 ..
     unsigned *done;                  // zero
-    int *rest;                       // [6] 1: the walk outlived the history
+    int *walked;                     // zero: walks done step by step
+    int *started;                    // zero: starting states done
+    int *rest;                       // [6], zero; 1: the walk outlived the history
 };
-cudaError_t launch_report(const ReportArgs &r, cudaStream_t s);
+size_t report_start_smem(int n, int T);   // shared memory of its starting state
+cudaError_t launch_report(const ReportArgs &r, const Scratch &sc, cudaStream_t s);
 // short scans in one launch (chunk_scan_kernel)
 constexpr int kChunkMaxN = 6144;     // 256 threads x 24 haplotypes
 int chunk_sort_threads(int n, long long m);      // threads that sort a chunk

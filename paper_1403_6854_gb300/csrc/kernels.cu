@@ -548,34 +548,9 @@ __global__ void __launch_bounds__(192) ehh_trace_kernel(ScanArgs a, long long lo
                                                         unsigned long long *denom, const int *rest)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    const int lane = threadIdx.x & 31;
-    const int q = threadIdx.x >> 5;           // walk w = q / 2, direction q % 2
-    if (rest && rest[q] == 0) return;         // done from the sorted state (warps do not meet)
-    WarpBufs b = make_bufs(smem + (size_t)q * slice_bytes(sc),
-                           sc.base + (size_t)q * sc.per_warp, sc);
-    init_window(b);
-    unsigned wpar[2] = {0u, 0u};
-    const int w = q >> 1, dir = q & 1;
-    WalkOut o = walk<1>(a, locus, dir, w, b, S + (size_t)q * cap, cap, 0, wpar);
-    if (lane == 0) {
-        long long steps = 0;
-        if (o.status == WALK_OK) steps = o.stop + 1;
-        else if (o.status == WALK_EDGE || o.status == WALK_GAP) steps = o.stop;
-        len[q] = steps;
-        stop[q] = o.stop;
-        status[q] = (int8_t)o.status;
-        ihh[q] = o.ihh[0];
-    }
-    if (q == 0 && lane == 0) {
-        // denominators from the core row
-        const unsigned int *row = (const unsigned int *)(a.hap + locus * a.ld);
-        unsigned long long c1 = 0;
-        for (int k = 0; k < 2 * a.W; ++k) c1 += (unsigned long long)__popc(row[k] & valid32(a, k));
-        const unsigned long long n = (unsigned long long)a.nA;
-        denom[0] = choose2(c1);
-        denom[1] = choose2(n - c1);
-        denom[2] = choose2(n);
-    }
+    const int q = threadIdx.x >> 5;
+    if (rest && rest[q] == 0) return;         // done before (warps do not meet)
+    trace_walk(a, locus, sc, smem + (size_t)q * slice_bytes(sc), q, S, cap, len, stop, status, ihh, denom);
 }
 
 cudaError_t launch_ehh(const ScanArgs &a, long long locus, const Scratch &sc,

@@ -437,6 +437,7 @@ template <int T, int EMAX, bool EXACT = false, int XP = -1>
 __global__ void __launch_bounds__(T, T == 512 ? 2 : (T == 256 ? 3 : 512 / T)) sweep_kernel(SweepArgs w)
 {
     extern __shared__ __align__(16) unsigned char smem[];
+    if (w.quit && *w.quit >= 6) return;
     if (blockIdx.x == 0 && threadIdx.x == 0) *w.walk_head = 0ull;   // the next walk launch's slot counter
     const int dir = blockIdx.x / w.nch, c = blockIdx.x % w.nch;
     const long long c0 = w.a.k0 + (long long)c * w.B;   // chunk c of [k0, k1)
@@ -1078,13 +1079,15 @@ static void (*walk_kernel_for(int xpehh))(SweepArgs)
 // Shared memory per haplotype: element (bit index | group start << 16) and
 // group (at its start: end | word level << 16) twice, the prefix sums, and the
 // level at which each boundary arose.
-size_t start_smem_bytes(int n, int T) { return (size_t)n * 22 + 8 + (size_t)(T / 32) * 4; }
+__host__ __device__ size_t start_smem_bytes(int n, int T) { return (size_t)n * 22 + 8 + (size_t)(T / 32) * 4; }
 
 namespace {
 
-template <int T>
-__device__ void start_state(const SweepArgs &w, unsigned char *smem, int dir, long long c0, long long c1,
-                            unsigned *st, int np)
+// QUIT: looked at once a round, w.quit ends it without a state (then false);
+// `quitting` is a word of shared memory of its own, zero.
+template <int T, bool QUIT = false>
+__device__ bool start_state(const SweepArgs &w, unsigned char *smem, int dir, long long c0, long long c1,
+                            unsigned *st, int np, volatile int *quitting = nullptr)
 {
     const int n = w.n, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     unsigned *el = (unsigned *)smem;             // [2][n]
@@ -1142,7 +1145,9 @@ __device__ void start_state(const SweepArgs &w, unsigned char *smem, int dir, lo
     __syncthreads();
     int cur = 0;
     int na = nlev > 0 && n > 1 ? n : 0;          // elements in unresolved groups
+    constexpr unsigned kQuit = 1u << 30;         // far above any count of elements
     while (na > few) {
+        const int walked = QUIT && tid == 0 ? *(const volatile int *)w.quit : 0;   // used at the round's end
         const unsigned *elc = el + cur * n, *ifc = inf + cur * n;
         // pass 1: this segment's elements below (low half) / equal to (high
         // half) their group's pivot, counted exclusively into pre
@@ -1203,7 +1208,9 @@ __device__ void start_state(const SweepArgs &w, unsigned char *smem, int dir, lo
                 if (g2 != g) bw[g2] = (unsigned short)l;
             }
         }
+        if (QUIT && walked >= 6) left += kQuit;
         block_prefix(left);
+        if (QUIT && total >= kQuit) return false;
         na = (int)total;
         cur ^= 1;
     }
@@ -1250,6 +1257,7 @@ __device__ void start_state(const SweepArgs &w, unsigned char *smem, int dir, lo
         bool more = true;
         __syncthreads();
         while (more) {
+            const int walked = QUIT && tid == 0 ? *(const volatile int *)w.quit : 0;
             unsigned v[EC], f[EC], d[EC];
             unsigned cnt = 0u;
 #pragma unroll
@@ -1309,7 +1317,11 @@ __device__ void start_state(const SweepArgs &w, unsigned char *smem, int dir, lo
                     if (g2 != g) bw[ap[g2]] = (unsigned short)l;
                 }
             }
+            // every thread has read `quitting` of the last round: block_prefix's
+            // barriers lie between
+            if (QUIT && walked >= 6) *quitting = 1;
             more = __syncthreads_or(left) != 0;
+            if (QUIT && *quitting) return false;
         }
     }
     // run lengths: neighbours of one group share the whole history, others part
@@ -1338,6 +1350,7 @@ __device__ void start_state(const SweepArgs &w, unsigned char *smem, int dir, lo
         }
         st[p] = bi | (M << 16);
     }
+    return true;
 }
 
 }  // namespace
@@ -1686,10 +1699,12 @@ static void (*sort_kernel(int n, int threads, bool xpehh))(SweepArgs)
     return E <= 8 ? sweep_kernel<32, 8> : E <= 16 ? sweep_kernel<32, 16> : sweep_kernel<32, 32>;
 }
 
+// narrow CTAs for small samples: a round is a few elements per thread
+static int start_threads(int n) { return n <= 512 ? 128 : n <= 2048 ? 256 : 512; }
+
 static cudaError_t launch_start(const SweepArgs &w, cudaStream_t s)
 {
-    // narrow CTAs for small samples: a round is a few elements per thread
-    const int T = w.n <= 512 ? 128 : w.n <= 2048 ? 256 : 512;
+    const int T = start_threads(w.n);
     void (*start)(SweepArgs) = T == 128 ? start_kernel<128> : T == 256 ? start_kernel<256> : start_kernel<512>;
     const size_t smem = start_smem_bytes(w.n, T);
     const cudaError_t e = allow_smem(start);
@@ -1731,6 +1746,55 @@ cudaError_t launch_sweep_path(const SweepArgs &w0, cudaStream_t s)
 // A walk that outlives the history is left to the per-step kernel (rest[q] = 1).
 // Bound by the chain of launches and rounds, not by a step at a time (204
 // haplotypes, 22,147 markers, a locus in a sweep: 269 us by the per-step kernel).
+//
+// How long the walks are shows only while they run, and walks of a dozen or two
+// steps are done step by step before the starting states are (2,000 haplotypes, 80
+// founders: 107 us step by step, 281 sorted; in a sweep 2,975 and 380).  So the two
+// CTAs of the starting states run beside the six per-step walks, whichever is done
+// first ends the other, and the results are the same (130 and 312 us).  Neither
+// waits for the other: each looks at a counter as it goes.
+struct QuitWhenStarted {
+    const volatile int *started;
+    // answer with the look of a step ago: its load holds nothing up, and the step
+    // may be the last (5,000 haplotypes, 10 steps: 226 us against 369); not where a
+    // step takes 60 us (10,000: 1,000 us against 830)
+    bool late;
+    int seen;
+    __device__ __forceinline__ bool operator()()
+    {
+        const int before = seen;
+        seen = *started;
+        return __shfl_sync(FULLMASK, late ? before : seen, 0) >= 2;
+    }
+};
+
+// where the word that start_state<T, true> quits by lies
+static __host__ __device__ size_t report_quit_at(int n, int T) { return (start_smem_bytes(n, T) + 15) & ~(size_t)15; }
+size_t report_start_smem(int n, int T) { return report_quit_at(n, T) + 16; }
+
+template <int T>
+__global__ void __launch_bounds__(T, 1) report_start_kernel(ReportArgs r, Scratch sc)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    const SweepArgs &w = r.w;
+    if (blockIdx.x < 2) {
+        volatile int *quitting = (volatile int *)(smem + report_quit_at(w.n, T));
+        if (threadIdx.x == 0) *quitting = 0;
+        __syncthreads();
+        const int np = (int)sweep_elements(w.n, w.threads);
+        if (!start_state<T, true>(w, smem, blockIdx.x, w.a.k0, w.a.k1, (unsigned *)w.st + (size_t)blockIdx.x * np, np,
+                                  quitting))
+            return;
+        if (threadIdx.x == 0) atomicAdd(r.started, 1);
+        return;
+    }
+    const int q = (int)(blockIdx.x - 2) * (T / 32) + (int)(threadIdx.x >> 5);
+    if (q >= 6) return;
+    const bool done = trace_walk(w.a, w.a.k0, sc, smem + (size_t)(threadIdx.x >> 5) * slice_bytes(sc), q,
+                                 (unsigned long long *)r.out.S, r.capacity, (long long *)r.out.len, r.out.stop, r.out.status,
+                                 r.out.ihh, (unsigned long long *)r.out.denom, QuitWhenStarted{r.started, w.n <= 6144, 0});
+    if (done && (threadIdx.x & 31) == 0) atomicAdd(r.walked, 1);
+}
 __global__ void __launch_bounds__(kSplitWarps * 32) report_kernel(ReportArgs r)
 {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -1739,6 +1803,7 @@ __global__ void __launch_bounds__(kSplitWarps * 32) report_kernel(ReportArgs r)
     const cg::thread_block_tile<32> tile = cg::tiled_partition<32>(cg::this_thread_block());
     const int lane = tile.thread_rank(), warp = threadIdx.x >> 5;
     const SweepArgs &w = r.w;
+    if (*r.walked >= 6) return;                   // done step by step
     const int n = w.n;
     const long long m = w.a.m, x0 = w.a.k0;
     {
@@ -1849,11 +1914,16 @@ __global__ void __launch_bounds__(kSplitWarps * 32) report_kernel(ReportArgs r)
     r.out.ihh[q] = D ? acc / (2.0 * (double)D) : 0.0;
 }
 
-cudaError_t launch_report(const ReportArgs &r, cudaStream_t s)
+cudaError_t launch_report(const ReportArgs &r, const Scratch &sc, cudaStream_t s)
 {
     const SweepArgs &w = r.w;
-    cudaError_t e = launch_start(w, s);
+    const int T = start_threads(w.n), per = T / 32 < 6 ? T / 32 : 6;      // walks of a CTA
+    void (*start)(ReportArgs, Scratch) = T == 128 ? report_start_kernel<128> : T == 256 ? report_start_kernel<256>
+                                       : report_start_kernel<512>;
+    const size_t a = report_start_smem(w.n, T), b = slice_bytes(sc) * (size_t)per;
+    cudaError_t e = allow_smem(start);
     if (e != cudaSuccess) return e;
+    start<<<2 + (6 + per - 1) / per, T, a > b ? a : b, s>>>(r, sc);
     void (*sweep)(SweepArgs) = sort_kernel(w.n, w.threads, w.a.nB > 0);
     const size_t ssm = sweep_smem_bytes(w.n, w.a.W, w.threads, 1);
     if ((e = allow_smem(sweep)) != cudaSuccess) return e;

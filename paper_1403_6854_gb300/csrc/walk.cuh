@@ -578,10 +578,15 @@ __device__ __forceinline__ void split_step(const ScanArgs &a, unsigned row_sa, c
 // (NPOP 1: the sample's S; NPOP 2: the pooled S).  max_steps > 0 ends a walk
 // still running after that many steps with WALK_UNFINISHED.
 // win_parity: the warp's two mbarrier phase bits, carried from walk to walk.
-template <int NPOP>
+// quit: asked before every step (the whole warp), true ends the walk in the same
+// way.
+struct NeverQuit {
+    __device__ __forceinline__ bool operator()() { return false; }
+};
+template <int NPOP, class Quit = NeverQuit>
 __device__ WalkOut walk(const ScanArgs &a, long long core, int dir, int sel, const WarpBufs &b,
                         unsigned long long *trace, long long tcap, int max_steps,
-                        unsigned win_parity[2])
+                        unsigned win_parity[2], Quit quit = Quit())
 {
     const int lane = threadIdx.x & 31;
     WalkOut o;
@@ -666,7 +671,7 @@ __device__ WalkOut walk(const ScanArgs &a, long long core, int dir, int sel, con
     for (long long i = 1;; ++i) {
         const long long x = core + step * i;
         if (x < 0 || x >= a.m) { o.status = WALK_EDGE; o.stop = (int)i; break; }
-        if (max_steps > 0 && i > max_steps) {
+        if ((max_steps > 0 && i > max_steps) || quit()) {
             o.status = WALK_UNFINISHED;
             o.stop = (int)i;
             o.key = (float)((double)(NPOP == 2 ? SP : S0) / (double)Dstop);
