@@ -129,13 +129,14 @@ SweepPlan make_sweep_plan(int n_total, long long m, int mode, const selscan_laun
 // A whole in-order scan in one launch of chunk_scan_kernel: any whole scan of
 // at most 65,000 markers (16-bit run lengths span it) and 6,144 haplotypes,
 // while its slots stay within 2 GiB, unless a field that shapes the per-step
-// walk is set.  As many chunks as the GPU holds CTAs at once, of at least 8
-// cores.
+// walk is set.  Not two haplotypes of iHS: no core of theirs has a walk (30,000
+// markers: 47 us per step, 160 sorted).  As many chunks as the GPU holds CTAs at
+// once, of at least two cores.
 constexpr long long kChunkMaxM = 65000;
 constexpr size_t kChunkSlotBudget = (size_t)2 << 30;
 bool chunk_plan(int n_total, long long m, int mode, const selscan_launch *L, SweepPlan *w)
 {
-    if (n_total < 2 || n_total > kChunkMaxN || m < 1 || m > kChunkMaxM || mode == SELSCAN_MODE_EHH) return false;
+    if (n_total < 3 || n_total > kChunkMaxN || m < 1 || m > kChunkMaxM || mode == SELSCAN_MODE_EHH) return false;
     if (L && (L->warps_per_cta || L->ctas_per_sm || L->smem_entries || L->probe_steps || L->window_rows ||
               L->cores_per_fetch || L->min_ctas_per_sm || L->big_group_entries))
         return false;
