@@ -734,6 +734,62 @@ __device__ __forceinline__ void sparse_terms(const Tile &tile, const SplitSmem &
     tile.sync();
 }
 
+// iHS, windows of kNarrow steps: S of the two classes at the step of this lane
+// (number lane mod 8 of the window; M <= that step <=> token < lim) from the K
+// listed boundaries, K0 of class 0.  Four lanes a step run over a quarter of a
+// class's list each; their first and last cuts join the quarters.
+constexpr int kNarrow = 8;
+__device__ __forceinline__ uint2 narrow_counts(const unsigned *tk, const unsigned *gtk, unsigned K0, unsigned K,
+                                            unsigned n0, unsigned n, unsigned lim)
+{
+    constexpr unsigned kTok = (unsigned)tok_smem(0), kNone = 0xFFFFFFFFu;
+    const int lane = threadIdx.x & 31;
+    unsigned S[2];
+#pragma unroll 1
+    for (int c = 0; c < 2; ++c) {
+        const unsigned ka = c ? K0 : 0u, kb = c ? K : K0, start = c ? n0 : 0u, end = c ? n : n0;
+        const unsigned per = (kb - ka + 3u) / 4u, from = ka + (unsigned)(lane >> 3) * per;
+        unsigned d = 0u, last = 0u, first = kNone;
+        if (K <= kTok) {
+#pragma unroll 4
+            for (unsigned x = 0; x < per; ++x) {
+                const unsigned k = from + x, t = k < kb ? tk[k] : kNone;
+                if (t < lim) {
+                    const unsigned p = t & 0xFFFFu, l = p - last;
+                    d += l * l;
+                    first = min(first, p);
+                    last = p;
+                }
+            }
+        } else {
+#pragma unroll 4
+            for (unsigned x = 0; x < per; ++x) {
+                const unsigned k = from + x, t = k < kb ? (k < kTok ? tk : gtk)[k] : kNone;
+                if (t < lim) {
+                    const unsigned p = t & 0xFFFFu, l = p - last;
+                    d += l * l;
+                    first = min(first, p);
+                    last = p;
+                }
+            }
+        }
+        unsigned sum = 0u, cur = start;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int src = (lane & 7) + 8 * q;
+            const unsigned f = __shfl_sync(0xFFFFFFFFu, first, src), e = __shfl_sync(0xFFFFFFFFu, last, src);
+            const unsigned dq = __shfl_sync(0xFFFFFFFFu, d, src);
+            if (f != kNone) {                         // a quarter's first cut was measured from 0
+                sum += dq - f * f + (f - cur) * (f - cur);
+                cur = e;
+            }
+        }
+        sum += (end - cur) * (end - cur);
+        S[c] = (sum - (end - start)) >> 1;
+    }
+    return make_uint2(S[0], S[1]);
+}
+
 }  // namespace
 
 size_t split_smem_per_warp(int n, int xpehh)
@@ -755,19 +811,20 @@ size_t split_scratch_per_warp(int n) { return n <= tok_smem(1) ? 0 : (((size_t)n
 // 17.2 ms against 24.1 with 32; 12.7 since its list is shorter, tok_smem).  Later
 // windows (win_steps) hold few boundaries among many older run starts: there each lane takes one boundary
 // (sparse_terms); a window with more than tok_smem of them is cut like the
-// first one.
+// first one.  NARROW (iHS): windows of kNarrow steps instead, for slots most of
+// whose boundaries part within the first 32 steps (wide_slot).
 // Pair counts fit 32 bits (C(16383, 2) < 2^32); the digest is 64-bit.  Lane
 // (i - 1) mod 32 adds step i's trapezoid term to its own FP64 partial sum, and
 // the partial sums meet in a fixed butterfly when the walk ends: the order of
 // the per-step walk, so a walk handed over to it gives the same bits.
-template <int NPOP, typename Tile>
+template <int NPOP, bool NARROW = false, typename Tile>
 __device__ __forceinline__ void walk_slot(const SweepArgs &w, const Tile &tile, const SplitSmem &s,
                                           const unsigned char *slot, long long k, int dir)
 {
     constexpr int G = 32;
     constexpr int NV = NPOP == 2 ? 3 : 2;     // S values: class 0, class 1; or A, B, pooled
     constexpr int NWK = NPOP == 2 ? 1 : 2;    // walks of a slot
-    constexpr int kDense = NPOP == 2 ? 16 : 32;   // steps of a window cut boundary by boundary
+    constexpr int kDense = NARROW ? kNarrow : NPOP == 2 ? 16 : 32;   // steps of a window cut boundary by boundary
     constexpr int kWin = win_steps(NPOP == 2);    // and of one taken one boundary per lane
     const int lane = tile.thread_rank();
     const int n = w.n;
@@ -846,7 +903,7 @@ __device__ __forceinline__ void walk_slot(const SweepArgs &w, const Tile &tile, 
         const int hi = lo + (dense ? kDense - 1 : kWin - 1);
         const int pa = NPOP == 1 && !act[0] ? n0 : 0, pb = NPOP == 1 && !act[NWK - 1] ? n0 : n;
         const unsigned K = mark_window<NPOP>(tile, s, M4, n, n0, hi, dense, merge, pa, pb, K0, sup);
-        if (!dense && K > (unsigned)tok_smem(NPOP == 2)) {    // redo as a window of 32 steps
+        if (!dense && K > (unsigned)tok_smem(NPOP == 2)) {    // redo as a window of fewer steps
             dense = true;
             merge = false;
             continue;
@@ -890,6 +947,11 @@ __device__ __forceinline__ void walk_slot(const SweepArgs &w, const Tile &tile, 
                     S[0] = (rc.d[NPOP == 2 ? 1 : 0] - (unsigned)w.a.nA) >> 1;
                     S[1] = (rc.d[NPOP == 2 ? 2 : 0] - (unsigned)w.a.nB) >> 1;
                     S[NV - 1] = (rc.d[0] - (unsigned)n) >> 1;
+                } else if (NARROW) {
+                    const uint2 c = narrow_counts(s.tk, s.gtk, K0, K, (unsigned)n0, (unsigned)n,
+                                                  (unsigned)(i0 + la + (lane & 7) + 1) << 16);
+                    S[0] = c.x;
+                    S[1] = c.y;
                 } else {
                     rc.lim = (unsigned)(i + 1) << 16;
                     S[0] = S[1] = 0u;
@@ -1008,16 +1070,54 @@ __device__ __forceinline__ void walk_slot(const SweepArgs &w, const Tile &tile, 
     tile.sync();
 }
 
+// iHS in samples of more than kWideBoundaries haplotypes: whether more than that many
+// run boundaries part within the first 32 steps, told from 256 run lengths (eight a
+// lane, spread over the slot).  Their walks last a dozen steps (unlinked alleles),
+// and a window of 32 that runs over all of them, mostly in global memory, takes
+// longer than windows of kNarrow steps with short lists: 5,000 x 100,000 unlinked
+// 11.3 ms against 6.4, 10,000 x 75,000 18.4 against 7.8.  Up to twice the on-chip
+// list the window of 32 is the faster one (8,000 haplotypes of 320 founders: 5.0
+// ms against 5.6).
+constexpr int kWideBoundaries = 2048;
+__device__ __forceinline__ bool wide_slot(const unsigned char *slot, int n, int lane)
+{
+    const uint4 v = __ldg((const uint4 *)(slot + 16) + (unsigned)lane * ((unsigned)n >> 8));
+    const unsigned P1 = 32u * 0x00010001u, PP = P1 + 0x00010001u;     // 16x2 clamps, as in mark_window
+    const unsigned f = (__vmaxu2(__vminu2(v.x, PP), P1) - P1) + (__vmaxu2(__vminu2(v.y, PP), P1) - P1) +
+                       (__vmaxu2(__vminu2(v.z, PP), P1) - P1) + (__vmaxu2(__vminu2(v.w, PP), P1) - P1);
+    const unsigned over = (unsigned)__reduce_add_sync(0xFFFFFFFFu, (int)((f & 0xFFFFu) + (f >> 16)));
+    return (256u - over) * (unsigned)n > 256u * (unsigned)kWideBoundaries;
+}
+
+// Walks the slots that a warp has put by: a list through a word per core and
+// direction (w.sk.sorted2, which the second pass fills later), from put_by - 1 on.
+__device__ __noinline__ void walk_put_by(const SweepArgs &w, unsigned *tk, unsigned *gtk, unsigned put_by)
+{
+    namespace cg = cooperative_groups;
+    const cg::thread_block_tile<32> tile = cg::tiled_partition<32>(cg::this_thread_block());
+    const int lane = tile.thread_rank();
+    const SplitSmem s = split_smem((unsigned char *)tk, (unsigned char *)gtk, w.n, 0);
+    while (put_by != 0u) {
+        const unsigned id = put_by - 1u;
+        const int dir = (int)(id & 1u);
+        const long long q = (long long)(id >> 1), c = q / w.B;
+        const long long c1 = (c + 1) * w.B < w.a.k1 - w.a.k0 ? (c + 1) * w.B : w.a.k1 - w.a.k0;
+        const long long r = (dir == 0 ? q - c * w.B : c1 - 1 - q) - (long long)w.stage * w.R;
+        walk_slot<1, true>(w, tile, s, w.slots + (size_t)((dir * w.nch + c) * w.R + r) * w.slot_bytes, w.a.k0 + q, dir);
+        unsigned nxt = 0u;
+        if (lane == 0) nxt = w.sk.sorted2[id];
+        put_by = tile.shfl(nxt, 0);
+    }
+}
+
 // Persistent: each warp takes slots of this stage (both directions) from a
-// counter.
-#ifndef SPLIT_MIN_CTAS
-#define SPLIT_MIN_CTAS 4
-#endif
-template <int NPOP, int G>
-__global__ void __launch_bounds__(kSplitWarps * 32, SPLIT_MIN_CTAS) split_walk_kernel(SweepArgs w)
+// counter.  WIDE: puts wide slots by and walks them at the end, out of line; in the
+// common walk's place their code cost it registers (1M iHS 25.3 ms; so 24.5, and
+// 24.2 without).
+template <int NPOP, int G, bool WIDE>
+__device__ __forceinline__ void split_walks(const SweepArgs &w, unsigned char *smem)
 {
     static_assert(G == 32, "lane l owns step l of a block of 32");
-    extern __shared__ __align__(16) unsigned char smem[];
     namespace cg = cooperative_groups;
     const cg::thread_block_tile<G> tile = cg::tiled_partition<G>(cg::this_thread_block());
     const int lane = tile.thread_rank(), tix = threadIdx.x / G;
@@ -1026,6 +1126,7 @@ __global__ void __launch_bounds__(kSplitWarps * 32, SPLIT_MIN_CTAS) split_walk_k
                                    w.wscratch + ((size_t)blockIdx.x * kSplitWarps + tix) * w.wscratch_bytes,
                                    n, NPOP == 2);
     const long long per_dir = (long long)w.nch * w.R;
+    unsigned put_by = 0u;                     // 1 + the last slot put by
     unsigned long long nxt = 0;               // the slot after this one, fetched ahead
     if (lane == 0) nxt = atomicAdd(w.walk_head, 1ull);
     for (;;) {
@@ -1056,14 +1157,45 @@ __global__ void __launch_bounds__(kSplitWarps * 32, SPLIT_MIN_CTAS) split_walk_k
         }
         if (w.sk.core_status[k] == (int8_t)SELSCAN_LOCUS_MAF_FILTERED) continue;
 
-        walk_slot<NPOP>(w, tile, s, w.slots + (size_t)gslot * w.slot_bytes, k, dir);
+        const unsigned char *slot = w.slots + (size_t)gslot * w.slot_bytes;
+        if (WIDE && wide_slot(slot, n, lane)) {
+            const unsigned id = (unsigned)(2 * (k - w.a.k0) + dir);
+            if (lane == 0) w.sk.sorted2[id] = put_by;
+            put_by = id + 1u;
+        } else {
+            walk_slot<NPOP>(w, tile, s, slot, k, dir);
+        }
     }
+    if (WIDE && put_by != 0u) walk_put_by(w, s.tk, s.gtk, put_by);
+}
+
+#ifndef SPLIT_MIN_CTAS
+#define SPLIT_MIN_CTAS 4
+#endif
+template <int NPOP, int G>
+__global__ void __launch_bounds__(kSplitWarps * 32, SPLIT_MIN_CTAS) split_walk_kernel(SweepArgs w)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    split_walks<NPOP, G, false>(w, smem);
 }
 
 template <int G>
 static void (*walk_kernel_for(int xpehh))(SweepArgs)
 {
     return xpehh ? split_walk_kernel<2, G> : split_walk_kernel<1, G>;
+}
+
+__global__ void __launch_bounds__(kSplitWarps * 32, SPLIT_MIN_CTAS)
+    split_walk_wide_kernel(const __grid_constant__ SweepArgs w)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    split_walks<1, 32, true>(w, smem);
+}
+
+// the walk kernel of a sample
+static void (*walk_kernel_of(int n, int xpehh))(SweepArgs)
+{
+    return !xpehh && n > kWideBoundaries ? split_walk_wide_kernel : walk_kernel_for<32>(xpehh);
 }
 
 // ---- the starting state of a chunk ----------------------------------------------
@@ -1663,9 +1795,9 @@ int split_walk_ctas(int n, int xpehh)
     // resident CTAs of the persistent walker
     int per_sm = 0;
     const size_t smem = split_smem_per_warp(n, xpehh) * kSplitWarps;
-    allow_smem(walk_kernel_for<32>(xpehh));
+    allow_smem(walk_kernel_of(n, xpehh));
     const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &per_sm, walk_kernel_for<32>(xpehh), kSplitWarps * 32, smem);
+        &per_sm, walk_kernel_of(n, xpehh), kSplitWarps * 32, smem);
     if (e != cudaSuccess || per_sm < 1) per_sm = 1;
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
@@ -1721,7 +1853,7 @@ cudaError_t launch_sweep_path(const SweepArgs &w0, cudaStream_t s)
     cudaError_t e = allow_smem(sweep);
     if (e != cudaSuccess) return e;
     const size_t wsm = (size_t)w.split_bytes * kSplitWarps;
-    void (*walk)(SweepArgs) = walk_kernel_for<32>(w.a.nB > 0);
+    void (*walk)(SweepArgs) = walk_kernel_of(w.n, w.a.nB > 0);
     if ((e = allow_smem(walk)) != cudaSuccess) return e;
     if (w.started && (e = launch_start(w, s)) != cudaSuccess) return e;
     for (int st = 0; st < w.nstages; ++st) {
