@@ -324,7 +324,10 @@ int selscan_batch_prepare(const selscan_scan *scan, void *stream);
  * u < nunits <= SELSCAN_BATCH_MAX_UNITS, nscans <= SELSCAN_BATCH_MAX_SCANS
  * (host arrays, read before the call returns: the tick copies nothing to the
  * device, its descriptors travel in the launch's parameter block).  Cores
- * are walked in unit order, one core per fetch of a warp.  max_n_total /
+ * are walked in chunks, in unit order; step by step, one core per fetch of a
+ * warp, where a scan with cores in the tick has more than 65,000 markers or
+ * 6,144 haplotypes or the workspace has no room for the chunks (their slots,
+ * about 4 n_total bytes a core, and the scans' rows once more).  max_n_total /
  * max_ld bound the scans of this tick.  SELSCAN_ERR_INVALID_ARG for counts
  * above the limits, ranges outside [0, m) or a scan that fails the checks of
  * selscan_batch_prepare; nothing is launched then. */

@@ -169,12 +169,13 @@ bool chunk_plan(int n_total, long long m, int mode, const selscan_launch *L, Swe
 }
 
 // The schedule of a default launch: the sorted sweep once the chromosome is
-// long, the in-order schedule otherwise.  Both sort (chunk_plan) wherever the
-// line runs below 65,000 markers and 6,144 haplotypes, and the line only
-// decides between one launch and several; it was drawn against the per-step
-// walk, which above it loses on mosaics of n / 25 founders (it lost from about
-// 7k markers at n = 100, 30k at 5,000), and is kept so that saved plans and
-// callers that ask for the schedule see the same answer.
+// long, the in-order schedule otherwise.  For whole scans of at most 65,000
+// markers and 6,144 haplotypes both sort (chunk_plan), and the line only decides
+// between one launch and several; larger samples and core ranges below it walk
+// every step.  It was drawn against the per-step walk, which above it loses on
+// mosaics of n / 25 founders (it lost from about 7k markers at n = 100, 30k at
+// 5,000), and is kept so that saved plans and callers that ask for the schedule
+// see the same answer.
 int default_schedule(int mode, long long n_total, long long m)
 {
     if (mode == SELSCAN_MODE_EHH || n_total < 2 || n_total > kSweepMaxN) return SELSCAN_SCHED_IN_ORDER;

@@ -1,10 +1,11 @@
-// Batched scans: several admitted scans (iHS and XPEHH, any sizes) share one
-// persistent walk launch ("tick").  The host hands each tick up to
-// SELSCAN_BATCH_MAX_UNITS core ranges from up to SELSCAN_BATCH_MAX_SCANS scans;
-// the tick walks the concatenation of those ranges, one core per queue fetch
-// (neighbouring cores near a sweep all have long walks, so finer fetches
-// balance the warps), so walks of different scans run side by side on the
-// GPU.  Used by the serving loop for continuous batching; the statistics are
+// Batched scans: several admitted scans (iHS and XPEHH, any sizes) share a
+// "tick".  The host hands each tick up to SELSCAN_BATCH_MAX_UNITS core ranges
+// from up to SELSCAN_BATCH_MAX_SCANS scans; the tick sorts and walks chunks of
+// those ranges in one launch (after one that makes the scans' 32-marker words),
+// or, where its scans or its workspace do not allow that, walks their
+// concatenation every step, one core per queue fetch (neighbouring cores near a
+// sweep all have long walks, so finer fetches balance the warps).  Either way
+// walks of different scans run side by side on the GPU.  Used by the serving loop for continuous batching; the statistics are
 // exactly those of selscan_ihs / selscan_xpehh (same walk code, same
 // finalize).  A tick issues no host-to-device copy: the scan descriptors and
 // the ranges travel as the kernel's parameter block.

@@ -115,6 +115,7 @@ cudaError_t launch_ehh(const ScanArgs &a, long long locus, const Scratch &sc,
                        cudaStream_t s);
 cudaError_t launch_pack(const uint8_t *hap01, int n, long long m, int hap_major,
                         unsigned long long *rows, long long ld, cudaStream_t s);
+int device_sms();
 int max_ctas_per_sm(int schedule, int warps_per_cta, size_t smem_bytes, int minb);
 
 // Second pass of the per-step walk over the items queued in sink.list2.

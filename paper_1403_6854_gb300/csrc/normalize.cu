@@ -399,9 +399,10 @@ void launch_apply(const double *score, const int8_t *status, const int32_t *n1, 
                   int32_t n, int32_t nbins, const double *bin_mean, const double *bin_sd,
                   const long long *bin_count, double *out, cudaStream_t s)
 {
-    // eight CTAs per SM of this part at most
+    // eight CTAs per SM at most
     long long blocks = (m + kApplyThreads * kApplyU - 1) / (kApplyThreads * kApplyU);
-    if (blocks > 1216) blocks = 1216;
+    const long long most = 8ll * device_sms();
+    if (blocks > most) blocks = most;
     norm_apply_kernel<<<(unsigned)blocks, kApplyThreads, (size_t)nbins * 24, s>>>(
         score, status, n1, m, n, nbins, bin_mean, bin_sd, bin_count, out);
 }

@@ -391,7 +391,7 @@ __device__ __forceinline__ void sort_chunk(const SweepArgs &w, unsigned char *sm
             // XPEHH: the same thread makes the population flags of its 8 positions
             // (16x2 clamps of the bit indices, as the walker marks windows) and four
             // neighbours' make a word: a third of the instructions of a ballot per
-            // word (1M: sort 19.0 -> 17.0 ms)
+            // word (1M: sort 19.0 -> 17.5 ms)
             const uint4 *P4 = (const uint4 *)Ps;
             uint4 *M4 = (uint4 *)(slot + 16);
             const int items = (n + 31) / 32 * 4;
@@ -1207,7 +1207,7 @@ static void (*walk_kernel_of(int n, int xpehh))(SweepArgs)
 // levels at once: per round every unresolved group splits three ways, stably,
 // about its middle element's word (the equal part goes on to the next word),
 // by one prefix sum over the CTA; once few are left, only they take part.
-// About 60 rounds replace 1,536 marker passes.
+// About 40 rounds (19 of all elements, 20 late ones at 1M) replace 1,536 marker passes.
 // Shared memory per haplotype: element (bit index | group start << 16) and
 // group (at its start: end | word level << 16) twice, the prefix sums, and the
 // level at which each boundary arose.
@@ -1700,7 +1700,7 @@ typedef void (*ChunkKernel)(ScanChunks);
 struct ChunkShape { int ts, tc, ctas; ChunkKernel ihs, xpehh; };
 static ChunkShape chunk_shape(int n, long long m)
 {
-    if (n <= 1024 && m < 16 * 2 * 152)
+    if (n <= 1024 && m < 16 * 2 * device_sms())
         return {128, 128, 5, chunk_scan_kernel<128, 128, 8, 5, 1, ScanChunks>, chunk_scan_kernel<128, 128, 8, 5, 2, ScanChunks>};
     if (n <= 256)
         return {32, 192, 4, chunk_scan_kernel<32, 192, 8, 4, 1, ScanChunks>, chunk_scan_kernel<32, 192, 8, 4, 2, ScanChunks>};

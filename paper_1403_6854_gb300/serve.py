@@ -3,7 +3,7 @@
 Requests (scans of any mode and size) arrive over time.  The server keeps the
 packed matrices of admitted scans resident in HBM, admits waiting requests in
 arrival order as soon as their HBM footprint fits the budget, and runs
-"ticks": one persistent walk launch (selscan_batch_run) over core ranges of
+"ticks": one launch (selscan_batch_run) that sorts and walks core ranges of
 the resident scans in policy order, so requests that arrive while others run
 join the very next tick and their walks share the GPU.  A scan whose cores
 are all walked is finalised, its results are copied to the host and its
@@ -124,7 +124,7 @@ class Scheduler:
         tick's core budget handed out in policy order ("fifo" oldest first,
         younger scans backfill what the oldest cannot use; "srpt" least
         remaining work first; "ps" equal shares).  The device walks the ranges
-        in this order, one core per warp fetch.  Returns the tick's scans and
+        in this order, in chunks of cores.  Returns the tick's scans and
         an int64 array of units (index into that list, c0, c1)."""
         live = [a for a in self.active if a.remaining > 0 and not a.whole]
         if not live:
